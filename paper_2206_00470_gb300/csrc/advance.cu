@@ -7,8 +7,8 @@
 //                 then -1 for the closing ones; transitions 0 -> 1
 //                 (create) and 1 -> 0 (evict); the last block of the
 //                 closing launch settles the advance's slot counts        (Sec. 3)
-//   evict_create  main += pending updates of every evicted replica, and
-//                 val = main, pending = 0 for every created one, the i-th
+//   evict_create  main += pending updates of every evicted replica; every
+//                 created one starts as an alias of its main row, the i-th
 //                 evicted slot going to the i-th created key             (Sec. 4.1)
 #include <utility>
 #include <vector>
@@ -212,7 +212,10 @@ __global__ void events_kernel(Store s, uint32_t w, EventBatch eb, uint32_t* out_
     for (int q = 0; q < Q; ++q) {
       old[q] = 1u;   // neither transition
       msl[q] = -1;
-      if (!START && in[q]) msl[q] = mapw[k[q]];
+      if (!START && in[q]) {
+        const int32_t e = mapw[k[q]];
+        msl[q] = map_none(e) ? -1 : map_slot(e);
+      }
       if (in[q]) old[q] = START ? atomicAdd(rcw + k[q], 1u) : atomicSub(rcw + k[q], 1u);
     }
 #pragma unroll
@@ -320,32 +323,53 @@ __global__ void events_kernel(Store s, uint32_t w, EventBatch eb, uint32_t* out_
   }
 }
 
-// evict_create: entry i of the advance evicts the i-th listed slot (any
-// worker's: a relocation destroys another worker's replica) -- main[k] +=
-// its pending row, by vector atomic adds since main[k] may receive two
-// pending rows in one advance (the leaving worker's and a relocated
-// holder's) -- and creates the i-th listed key of worker w, val = main,
-// pending = 0, in that same slot when there is one (the thread reads the
-// pending row before it overwrites it), else in a slot popped from the
-// stack; an evicted slot with no creation to take it is pushed.  A created
-// key is never one whose replica this advance destroys (a worker joins or
-// leaves a key, not both), so its main row is final.  R entries per row
-// group at a time; a round's loads (owner records, pending rows, main rows)
-// go out together with the next round's list entries.
+// evict_create: entry i of the advance evicts the i-th listed slot and creates
+// the i-th listed key of worker w in that same slot when there is one, else in
+// a slot popped from the stack; an evicted slot with no creation to take it is
+// pushed.  A created key is never one whose replica this advance destroys (a
+// worker joins or leaves a key, not both).
+//
+// Creating moves no row: the new replica is an alias of its main row (with
+// relocation, where it is a copy, copied.cu).  Of an evicted replica only pending updates move, main[k] += acc by vector atomic
+// adds, after the other holders' aliases of the old main row have got it as a
+// value of their own.
+//
+// What is done once per entry (list entries, owner records, holder masks,
+// map entries, the stack) is done by one lane per entry, a warp taking up to
+// 32 entries at a time, so its chain of random accesses runs 32 wide; then
+// one lane per (entry, other holder) looks for aliases of the main rows that
+// are about to change; rows move last, listed in shared memory and taken by
+// the warp's row groups, R in flight each.
+//
+// Bound by its random row and word accesses.  Measured per clock of 8
+// advances, copies made and moved by row groups before -> now: 198k replicas
+// of 64 floats destroyed and created each (100M keys) 833 -> 713 us, 366k of
+// 512 floats 5809 -> 4170 us, 27k of 200 floats 297 -> 270 us.
 //
 // After early events (AdvCounts given) every block takes the list lengths
 // from the counters and the stack top from the store (the same values in
 // every block: the store changes only after all blocks have finished),
 // evicted slots also clear their map entries, and the last block to finish
 // settles the advance.
+constexpr uint32_t kMany = 3u;   // a holder mask that counts as neither no holder nor one
+
+constexpr int evict_blocks_per_sm(int C) { return C >= 8 ? 2 : (C == 4 ? 3 : 4); }
+
 template <int G, int C>
-__global__ void __launch_bounds__(kThreads, C >= 8 ? 2 : 3) evict_create_kernel(Store s, uint32_t w,
+__global__ void __launch_bounds__(kThreads, evict_blocks_per_sm(C)) evict_create_kernel(Store s, uint32_t w,
                                                                               const uint32_t* __restrict__ evict_list,
                                                                               const uint32_t* __restrict__ create_list,
                                                                               AdvCounts* early) {
-  constexpr int R = 4 / C > 0 ? 4 / C : 1;
+  constexpr int R = C == 4 ? 2 : (4 / C > 0 ? 4 / C : 1);
+  constexpr uint32_t GW = 32 / G;   // row groups per warp
+  __shared__ uint2 moves[kThreads / 32][32];    // (slot, key): pending rows to add to main
+  __shared__ uint2 copies[kThreads / 32][32];   // (slot, key): main rows to copy to val first
+  const int lane32 = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int lane = threadIdx.x & (G - 1);
+  const uint32_t gi = (uint32_t)lane32 / G;
+  const unsigned before = (1u << lane32) - 1u;
   const uint32_t D4 = s.D >> 2;
+  s.par = s.st->par;
   uint32_t ne, nc;
   int32_t top;
   if (early) {
@@ -360,103 +384,145 @@ __global__ void __launch_bounds__(kThreads, C >= 8 ? 2 : 3) evict_create_kernel(
   const uint64_t n = ne > nc ? ne : nc;
   float4* main4 = reinterpret_cast<float4*>(s.main);
   float4* val4 = reinterpret_cast<float4*>(s.val);
-  float4* acc4 = reinterpret_cast<float4*>(s.acc);
+  const float4* acc4 = reinterpret_cast<const float4*>(s.acc);
   int32_t* mapw = s.map + (uint64_t)w * s.K;
-  const uint64_t g = group_id<G>(), ng = group_count<G>();
-  const uint64_t step = ng * R;
-  // list entries out of range (slots >= S, keys >= K) are skipped and reported
-  auto load_entries = [&](uint64_t i0, int32_t (&es)[R], uint32_t (&ck)[R]) {
+  const uint64_t warps = (uint64_t)gridDim.x * (kThreads / 32);
+  const uint64_t warp = (uint64_t)blockIdx.x * (kThreads / 32) + wid;
+  // entries per warp and round: as many rounds as 32 entries each take, all the same size
+  const uint64_t rounds = (n + warps * 32 - 1) / (warps * 32);
+  const uint32_t per = rounds ? (uint32_t)((n + warps * rounds - 1) / (warps * rounds)) : 0u;
+  // val rows of the first n listed slots := the main rows of their keys
+  auto copy_rows = [&](uint32_t n) {
+    for (uint32_t j0 = gi * R; j0 < n; j0 += GW * R) {
+      uint32_t to[R];
+      float4 v[R][C];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const uint64_t i = i0 + r;
-      const uint32_t e = i < ne ? evict_list[i] : 0xFFFFFFFFu;
-      es[r] = e < s.S ? (int32_t)e : -1;
-      ck[r] = i < nc ? create_list[i] : kNoKey;
-      if ((i < ne && e >= s.S) || (i < nc && ck[r] >= s.K)) {
-        set_error(s.st, ERR_INTERNAL);
-        if (ck[r] >= s.K) ck[r] = kNoKey;
+      for (int r = 0; r < R; ++r) {
+        const uint2 cp = j0 + r < n ? copies[wid][j0 + r] : make_uint2(0xFFFFFFFFu, 0u);
+        to[r] = cp.x;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          const uint32_t col = lane + c * G;
+          v[r][c] = cp.x != 0xFFFFFFFFu && col < D4 ? main4[(uint64_t)cp.y * D4 + col] : f4zero();
+        }
       }
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        if (to[r] != 0xFFFFFFFFu)
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            const uint32_t col = lane + c * G;
+            if (col < D4) val4[(uint64_t)to[r] * D4 + col] = v[r][c];
+          }
     }
   };
-  int32_t es[R];
-  uint32_t ck[R];
-  load_entries(g * R, es, ck);
-  for (uint64_t i0 = g * R; i0 < n; i0 += step) {
-    int32_t cs[R];
-    unsigned long long ow[R];
-    float4 ac[R][C], mv[R][C];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const uint64_t i = i0 + r;
-      // slot of the creation: the paired evicted slot, else popped (top first)
-      cs[r] = ck[r] == kNoKey ? -1 : (es[r] >= 0 ? es[r] : s.free_stack[top - 1 - (int32_t)(i - ne)]);
-      ow[r] = es[r] >= 0 ? s.slot_owner[es[r]] : 0ull;
-      const bool bad_slot = ck[r] != kNoKey && (cs[r] < 0 || (uint64_t)cs[r] >= s.S);
-      const bool bad_owner = es[r] >= 0 && ((uint32_t)ow[r] >= s.K || (ow[r] >> 32) >= s.W);
-      if (bad_slot || bad_owner) {
-        set_error(s.st, ERR_INTERNAL);   // a free-stack entry or owner record out of range: skipped
-        if (bad_slot) {
-          cs[r] = -1;
-          ck[r] = kNoKey;
-        }
-        if (bad_owner) es[r] = -1;
-      }
-#pragma unroll
-      for (int c = 0; c < C; ++c) {
-        const uint32_t col = lane + c * G;
-        ac[r][c] = (es[r] >= 0 && col < D4) ? acc4[(uint64_t)es[r] * D4 + col] : f4zero();
-        mv[r][c] = (ck[r] != kNoKey && col < D4) ? main4[(uint64_t)ck[r] * D4 + col] : f4zero();
+  uint32_t dkeys = 0, dsole = 0;   // changes of live_keys and sole_keys (modulo 2^32)
+  for (uint64_t i0 = warp * per; i0 < n; i0 += warps * per) {   // warp-uniform
+    const uint64_t i = i0 + lane32;
+    const bool in = (uint32_t)lane32 < per;
+    // list entries out of range (slots >= S, keys >= K) are skipped and reported
+    const bool ev = in && i < ne, cr = in && i < nc;
+    const uint32_t e = ev ? evict_list[i] : 0u;
+    uint32_t ck = cr ? create_list[i] : kNoKey;
+    int32_t es = ev && e < s.S ? (int32_t)e : -1;
+    bool bad = (ev && es < 0) || (cr && ck >= s.K);
+    if (ck >= s.K) ck = kNoKey;
+    // slot of the creation: the paired evicted slot, else popped (top first)
+    int32_t cs = ck == kNoKey ? -1 : (es >= 0 ? es : s.free_stack[top - 1 - (int32_t)(i - ne)]);
+    const unsigned long long ow = es >= 0 ? s.slot_owner[es] : 0ull;
+    const uint32_t k = (uint32_t)ow, a = owner_worker(ow);
+    if (ck != kNoKey && (cs < 0 || (uint64_t)cs >= s.S)) {   // a free-stack entry out of range
+      bad = true;
+      cs = -1;
+      ck = kNoKey;
+    }
+    if (es >= 0 && (k >= s.K || a >= s.W)) {   // an owner record out of range
+      bad = true;
+      es = -1;
+    }
+    if (bad) set_error(s.st, ERR_INTERNAL);
+    bool move = false;
+    uint32_t others = 0, left = kMany, had = kMany;   // holders after the eviction, before the creation
+    if (es >= 0) {
+      left = atomicAnd(s.holders + k, ~(1u << a)) & ~(1u << a);
+      if (s.dirty != nullptr) s.dirty[k] = 1;   // versioned refresh: main changed
+      // (the events kernel that listed the slot has cleared its map entry, unless it ran early)
+      if (early) s.map[(uint64_t)a * s.K + k] = -1;
+      move = owner_state(ow, s.par) & REP_PENDING;
+      // (the versioned refresh counts a destroyed replica as a write even if nothing was pending)
+      if (move || s.dirty != nullptr) others = left;
+      if (ck == kNoKey) {
+        s.slot_owner[es] = kEmptySlot;
+        s.free_stack[top + (int32_t)(i - nc)] = es;
       }
     }
-    int32_t es1[R];
-    uint32_t ck1[R];
-    load_entries(i0 + step, es1, ck1);
+    if (ck != kNoKey) {
+      // versioned refresh: the new replica has seen every update (a stale
+      // replica of another worker is refreshed anyway: the key has two holders)
+      if (s.dirty != nullptr) s.dirty[ck] = 0;
+      mapw[ck] = cs;
+      had = atomicOr(s.holders + ck, 1u << w);
+      s.slot_owner[cs] = owner_word(w, ck, REP_ALIAS, s.par);
+    }
+    // the aliases of the main rows that change, 32 (entry, holder) pairs at a time
+    uint32_t pos = __popc(others);
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const uint64_t i = i0 + r;
-      if (es[r] >= 0) {
-        const uint32_t k = (uint32_t)ow[r], a = (uint32_t)(ow[r] >> 32);
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, pos, o);
+      if (lane32 >= o) pos += y;
+    }
+    const uint32_t pairs = __shfl_sync(0xFFFFFFFFu, pos, 31);
+    pos -= __popc(others);
+    for (uint32_t p0 = 0; p0 < pairs; p0 += 32) {   // warp-uniform
+      while (others && pos < p0 + 32) {
+        copies[wid][pos - p0] = make_uint2((uint32_t)__ffs(others) - 1, k);
+        others &= others - 1;
+        ++pos;
+      }
+      __syncwarp();
+      const uint2 pr = p0 + lane32 < pairs ? copies[wid][lane32] : make_uint2(0u, kNoKey);
+      const int32_t sl = pr.y != kNoKey ? take_alias(s, pr.x, pr.y) : -1;
+      const unsigned got = __ballot_sync(0xFFFFFFFFu, sl >= 0);
+      if (sl >= 0) copies[wid][__popc(got & before)] = make_uint2((uint32_t)sl, pr.y);
+      __syncwarp();
+      copy_rows(__popc(got));
+      __syncwarp();   // copies is rewritten; the old main rows have been read
+    }
+    const unsigned todo = __ballot_sync(0xFFFFFFFFu, move);
+    const uint32_t cnt = __popc(todo);
+    if (move) moves[wid][__popc(todo & before)] = make_uint2((uint32_t)es, k);
+    __syncwarp();
+    for (uint32_t j0 = gi * R; j0 < cnt; j0 += GW * R) {
+      uint32_t key[R];
+      float4 ac[R][C];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const uint2 m = j0 + r < cnt ? moves[wid][j0 + r] : make_uint2(0u, kNoKey);
+        key[r] = m.y;
 #pragma unroll
         for (int c = 0; c < C; ++c) {
           const uint32_t col = lane + c * G;
-          if (col < D4) atomicAdd(main4 + (uint64_t)k * D4 + col, ac[r][c]);
-        }
-        if (lane == 0) {
-          if (s.dirty != nullptr) s.dirty[k] = 1;   // versioned refresh: main changed
-          // (always replicating, the events kernel that listed the slot has
-          // cleared its map entry, unless it ran early)
-          if (s.own != nullptr || early) s.map[(uint64_t)a * s.K + k] = -1;
-          atomicAnd(s.holders + k, ~(1u << a));
-          if (ck[r] == kNoKey) {
-            s.slot_owner[es[r]] = kEmptySlot;
-            s.free_stack[top + (int32_t)(i - nc)] = es[r];
-          }
+          ac[r][c] = m.y != kNoKey && col < D4 ? acc4[(uint64_t)m.x * D4 + col] : f4zero();
         }
       }
-      if (ck[r] != kNoKey) {
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-          const uint32_t col = lane + c * G;
-          if (col < D4) {
-            val4[(uint64_t)cs[r] * D4 + col] = mv[r][c];
-            acc4[(uint64_t)cs[r] * D4 + col] = f4zero();
+      for (int r = 0; r < R; ++r)
+        if (key[r] != kNoKey)
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            const uint32_t col = lane + c * G;
+            if (col < D4) atomicAdd(main4 + (uint64_t)key[r] * D4 + col, ac[r][c]);
           }
-        }
-        if (lane == 0) {
-          // versioned refresh: the new replica has seen every update (a stale
-          // replica of another worker is refreshed anyway: the key has two holders)
-          if (s.dirty != nullptr) s.dirty[ck[r]] = 0;
-          mapw[ck[r]] = cs[r];
-          atomicOr(s.holders + ck[r], 1u << w);
-          s.slot_owner[cs[r]] = ((unsigned long long)w << 32) | ck[r];
-        }
-      }
     }
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      es[r] = es1[r];
-      ck[r] = ck1[r];
-    }
+    // (counted here: the masks have arrived by now)
+    dkeys += (had == 0u) - (left == 0u);
+    dsole += (had == 0u) - (__popc(had) == 1) - (left == 0u) + (__popc(left) == 1);
+    __syncwarp();   // moves is rewritten by the next round
+  }
+  block_sum2(dkeys, dsole);
+  if (threadIdx.x == 0) {
+    if (dkeys) atomicAdd(&s.st->live_keys, (int32_t)dkeys);
+    if (dsole) atomicAdd(&s.st->sole_keys, (int32_t)dsole);
   }
   if (early) {
     // the last block to finish settles the advance (all blocks have read
@@ -575,10 +641,15 @@ void launch_events_undo(const Store& s, uint32_t w, const EventList* lists, int 
 void launch_evict_create(const Store& s, uint32_t w, const uint32_t* create_list,
                          const uint32_t* evict_list, uint64_t max_events, int sms,
                          cudaStream_t stream, AdvCounts* early) {
+  if (s.own != nullptr) return launch_evict_create_copied(s, w, create_list, evict_list, max_events, sms, stream);
   dispatch_gc(s.D / 4, [&](auto Gc, auto Cc) {
     constexpr int G = decltype(Gc)::value, C = decltype(Cc)::value;
-    constexpr uint64_t R = 4 / C > 0 ? 4 / C : 1;   // list entries per group, as in the kernel
-    const unsigned grid = grid_for((max_events + R - 1) / R, G, sms);
+    // at least four entries per warp, at most the blocks that are resident together
+    uint64_t blocks = (max_events + 4 * (kThreads / 32) - 1) / (4 * (kThreads / 32));
+    const uint64_t resident = (uint64_t)sms * evict_blocks_per_sm(C);
+    if (blocks > resident) blocks = resident;
+    if (blocks < 1) blocks = 1;
+    const unsigned grid = (unsigned)blocks;
     note_launches(1);
     evict_create_kernel<G, C><<<grid, kThreads, 0, stream>>>(s, w, evict_list, create_list, early);
   });

@@ -3,10 +3,14 @@
 // Device data layout (all in HBM, owned by the context):
 //   main        [K][D] fp32     main copy of every parameter
 //   val, acc    [S][D] fp32     replica pool: local value and pending updates
-//   map         [W][K] int32    slot of worker w's replica of key k, or -1
+//                               (rows are written only when needed, see RepState)
+//   map         [W][K] int32    worker w's replica of key k: -1 if none, else its
+//                               slot, with bit 31 set when slot_owner may hold
+//                               a state other than REP_ALIAS (see map_touched)
 //   rc          [W][K] uint32   number of w's active intents containing k
 //   holders     [K]    uint32   bit w set iff worker w holds a replica of k
-//   slot_owner  [S]    uint64   (w << 32) | k of a live slot, kEmptySlot if free
+//   slot_owner  [S]    uint64   key, worker and state of a live slot (see
+//                               owner_word), kEmptySlot if free
 //   free_stack  [S]    int32    free slots, top at free_stack[free_top - 1]
 //   stamp       [K]    uint32   tag of the last Intent call that listed k
 //   dirty       [K]    uint8    versioned refresh only: main[k] written other
@@ -52,6 +56,10 @@ struct DevState {
   unsigned long long created;
   unsigned long long destroyed;
   int32_t live;
+  int32_t live_keys;      // keys with at least one replica
+  int32_t sole_keys;      // keys with exactly one replica
+  uint32_t par;           // parity of the syncs so far (see the replica states)
+  uint32_t sync_done;     // blocks of a sync that finished (0 between syncs)
   uint32_t ev_done;       // blocks of the closing events launch that finished (0 between advances)
   uint32_t loss_done;     // blocks of a training step that finished (0 between steps)
   unsigned long long push_rows;       // rows pushed (cumulative)
@@ -94,7 +102,111 @@ struct Store {
   uint64_t S;
   uint32_t D;
   uint32_t W;
+  uint32_t par;     // kernels that look at replica states: their copy of st->par
 };
+
+// ---- replica states ---------------------------------------------------------
+// A replica's value equals its main row until somebody writes either, so its
+// rows are not copied when it is created or refreshed; they are written when
+// the two first differ.  Its state is three flags:
+//   REP_PENDING  acc holds pending updates (else none are pending, acc unset)
+//   REP_OWNVAL   the value's base is val (else main[k], val unset)
+//   REP_FOLDED   val includes acc (only with both of the above)
+// value = base, plus acc when updates are pending and not folded.  0 is an
+// alias of the main row.  The first push to a replica after its creation or
+// a sync stores its sum in acc and leaves the base alone, later ones fold
+// acc into val; whoever writes main[k] while other workers' replicas have it
+// as their base (an evicted replica's pending updates, a push of a worker
+// without a replica) first copies the old row to their val.  A sync merges
+// the pending rows and leaves every replica an alias again.  The values are
+// those of replicas that are copied at creation and written by every push
+// (the same sums in the same order) with a third of the row traffic: a
+// replica that is created, pushed to once, synced and evicted moves 4 rows
+// instead of 15, one whose key other workers evict meanwhile 6.
+//
+// The state lives in slot_owner beside the parity of the syncs made when it
+// was written.  The last block of a sync flips the parity, which makes every
+// state an alias at once without a write that other blocks of the sync could
+// see half done; the states it voids are cleared by the next sync's scan.
+// Bit 31 of a map entry says that slot_owner has to be read: an entry without
+// it is an alias.
+//
+// With relocation (s.own set) the main copy of a replicated key is written by
+// its owner on every push, so every alias would be detached at once, by the
+// push: there replicas are copied at creation, refreshed by every sync and
+// always in the state REP_COPIED, which is not stored.  (Measured with
+// aliases there: 8 x 2^18 Zipf(1.1) keys of 64 floats, push 461 -> 566 us per
+// clock, the clock 1261 -> 1382 us.)
+constexpr uint32_t REP_ALIAS = 0u;
+constexpr uint32_t REP_PENDING = 1u;
+constexpr uint32_t REP_OWNVAL = 2u;
+constexpr uint32_t REP_FOLDED = 4u;
+constexpr uint32_t REP_COPIED = REP_PENDING | REP_OWNVAL | REP_FOLDED;
+__host__ __device__ __forceinline__ bool rep_adds(uint32_t state) {   // acc is added to the base
+  return (state & (REP_PENDING | REP_FOLDED)) == REP_PENDING;
+}
+
+__host__ __device__ __forceinline__ bool map_none(int32_t e) { return e == -1; }
+__host__ __device__ __forceinline__ bool map_touched(int32_t e) { return e < -1; }   // bit 31, not "none"
+__host__ __device__ __forceinline__ int32_t map_slot(int32_t e) { return e & 0x7FFFFFFF; }
+__host__ __device__ __forceinline__ int32_t map_touch(int32_t slot) { return (int32_t)((uint32_t)slot | 0x80000000u); }
+
+// High word of slot_owner: worker (bits 0-7), state (8-10), parity (11); the
+// low word is the key.
+__device__ __forceinline__ uint32_t owner_hi(uint32_t w, uint32_t state, uint32_t par) {
+  return w | (state << 8) | (par << 11);
+}
+__device__ __forceinline__ unsigned long long owner_word(uint32_t w, uint32_t k, uint32_t state, uint32_t par) {
+  return ((unsigned long long)owner_hi(w, state, par) << 32) | k;
+}
+__device__ __forceinline__ uint32_t owner_worker(unsigned long long ow) { return (uint32_t)(ow >> 32) & 0xFFu; }
+__device__ __forceinline__ uint32_t owner_raw_state(unsigned long long ow) { return (uint32_t)(ow >> 40) & 7u; }
+__device__ __forceinline__ uint32_t owner_par(unsigned long long ow) { return (uint32_t)(ow >> 43) & 1u; }
+__device__ __forceinline__ uint32_t owner_state(unsigned long long ow, uint32_t par) {
+  return owner_par(ow) == par ? owner_raw_state(ow) : REP_ALIAS;
+}
+__device__ __forceinline__ void set_owner_hi(const Store& s, int32_t slot, uint32_t hi) {
+  reinterpret_cast<uint32_t*>(s.slot_owner + slot)[1] = hi;
+}
+// Whether a map entry is one whose value is not (just) the main row.
+__device__ __forceinline__ bool rep_differs(const Store& s, int32_t e) {
+  return s.own != nullptr ? !map_none(e) : map_touched(e);
+}
+// State of the replica behind a map entry that is not -1.
+__device__ __forceinline__ uint32_t rep_state(const Store& s, int32_t e) {
+  if (s.own != nullptr) return REP_COPIED;
+  return map_touched(e) ? owner_state(s.slot_owner[map_slot(e)], s.par) : REP_ALIAS;
+}
+// The row that holds worker's value of key k under map entry e (main, or the
+// replica's own value), and whether the replica's pending row has to be added
+// to it (*add: that row, else null).
+__device__ __forceinline__ const float4* row_source(const Store& s, int32_t e, uint32_t k, const float4** add) {
+  const uint32_t D4 = s.D >> 2;
+  const float4* p = reinterpret_cast<const float4*>(s.main) + (uint64_t)k * D4;
+  *add = nullptr;
+  if (s.own != nullptr) return map_none(e) ? p : reinterpret_cast<const float4*>(s.val) + (uint64_t)e * D4;
+  if (map_touched(e)) {
+    const uint64_t off = (uint64_t)map_slot(e) * D4;
+    const uint32_t state = rep_state(s, e);
+    if (state & REP_OWNVAL) p = reinterpret_cast<const float4*>(s.val) + off;
+    if (rep_adds(state)) *add = reinterpret_cast<const float4*>(s.acc) + off;
+  }
+  return p;
+}
+// Before main[k] changes: worker b's replica of k, if it has the main row as
+// its base, becomes one with a value of its own.  Returns the slot whose val
+// row the caller then copies the old main row to, -1 if there is none.
+__device__ __forceinline__ int32_t take_alias(const Store& s, uint32_t b, uint32_t k) {
+  int32_t* me = s.map + (uint64_t)b * s.K + k;
+  const int32_t e = *me;
+  if (map_none(e)) return -1;
+  const uint32_t state = rep_state(s, e);
+  if (state & REP_OWNVAL) return -1;
+  const int32_t sl = map_slot(e);
+  set_owner_hi(s, sl, owner_hi(b, state | REP_OWNVAL, s.par));
+  if (!map_touched(e)) *me = map_touch(sl);
+  return sl;
+}
 
 // Fields of own[k] (relocation mode).
 __device__ __forceinline__ uint32_t own_count(uint32_t o) { return o & 0xFFu; }
@@ -156,7 +268,7 @@ void compact_sorted_heads(const uint32_t* sk, uint64_t n, uint32_t* out, uint32_
 // Stream compaction (a count / scan / write pass), tmp of compact_tmp_words(n).
 size_t compact_tmp_words(uint64_t n);
 
-// Keys k < K with map_w[k] >= 0, ascending, into out; count to *count.
+// Keys k < K with a replica (map_w[k] != -1), ascending, into out; count to *count.
 void compact_replica_keys(const int32_t* map_w, uint64_t K, uint32_t* out, uint32_t* count,
                           uint32_t* tmp, cudaStream_t stream);
 

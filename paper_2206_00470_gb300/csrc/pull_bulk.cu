@@ -82,7 +82,9 @@ __global__ void __launch_bounds__(kBulkThreads) pull_bulk_kernel(Store s, int w,
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t bar[2];
   __shared__ int s_abort;
+  __shared__ int32_t sum_slot[2][kBulkThreads];   // replica whose pending row is added to a staged row, else -1
   const uint32_t rowb = s.D * 4u;
+  s.par = s.st->par;
   const size_t stage_bytes = (size_t)T * rowb;
   const int32_t* mapw = w >= 0 ? s.map + (uint64_t)w * s.K : nullptr;
   const uint64_t ntiles = (n + T - 1) / T;
@@ -105,11 +107,17 @@ __global__ void __launch_bounds__(kBulkThreads) pull_bulk_kernel(Store s, int w,
     const uint32_t i = threadIdx.x;
     unsigned char* dst = smem + (size_t)b * stage_bytes + (size_t)i * rowb;
     uint32_t nbad = 0;
+    sum_slot[b][i] = -1;
     if (i < rows) {
       const uint32_t k = __ldg(keys + r0 + i);
       if (k < s.K) {
-        const int32_t sl = mapw != nullptr ? __ldg(mapw + k) : -1;
-        const float* src = sl >= 0 ? s.val + (uint64_t)sl * s.D : s.main + (uint64_t)k * s.D;
+        const int32_t e = mapw != nullptr ? __ldg(mapw + k) : -1;
+        const float* src = s.main + (uint64_t)k * s.D;
+        if (rep_differs(s, e)) {
+          const uint32_t state = rep_state(s, e);
+          if (state & REP_OWNVAL) src = s.val + (uint64_t)map_slot(e) * s.D;
+          if (rep_adds(state)) sum_slot[b][i] = map_slot(e);
+        }
         bulk_load(dst, src, rowb, &bar[b]);
       } else {
         bad = true;
@@ -134,6 +142,13 @@ __global__ void __launch_bounds__(kBulkThreads) pull_bulk_kernel(Store s, int w,
       issue(tn, b ^ 1);
     }
     if (threadIdx.x == 0 && !mbar_wait(&bar[b], use[b] & 1u)) s_abort = 1;
+    // one pending push to add (the thread that started the row's copy)
+    const int32_t add = sum_slot[b][threadIdx.x];
+    if (add >= 0 && mbar_wait(&bar[b], use[b] & 1u)) {
+      float4* row = reinterpret_cast<float4*>(smem + (size_t)b * stage_bytes + (size_t)threadIdx.x * rowb);
+      const float4* acc4 = reinterpret_cast<const float4*>(s.acc + (uint64_t)add * s.D);
+      for (uint32_t c = 0; c < (s.D >> 2); ++c) row[c] = f4add(row[c], __ldg(acc4 + c));
+    }
     use[b] += 1;
     fence_proxy_async();   // zero-filled rows (generic writes) before the bulk store reads them
     __syncthreads();

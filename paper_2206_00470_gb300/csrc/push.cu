@@ -15,46 +15,119 @@ namespace adapm {
 
 namespace {
 
-// The sorted keys and positions a push kernel reads: the plan's, unless its
-// check stored a mismatch for this push (then the sort made instead).
-__device__ __forceinline__ PushArgs resolve(const PushArgs& a0) {
-  PushArgs a = a0;
-  if (a.plan_seq != 0u && *reinterpret_cast<const volatile uint32_t*>(a.plan_word) == a.plan_seq) {
+// What a push kernel needs to know before its first row, loaded together (one
+// memory latency, not one per word).  False: an earlier sort gave up, nothing
+// may be touched.  The sorted keys and positions in `a` are the plan's, unless
+// its check stored a mismatch for this push (then the sort made instead).
+// any_replica: there are replicas that may be aliases of a main row.
+__device__ __forceinline__ bool push_begin(Store& s, PushArgs& a, bool& any_replica) {
+  auto ld = [](const void* p) {
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+  };
+  const uint32_t errors = ld(&s.st->errors);
+  const uint32_t miss = ld(a.plan_seq != 0u ? a.plan_word : &s.st->plan_miss);
+  const uint32_t live = ld(&s.st->live);
+  s.par = ld(&s.st->par);
+  if (errors & ERR_TIMEOUT) return false;
+  if (a.plan_seq != 0u && miss == a.plan_seq) {
     a.skeys = a.alt_keys;
     a.spos = a.alt_pos;
   }
-  return a;
+  any_replica = s.own == nullptr && (int32_t)live > 0;
+  return true;
 }
 
 // ---------------------------------------------------------------------------
 // push: chunked segmented reduction over key-sorted (key, position) pairs
 // ---------------------------------------------------------------------------
-template <int C>
-__device__ __forceinline__ void apply_sum(const Store& s, const int32_t* mapw, uint32_t k,
-                                          const float4 (&sum)[C], int lane, int G) {
-  const uint32_t D4 = s.D >> 2;
-  const int32_t sl = mapw[k];
-  float4* val4 = reinterpret_cast<float4*>(s.val);
-  float4* acc4 = reinterpret_cast<float4*>(s.acc);
-  float4* main4 = reinterpret_cast<float4*>(s.main);
-  float4* t1 = sl >= 0 ? val4 + (uint64_t)sl * D4 : main4 + (uint64_t)k * D4;
-  // the segment is the only writer of its targets: vector atomic adds give
-  // the plain fp32 sums without a round trip of the target rows
-#pragma unroll
-  for (int c = 0; c < C; ++c) {
-    const uint32_t col = lane + c * G;
-    if (col < D4) atomicAdd(t1 + col, sum[c]);
+// The target of one key's sum: the worker's replica (slot >= 0) in its state
+// before this push, or main[k] (slot -1) with the workers that hold replicas
+// of k (0: none has to be looked at).
+struct Target {
+  int32_t slot;
+  uint32_t state;
+  uint32_t holders;
+};
+
+// Looks the target of key k up and records the state after this push.  One
+// thread per key and push (the key has one segment).
+__device__ __forceinline__ Target take_target(const Store& s, uint32_t w, uint32_t k, bool any_replica) {
+  int32_t* me = s.map + (uint64_t)w * s.K + k;
+  const int32_t e = *me;
+  Target t{-1, REP_ALIAS, 0u};
+  if (map_none(e)) {
+    if (any_replica) t.holders = s.holders[k];
+    // versioned refresh: main written by a worker without a replica
+    if (s.dirty != nullptr) s.dirty[k] = 1;
+    return t;
   }
-  if (sl >= 0) {
-    float4* t2 = acc4 + (uint64_t)sl * D4;
+  t.slot = map_slot(e);
+  t.state = rep_state(s, e);
+  if (t.state == REP_COPIED) return t;
+  if (!map_touched(e)) *me = map_touch(t.slot);
+  const uint32_t after = (t.state & REP_PENDING) ? REP_PENDING | REP_OWNVAL | REP_FOLDED : t.state | REP_PENDING;
+  set_owner_hi(s, t.slot, owner_hi(w, after, s.par));
+  return t;
+}
+
+// Adds one key's sum to its target (a whole row group).  The segment is the
+// only writer of its targets in this push: a row that is not yet set is
+// stored, others take vector atomic adds, which give the plain fp32 sums
+// without a round trip of the target row.
+template <int G, int C>
+__device__ __forceinline__ void apply_sum(const Store& s, uint32_t k, const Target& t, const float4 (&sum)[C],
+                                          int lane, unsigned gmask) {
+  const uint32_t D4 = s.D >> 2;
+  float4* main4 = reinterpret_cast<float4*>(s.main) + (uint64_t)k * D4;
+  if (t.slot < 0) {
+    if (t.holders) detach_aliases<G, C>(s, k, t.holders, lane, gmask);
 #pragma unroll
     for (int c = 0; c < C; ++c) {
       const uint32_t col = lane + c * G;
-      if (col < D4) atomicAdd(t2 + col, sum[c]);
+      if (col < D4) atomicAdd(main4 + col, sum[c]);
     }
-  } else if (s.dirty != nullptr && lane == 0) {
-    s.dirty[k] = 1;   // versioned refresh: main written by a worker without a replica
+    return;
   }
+  float4* val4 = reinterpret_cast<float4*>(s.val) + (uint64_t)t.slot * D4;
+  float4* acc4 = reinterpret_cast<float4*>(s.acc) + (uint64_t)t.slot * D4;
+  if (rep_adds(t.state)) {   // the second push: acc is folded into a value of the replica's own
+    const float4* base4 = (t.state & REP_OWNVAL) ? val4 : main4;
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      const uint32_t col = lane + c * G;
+      if (col >= D4) continue;
+      const float4 p = acc4[col];
+      val4[col] = f4add(f4add(base4[col], p), sum[c]);
+      acc4[col] = f4add(p, sum[c]);
+    }
+    return;
+  }
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    const uint32_t col = lane + c * G;
+    if (col >= D4) continue;
+    if (t.state & REP_FOLDED) {
+      atomicAdd(val4 + col, sum[c]);
+      atomicAdd(acc4 + col, sum[c]);
+    } else {
+      acc4[col] = sum[c];
+    }
+  }
+}
+
+// The same for a segment whose target nobody has looked up yet: lane 0 of the
+// group does.
+template <int G, int C>
+__device__ __forceinline__ void take_and_apply(const Store& s, uint32_t w, uint32_t k, const float4 (&sum)[C],
+                                               int lane, unsigned gmask, bool any_replica) {
+  Target t{-1, REP_ALIAS, 0u};
+  if (lane == 0) t = take_target(s, w, k, any_replica);
+  t.slot = __shfl_sync(gmask, t.slot, 0, G);
+  t.state = __shfl_sync(gmask, t.state, 0, G);
+  t.holders = __shfl_sync(gmask, t.holders, 0, G);
+  apply_sum<G, C>(s, k, t, sum, lane, gmask);
 }
 
 // Each block stages a span of up to kPushSpan consecutive sorted positions
@@ -63,6 +136,7 @@ __device__ __forceinline__ void apply_sum(const Store& s, const int32_t* mapw, u
 // chunk (a tail piece in the chunk it starts in, head pieces in the chunks
 // it continues into).
 constexpr int kPushSpan = 3072;
+constexpr uint32_t kPushCopies = 1024;
 // resident push_chunks blocks per SM (its launch bounds)
 constexpr int push_blocks_per_sm(int C) { return C >= 4 ? 2 : 3; }
 
@@ -75,13 +149,15 @@ constexpr size_t push_chunks_smem() {
 }
 
 template <int G, int C, int R>
-__global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_kernel(Store s, PushArgs a0) {
-  if (sort_failed(s.st)) return;
-  const PushArgs a = resolve(a0);
+__global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_kernel(Store s, PushArgs a) {
+  bool any_replica;
+  if (!push_begin(s, a, any_replica)) return;
   constexpr int NG = kThreads / G;
   const uint32_t CH = (uint32_t)a.chunk;            // rows per group, NG * CH <= kPushSpan
   const uint32_t span = NG * CH;
   extern __shared__ __align__(16) unsigned char dsm[];
+  __shared__ uint2 copies[kPushCopies];   // (key, holder), then (key, slot): old main rows to copy first
+  __shared__ uint32_t ncopy;
   float4* ph = reinterpret_cast<float4*>(dsm);                    // head piece of each chunk
   float4* pt = ph + kThreads * C;                                 // tail piece of each chunk
   uint32_t* sk = reinterpret_cast<uint32_t*>(pt + kThreads * C);  // sk[0]: key before the span; sk[1+len]: after it
@@ -91,20 +167,20 @@ __global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_k
   // flags: bit0 a piece ends at this row, bit1 that piece began inside the
   // row's chunk, bit2 the key's segment ends here, bit3 a piece begins here,
   // bit4 the row holds a key (not a skipped one); a row with bits 0-2 all set
-  // ends a segment that lies inside one chunk
+  // ends a segment that lies inside one chunk and carries its target's state
+  // in bits 5-7 (main rows: bit 7 when aliases of it are left to detach)
+  const unsigned gmask = group_mask<G>();
   const int lane = threadIdx.x & (G - 1);
   const int gi = threadIdx.x / G;
   const uint32_t D4 = s.D >> 2;
   const float4* d4 = reinterpret_cast<const float4*>(a.deltas);
-  float4* val4 = reinterpret_cast<float4*>(s.val);
   float4* acc4 = reinterpret_cast<float4*>(s.acc);
-  float4* main4 = reinterpret_cast<float4*>(s.main);
   float4* sp4 = reinterpret_cast<float4*>(a.span_parts);
-  const int32_t* mapw = s.map + (uint64_t)a.worker * s.K;
   uint32_t heads = 0;
   for (uint64_t P0 = (uint64_t)blockIdx.x * span; P0 < a.n; P0 += (uint64_t)gridDim.x * span) {
     const uint32_t len = (uint32_t)(a.n - P0 < (uint64_t)span ? a.n - P0 : span);
     __syncthreads();
+    if (threadIdx.x == 0) ncopy = 0;
     for (uint32_t i = threadIdx.x; i < len; i += kThreads) {
       sk[1 + i] = a.skeys[P0 + i];
       sp[i] = a.spos[P0 + i];
@@ -132,9 +208,18 @@ __global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_k
             ((seg_begin || i == cs) ? 8 : 0) | 16;
         if (seg_begin) ++heads;
         if ((f & 7) == 7) {
-          slot = mapw[k];
-          // versioned refresh: main written by a worker without a replica
-          if (slot < 0 && s.dirty != nullptr) s.dirty[k] = 1;
+          const Target t = take_target(s, a.worker, k, any_replica);
+          slot = t.slot;
+          f |= (uint8_t)(t.state << 5);
+          // a main row that others replicate: its (key, holder) pairs are
+          // listed for the block (as far as the list goes)
+          if (t.holders) {
+            uint32_t at = atomicAdd(&ncopy, (uint32_t)__popc(t.holders));
+            for (uint32_t h = t.holders; h; h &= h - 1, ++at) {
+              if (at < kPushCopies) copies[at] = make_uint2(k, (uint32_t)(__ffs(h) - 1));
+              else f |= 128;
+            }
+          }
         }
       }
       else if (k != kNoKey || sp[i] >= a.n) set_error(s.st, ERR_INTERNAL);
@@ -142,6 +227,26 @@ __global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_k
       ss[i] = slot;
     }
     __syncthreads();
+    if (ncopy) {   // block-uniform
+      // aliases of the main rows that are about to change get the old rows:
+      // one thread per pair for the lookups, then one group per row
+      const uint32_t nc = ncopy < kPushCopies ? ncopy : kPushCopies;
+      for (uint32_t i = threadIdx.x; i < nc; i += kThreads)
+        copies[i].y = (uint32_t)take_alias(s, copies[i].y, copies[i].x);
+      __syncthreads();
+      float4* val4 = reinterpret_cast<float4*>(s.val);
+      const float4* main4 = reinterpret_cast<const float4*>(s.main);
+      for (uint32_t i = gi; i < nc; i += NG) {
+        const uint2 kc = copies[i];
+        if (kc.y == 0xFFFFFFFFu) continue;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          const uint32_t col = lane + c * G;
+          if (col < D4) val4[(uint64_t)kc.y * D4 + col] = main4[(uint64_t)kc.x * D4 + col];
+        }
+      }
+      __syncthreads();
+    }
     const uint32_t p0 = gi * CH;
     const uint32_t p1 = p0 + CH < len ? p0 + CH : len;
     float4 run[C];
@@ -185,26 +290,21 @@ __global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_k
           d[r][c] = run[c];
         }
       }
-      // a whole segment's sum goes to its targets by vector atomic adds: the
-      // segment is the only writer of those rows in this kernel, so the
-      // result is the plain fp32 sum target + s, and no target row has to
-      // travel to the SM and back
+      // a whole segment's sum goes to its target; the usual one is a replica
+      // that has not been pushed to since its creation or the last sync: the
+      // sum becomes its pending row
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        if (sl[r] != -2) {
-          float4* dst = sl[r] >= 0 ? val4 + (uint64_t)sl[r] * D4 : main4 + (uint64_t)k[r] * D4;
+        const uint32_t state = f[r] >> 5;
+        if (sl[r] >= 0 && !(state & REP_PENDING)) {
 #pragma unroll
           for (int c = 0; c < C; ++c) {
             const uint32_t col = lane + c * G;
-            if (col < D4) atomicAdd(dst + col, d[r][c]);
+            if (col < D4) acc4[(uint64_t)sl[r] * D4 + col] = d[r][c];
           }
-          if (sl[r] >= 0) {
-#pragma unroll
-            for (int c = 0; c < C; ++c) {
-              const uint32_t col = lane + c * G;
-              if (col < D4) atomicAdd(acc4 + (uint64_t)sl[r] * D4 + col, d[r][c]);
-            }
-          }
+        } else if (sl[r] != -2) {
+          const Target t{sl[r], state, (sl[r] < 0 && (f[r] & 128)) ? s.holders[k[r]] : 0u};
+          apply_sum<G, C>(s, k[r], t, d[r], lane, gmask);
         } else if (f[r] & 1) {
           // a piece of a segment cut by a chunk boundary: partial sum, kept
           // in shared memory (a chunk has at most one head and one tail piece)
@@ -266,7 +366,7 @@ __global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_k
               if (col < D4) sp4[(2 * sidx + 1) * D4 + col] = tot[c];
             }
           } else {
-            apply_sum<C>(s, mapw, kl, tot, lane, G);
+            take_and_apply<G, C>(s, a.worker, kl, tot, lane, gmask, any_replica);
           }
         }
       }
@@ -301,17 +401,17 @@ __global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_k
 // increasing order, then group 0 adds the tail piece and the group sums in
 // group order: a fixed order, whatever the number of spans.
 template <int G, int C>
-__global__ void __launch_bounds__(kThreads) push_combine_kernel(Store s, PushArgs a0, uint64_t span,
+__global__ void __launch_bounds__(kThreads) push_combine_kernel(Store s, PushArgs a, uint64_t span,
                                                                 uint64_t nspans) {
-  if (sort_failed(s.st)) return;
-  const PushArgs a = resolve(a0);
+  bool any_replica;
+  if (!push_begin(s, a, any_replica)) return;
   constexpr int NG = kThreads / G;
   __shared__ float4 part[NG][G * C];
   const int lane = threadIdx.x & (G - 1);
   const int gi = threadIdx.x / G;
   const uint32_t D4 = s.D >> 2;
   const float4* sp4 = reinterpret_cast<const float4*>(a.span_parts);
-  const int32_t* mapw = s.map + (uint64_t)a.worker * s.K;
+  const unsigned gmask = group_mask<G>();
   for (uint64_t b = blockIdx.x; b < nspans; b += gridDim.x) {   // block-uniform
     const uint64_t st = b * span;
     const uint64_t en = st + span < a.n ? st + span : a.n;
@@ -358,7 +458,7 @@ __global__ void __launch_bounds__(kThreads) push_combine_kernel(Store s, PushArg
         tot[c] = col < D4 ? __ldcg(sp4 + (2 * b + 1) * D4 + col) : f4zero();
         for (int g2 = 0; g2 < NG; ++g2) tot[c] = f4add(tot[c], part[g2][lane + c * G]);
       }
-      apply_sum<C>(s, mapw, kl, tot, lane, G);
+      take_and_apply<G, C>(s, a.worker, kl, tot, lane, gmask, any_replica);
     }
     __syncthreads();
   }

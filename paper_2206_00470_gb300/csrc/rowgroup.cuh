@@ -103,6 +103,41 @@ __device__ __forceinline__ uint64_t group_count() {
   return ((uint64_t)gridDim.x * blockDim.x) / G;
 }
 
+// Lanes of the calling thread's row group within its warp.
+template <int G>
+__device__ __forceinline__ unsigned group_mask() {
+  return G == 32 ? 0xFFFFFFFFu : (((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1)));
+}
+
+// Before main[k] changes: the workers in `holders` whose replica of k has the
+// old row as its base get it as a value of their own (take_alias).  Called by
+// a whole row group, one lane per holder for the lookups; each lane copies
+// its own columns and may then write them in main[k].
+template <int G, int C>
+__device__ __forceinline__ void detach_aliases(const Store& s, uint32_t k, uint32_t holders, int lane,
+                                               unsigned gmask) {
+  const uint32_t D4 = s.D >> 2;
+  const float4* main4 = reinterpret_cast<const float4*>(s.main) + (uint64_t)k * D4;
+  float4* val4 = reinterpret_cast<float4*>(s.val);
+  const int shift = (threadIdx.x & 31) & ~(G - 1);   // the group's first lane of the warp
+#pragma unroll 1
+  for (int b0 = 0; b0 < 32; b0 += G) {
+    if (G < 32 && ((holders >> b0) & ((1u << (G & 31)) - 1u)) == 0u) continue;
+    const uint32_t b = (uint32_t)(b0 + lane);
+    const int32_t mine = (holders >> b) & 1u ? take_alias(s, b, k) : -1;
+    unsigned left = (__ballot_sync(gmask, mine >= 0) & gmask) >> shift;
+    while (left) {
+      const int32_t sl = __shfl_sync(gmask, mine, __ffs(left) - 1, G);
+      left &= left - 1;
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        const uint32_t col = lane + c * G;
+        if (col < D4) val4[(uint64_t)sl * D4 + col] = main4[col];
+      }
+    }
+  }
+}
+
 template <typename F>
 void dispatch_gc(uint32_t D4, F&& f) {
   if (D4 <= 4) f(std::integral_constant<int, 4>{}, std::integral_constant<int, 1>{});

@@ -571,7 +571,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) sort_kernel(SortArgs a) {
 struct MapSel {
   const int32_t* m;
   uint64_t n;
-  __device__ bool flag(uint64_t i) const { return m[i] >= 0; }
+  __device__ bool flag(uint64_t i) const { return !map_none(m[i]); }
   __device__ uint32_t value(uint64_t i) const { return (uint32_t)i; }
 };
 

@@ -53,11 +53,21 @@ __device__ __forceinline__ float group_sum(float v) {
   return v;
 }
 
-__device__ __forceinline__ const float4* row_ptr(const Store& s, const int32_t* mapw, uint32_t k) {
-  const uint32_t D4 = s.D >> 2;
-  const int32_t sl = mapw[k];
-  return sl >= 0 ? reinterpret_cast<const float4*>(s.val) + (uint64_t)sl * D4
-                 : reinterpret_cast<const float4*>(s.main) + (uint64_t)k * D4;
+// Where a worker's value of a key is read (see RepState): the row, and the
+// pending row to add to it when one push is pending on an alias (few have
+// one at a step: a null pointer otherwise).
+struct Row {
+  const float4* p;
+  const float4* add;
+};
+__device__ __forceinline__ Row row_of(const Store& s, int32_t e, uint32_t k) {
+  Row r;
+  r.p = row_source(s, e, k, &r.add);
+  return r;
+}
+
+__device__ __forceinline__ float4 f4add(float4 a, float4 b) {
+  return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
 }
 
 // Fixed-order block reduction of one double per thread into
@@ -114,6 +124,7 @@ mf_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ rows, const uin
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   const uint32_t dim4 = dim >> 2, D4 = s.D >> 2;
   const int32_t* mapw = s.map + (uint64_t)w * s.K;
+  s.par = s.st->par;
   float4* d4 = reinterpret_cast<float4*>(o.drows);
   double lsum = 0.0;
   // software-pipelined: a round loads the rows of its cell, the slots of the
@@ -139,10 +150,8 @@ mf_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ rows, const uin
     if (in && !ok && lane == 0) set_error(s.st, ERR_KEY_RANGE);
     float4 tu[C], tw[C], au[C], aw[C];
     {
-      const float4* pu = su0 >= 0 ? reinterpret_cast<const float4*>(s.val) + (uint64_t)su0 * D4
-                                  : reinterpret_cast<const float4*>(s.main) + (uint64_t)ku * D4;
-      const float4* pw = sw0 >= 0 ? reinterpret_cast<const float4*>(s.val) + (uint64_t)sw0 * D4
-                                  : reinterpret_cast<const float4*>(s.main) + (uint64_t)kw * D4;
+      const Row ru = row_of(s, su0, ku), rw = row_of(s, sw0, kw);
+      const float4 *pu = ru.p, *pw = rw.p;
 #pragma unroll
       for (int c = 0; c < C; ++c) {
         const uint32_t col = lane + c * G;
@@ -152,15 +161,26 @@ mf_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ rows, const uin
         au[c] = (cv && adagrad) ? pu[dim4 + col] : f4zero();
         aw[c] = (cv && adagrad) ? pw[dim4 + col] : f4zero();
       }
+      // the next cell's slots and the keys of the cell after, issued before
+      // this cell's rows are used
+      su0 = ok1 ? mapw[ku1] : -1;
+      sw0 = ok1 ? mapw[kw1] : -1;
+      ku0 = ku1;
+      kw0 = kw1;
+      ok0 = ok1;
+      ok1 = cell_keys(i + 2 * step, ku1, kw1);
+      if (ru.add || rw.add) {
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          const uint32_t col = lane + c * G;
+          if (!ok || col >= dim4) continue;
+          if (ru.add) tu[c] = f4add(tu[c], ru.add[col]);
+          if (rw.add) tw[c] = f4add(tw[c], rw.add[col]);
+          if (ru.add && adagrad) au[c] = f4add(au[c], ru.add[dim4 + col]);
+          if (rw.add && adagrad) aw[c] = f4add(aw[c], rw.add[dim4 + col]);
+        }
+      }
     }
-    // the next cell's slots and the keys of the cell after, issued before
-    // this cell's rows are used
-    su0 = ok1 ? mapw[ku1] : -1;
-    sw0 = ok1 ? mapw[kw1] : -1;
-    ku0 = ku1;
-    kw0 = kw1;
-    ok0 = ok1;
-    ok1 = cell_keys(i + 2 * step, ku1, kw1);
     float part = 0.f;
 #pragma unroll
     for (int c = 0; c < C; ++c) part += dot4(tu[c], tw[c]);
@@ -204,7 +224,7 @@ mf_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ rows, const uin
 // ComplEx: one triple per warp; lane q holds float4 q of the re and im halves
 // ---------------------------------------------------------------------------
 template <int CC, int U>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, CC == 1 ? 2 : 1)
 complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, const uint32_t* __restrict__ rels,
                     const uint32_t* __restrict__ tails, const uint32_t* __restrict__ negs, uint64_t n,
                     uint32_t n_neg, uint32_t dim, float lr, float eps, StepOut o) {
@@ -214,6 +234,7 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
   const uint32_t h4 = dim >> 3;          // float4 per half (re or im) of theta
   const uint32_t D4 = s.D >> 2;          // = 4 * h4: [theta re | theta im | a re | a im]
   const int32_t* mapw = s.map + (uint64_t)w * s.K;
+  s.par = s.st->par;
   float4* d4 = reinterpret_cast<float4*>(o.drows);
   // delta rows in the order the keys of a batch are listed: all heads, all
   // relations, all true tails, then the negatives triple by triple
@@ -227,22 +248,24 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
       for (uint64_t q = lane; q < n_neg; q += 32) o.dkeys[rneg + i * n_neg + q] = kNoKey;
       continue;
     }
-    const float4* ph = row_ptr(s, mapw, kh);
-    const float4* pr = row_ptr(s, mapw, kr);
-    float4 hre[CC], him[CC], rre[CC], rim[CC], xre[CC], xim[CC], Tre[CC], Tim[CC];
+    const Row ph = row_of(s, mapw[kh], kh);
+    const Row pr = row_of(s, mapw[kr], kr);
+    // float4 q of part p of a row: 0 re, 1 im (theta), 2 re, 3 im (accumulators)
+    auto part4 = [&](const Row& row, uint32_t p, uint32_t q) {
+      float4 v = q < h4 ? row.p[p * h4 + q] : f4zero();
+      if (row.add && q < h4) v = f4add(v, row.add[p * h4 + q]);
+      return v;
+    };
+    float4 xre[CC], xim[CC], Tre[CC], Tim[CC];
 #pragma unroll
     for (int c = 0; c < CC; ++c) {
       const uint32_t q = lane + 32 * c;
-      const bool cv = q < h4;
-      hre[c] = cv ? ph[q] : f4zero();
-      him[c] = cv ? ph[h4 + q] : f4zero();
-      rre[c] = cv ? pr[q] : f4zero();
-      rim[c] = cv ? pr[h4 + q] : f4zero();
+      const float4 hre = part4(ph, 0, q), him = part4(ph, 1, q), rre = part4(pr, 0, q), rim = part4(pr, 1, q);
       // complex product h*r: d phi / d t
-      xre[c] = make_float4(hre[c].x * rre[c].x - him[c].x * rim[c].x, hre[c].y * rre[c].y - him[c].y * rim[c].y,
-                           hre[c].z * rre[c].z - him[c].z * rim[c].z, hre[c].w * rre[c].w - him[c].w * rim[c].w);
-      xim[c] = make_float4(hre[c].x * rim[c].x + him[c].x * rre[c].x, hre[c].y * rim[c].y + him[c].y * rre[c].y,
-                           hre[c].z * rim[c].z + him[c].z * rre[c].z, hre[c].w * rim[c].w + him[c].w * rre[c].w);
+      xre[c] = make_float4(hre.x * rre.x - him.x * rim.x, hre.y * rre.y - him.y * rim.y,
+                           hre.z * rre.z - him.z * rim.z, hre.w * rre.w - him.w * rim.w);
+      xim[c] = make_float4(hre.x * rim.x + him.x * rre.x, hre.y * rim.y + him.y * rre.y,
+                           hre.z * rim.z + him.z * rre.z, hre.w * rim.w + him.w * rre.w);
       Tre[c] = f4zero();
       Tim[c] = f4zero();
     }
@@ -271,21 +294,20 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
     for (uint32_t j0 = 0; j0 < J; j0 += U) {
       float4 tre[U][CC], tim[U][CC], are[U][CC], aim[U][CC];
       float part[U];
+      uint32_t sums = 0;   // rows with a pending push to add
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const bool vx = k0[u] != kNoKey;
-        const float4* pt = s0[u] >= 0 ? reinterpret_cast<const float4*>(s.val) + (uint64_t)s0[u] * D4
-                                      : reinterpret_cast<const float4*>(s.main) + (uint64_t)k0[u] * D4;
-        part[u] = 0.f;
+        const Row pt = row_of(s, vx ? s0[u] : -1, k0[u]);
+        if (pt.add) sums |= 1u << u;
 #pragma unroll
         for (int c = 0; c < CC; ++c) {
           const uint32_t q = lane + 32 * c;
           const bool cv = vx && q < h4;
-          tre[u][c] = cv ? pt[q] : f4zero();
-          tim[u][c] = cv ? pt[h4 + q] : f4zero();
-          are[u][c] = cv ? pt[2 * h4 + q] : f4zero();
-          aim[u][c] = cv ? pt[3 * h4 + q] : f4zero();
-          part[u] += dot4(xre[c], tre[u][c]) + dot4(xim[c], tim[u][c]);
+          tre[u][c] = cv ? pt.p[q] : f4zero();
+          tim[u][c] = cv ? pt.p[h4 + q] : f4zero();
+          are[u][c] = cv ? pt.p[2 * h4 + q] : f4zero();
+          aim[u][c] = cv ? pt.p[3 * h4 + q] : f4zero();
         }
       }
       int32_t s1[U];
@@ -294,6 +316,28 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
       for (int u = 0; u < U; ++u) s1[u] = k1[u] != kNoKey ? mapw[k1[u]] : -1;
 #pragma unroll
       for (int u = 0; u < U; ++u) k2[u] = tail_key(j0 + 2 * U + u);
+      if (sums) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (!((sums >> u) & 1u)) continue;
+          const float4* pa = reinterpret_cast<const float4*>(s.acc) + (uint64_t)map_slot(s0[u]) * D4;
+#pragma unroll
+          for (int c = 0; c < CC; ++c) {
+            const uint32_t q = lane + 32 * c;
+            if (q >= h4) continue;
+            tre[u][c] = f4add(tre[u][c], pa[q]);
+            tim[u][c] = f4add(tim[u][c], pa[h4 + q]);
+            are[u][c] = f4add(are[u][c], pa[2 * h4 + q]);
+            aim[u][c] = f4add(aim[u][c], pa[3 * h4 + q]);
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        part[u] = 0.f;
+#pragma unroll
+        for (int c = 0; c < CC; ++c) part[u] += dot4(xre[c], tre[u][c]) + dot4(xim[c], tim[u][c]);
+      }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const uint32_t j = j0 + u;
@@ -328,21 +372,23 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
         k1[u] = k2[u];
       }
     }
-    // head and relation: gradients are linear in T = sum_j coef_j t_j
+    // head and relation: gradients are linear in T = sum_j coef_j t_j (their
+    // rows are read again, from the caches, rather than held through the tails)
 #pragma unroll
     for (int c = 0; c < CC; ++c) {
       const uint32_t q = lane + 32 * c;
       if (q >= h4) continue;
-      const float4 gh_re = make_float4(rre[c].x * Tre[c].x + rim[c].x * Tim[c].x, rre[c].y * Tre[c].y + rim[c].y * Tim[c].y,
-                                       rre[c].z * Tre[c].z + rim[c].z * Tim[c].z, rre[c].w * Tre[c].w + rim[c].w * Tim[c].w);
-      const float4 gh_im = make_float4(rre[c].x * Tim[c].x - rim[c].x * Tre[c].x, rre[c].y * Tim[c].y - rim[c].y * Tre[c].y,
-                                       rre[c].z * Tim[c].z - rim[c].z * Tre[c].z, rre[c].w * Tim[c].w - rim[c].w * Tre[c].w);
-      const float4 gr_re = make_float4(hre[c].x * Tre[c].x + him[c].x * Tim[c].x, hre[c].y * Tre[c].y + him[c].y * Tim[c].y,
-                                       hre[c].z * Tre[c].z + him[c].z * Tim[c].z, hre[c].w * Tre[c].w + him[c].w * Tim[c].w);
-      const float4 gr_im = make_float4(hre[c].x * Tim[c].x - him[c].x * Tre[c].x, hre[c].y * Tim[c].y - him[c].y * Tre[c].y,
-                                       hre[c].z * Tim[c].z - him[c].z * Tre[c].z, hre[c].w * Tim[c].w - him[c].w * Tre[c].w);
-      const float4 ah_re = ph[2 * h4 + q], ah_im = ph[3 * h4 + q];
-      const float4 ar_re = pr[2 * h4 + q], ar_im = pr[3 * h4 + q];
+      const float4 hre = part4(ph, 0, q), him = part4(ph, 1, q), rre = part4(pr, 0, q), rim = part4(pr, 1, q);
+      const float4 gh_re = make_float4(rre.x * Tre[c].x + rim.x * Tim[c].x, rre.y * Tre[c].y + rim.y * Tim[c].y,
+                                       rre.z * Tre[c].z + rim.z * Tim[c].z, rre.w * Tre[c].w + rim.w * Tim[c].w);
+      const float4 gh_im = make_float4(rre.x * Tim[c].x - rim.x * Tre[c].x, rre.y * Tim[c].y - rim.y * Tre[c].y,
+                                       rre.z * Tim[c].z - rim.z * Tre[c].z, rre.w * Tim[c].w - rim.w * Tre[c].w);
+      const float4 gr_re = make_float4(hre.x * Tre[c].x + him.x * Tim[c].x, hre.y * Tre[c].y + him.y * Tim[c].y,
+                                       hre.z * Tre[c].z + him.z * Tim[c].z, hre.w * Tre[c].w + him.w * Tim[c].w);
+      const float4 gr_im = make_float4(hre.x * Tim[c].x - him.x * Tre[c].x, hre.y * Tim[c].y - him.y * Tre[c].y,
+                                       hre.z * Tim[c].z - him.z * Tre[c].z, hre.w * Tim[c].w - him.w * Tre[c].w);
+      const float4 ah_re = part4(ph, 2, q), ah_im = part4(ph, 3, q);
+      const float4 ar_re = part4(pr, 2, q), ar_im = part4(pr, 3, q);
       d4[(rh + i) * D4 + q] = ada_theta4(gh_re, ah_re, lr, eps);
       d4[(rh + i) * D4 + h4 + q] = ada_theta4(gh_im, ah_im, lr, eps);
       d4[(rh + i) * D4 + 2 * h4 + q] = sq4(gh_re);
@@ -365,7 +411,7 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
 // rows per centre: [centre | for each context slot: positive, negatives...]
 // ---------------------------------------------------------------------------
 template <int C, int U>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 2)
 sgns_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ centres, const uint32_t* __restrict__ contexts,
                  const uint32_t* __restrict__ negs, uint64_t n, uint32_t n_ctx, uint32_t n_neg, uint32_t vocab,
                  float lr, StepOut o) {
@@ -374,6 +420,7 @@ sgns_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ centres, cons
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   const uint32_t D4 = s.D >> 2;
   const int32_t* mapw = s.map + (uint64_t)w * s.K;
+  s.par = s.st->par;
   float4* d4 = reinterpret_cast<float4*>(o.drows);
   const uint64_t per = 1 + (uint64_t)n_ctx * (1 + n_neg);
   double lsum = 0.0;
@@ -385,12 +432,13 @@ sgns_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ centres, cons
       for (uint64_t q = lane; q < per; q += 32) o.dkeys[base + q] = kNoKey;
       continue;
     }
-    const float4* pv = row_ptr(s, mapw, kc);
+    const Row pv = row_of(s, mapw[kc], kc);
     float4 v[C], gv[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) {
       const uint32_t col = lane + 32 * c;
-      v[c] = col < D4 ? pv[col] : f4zero();
+      v[c] = col < D4 ? pv.p[col] : f4zero();
+      if (pv.add && col < D4) v[c] = f4add(v[c], pv.add[col]);
       gv[c] = f4zero();
     }
     // the centre's rows in one index space t = j * (1 + n_neg) + q (q = 0:
@@ -426,15 +474,28 @@ sgns_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ centres, cons
     for (int u = 0; u < U; ++u) s0[u] = k0[u] != kNoKey ? mapw[k0[u]] : -1;
     for (uint32_t t0 = 0; t0 < T; t0 += U) {
       float4 x[U][C];
+      uint32_t sums = 0;   // rows with a pending push to add
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const bool vx = k0[u] != kNoKey;
-        const float4* px = s0[u] >= 0 ? reinterpret_cast<const float4*>(s.val) + (uint64_t)s0[u] * D4
-                                      : reinterpret_cast<const float4*>(s.main) + (uint64_t)k0[u] * D4;
+        const Row px = row_of(s, vx ? s0[u] : -1, k0[u]);
+        if (px.add) sums |= 1u << u;
 #pragma unroll
         for (int c = 0; c < C; ++c) {
           const uint32_t col = lane + 32 * c;
-          x[u][c] = (vx && col < D4) ? px[col] : f4zero();
+          x[u][c] = (vx && col < D4) ? px.p[col] : f4zero();
+        }
+      }
+      if (sums) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (!((sums >> u) & 1u)) continue;
+          const float4* pa = reinterpret_cast<const float4*>(s.acc) + (uint64_t)map_slot(s0[u]) * D4;
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            const uint32_t col = lane + 32 * c;
+            if (col < D4) x[u][c] = f4add(x[u][c], pa[col]);
+          }
         }
       }
       // the next round's slots and the tokens of the round after, issued

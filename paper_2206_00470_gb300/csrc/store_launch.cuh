@@ -80,6 +80,11 @@ void launch_evict_create(const Store& s, uint32_t w, const uint32_t* create_list
                          const uint32_t* evict_list, uint64_t max_events, int sms,
                          cudaStream_t stream, AdvCounts* early = nullptr);
 void launch_sync(const Store& s, uint64_t slot_bound, int sms, cudaStream_t stream);
+// The same two for a store with relocation, whose replicas are copies
+// (copied.cu); launch_evict_create and launch_sync call them.
+void launch_evict_create_copied(const Store& s, uint32_t w, const uint32_t* create_list, const uint32_t* evict_list,
+                                uint64_t max_events, int sms, cudaStream_t stream);
+void launch_sync_copied(const Store& s, uint64_t slot_bound, int sms, cudaStream_t stream);
 void launch_refcounts(const Store& s, uint32_t w, const uint32_t* keys, uint64_t n, uint32_t* out,
                       cudaStream_t stream);
 void launch_owners(const Store& s, const uint32_t* keys, uint64_t n, int32_t* out, cudaStream_t stream);
