@@ -58,7 +58,8 @@ METRIC = "pulled+pushed keys/s and training samples/s on 1 GB300; % of HBM roofl
 # workload, scaled by rows); a figure stands for the kernels only while their source is the one captured
 # (source_digest: first 16 hex digits of the sha256 of their code without comments), otherwise the traffic
 # is reported as null.
-PUSH_SOURCES = ("paper_2206_00470_gb300/csrc/push.cu", "paper_2206_00470_gb300/csrc/rowgroup.cuh")
+PUSH_SOURCES = ("paper_2206_00470_gb300/csrc/push.cu", "paper_2206_00470_gb300/csrc/push_kernels.cuh",
+                "paper_2206_00470_gb300/csrc/rowgroup.cuh")
 PUSH_TRAFFIC = {
     "mf": {"bytes_per_row": 79.106e6 / 65536, "sha256_16": "b7ebddd50ef3a39f"},   # profiles/push_scatter_mf_2Mx200K.md
     "micro": {"bytes_per_row": None, "sha256_16": None},

@@ -539,10 +539,22 @@ IntentList* find_plan(adapm_ctx* ctx, uint32_t w, uint64_t n) {
   return nullptr;
 }
 
-// plans = false: the caller knows its keys never follow an intent's order
+// What a training step's push forms its delta rows from (see PushArgs).
+PushArgs step_factors(const StepOut& o, uint32_t kind, uint64_t n, uint32_t per) {
+  PushArgs f{};
+  f.deltas = o.x;
+  f.coef = o.coef;
+  f.x_kind = kind;
+  f.x_n = (uint32_t)n;
+  f.x_per = per;
+  return f;
+}
+
+// `source`: the rows (deltas), or a step's factors.  plans = false: the caller
+// knows its keys never follow an intent's order
 // (the SGNS step), so no plan is looked up.
 adapm_status push_device(adapm_ctx* ctx, uint32_t w, const uint32_t* dkeys, uint64_t n,
-                         const float* drows, bool allow_nokey, bool plans = true) {
+                         const PushArgs& source, bool allow_nokey, bool plans = true) {
   if (n == 0) return ADAPM_OK;
   {
     const adapm_status st = early_make(ctx, w);
@@ -577,7 +589,14 @@ adapm_status push_device(adapm_ctx* ctx, uint32_t w, const uint32_t* dkeys, uint
                &ctx->bar_base, &ctx->dstate->last_unique, nullptr, ctx->stream, &sk, &sp,
                plan ? plan->px : nullptr, plan ? &ctx->dstate->plan_miss : nullptr, seq));
   ctx->push_rows_host += n;
-  PushArgs a{sk, sp, n, drows, chunk, nchunks, w, sparts};
+  PushArgs a = source;
+  a.skeys = sk;
+  a.spos = sp;
+  a.n = n;
+  a.chunk = chunk;
+  a.nchunks = nchunks;
+  a.worker = w;
+  a.span_parts = sparts;
   if (plan) {
     a.skeys = plan->psk;
     a.spos = plan->psp;
@@ -1061,7 +1080,9 @@ adapm_status adapm_push(adapm_ctx* ctx, uint32_t worker, const uint32_t* keys, u
     id.owned = aligned;
     id.dev = aligned;
   }
-  st = push_device(ctx, worker, ik.dev, n, id.dev, false);
+  PushArgs rows{};
+  rows.deltas = id.dev;
+  st = push_device(ctx, worker, ik.dev, n, rows, false);
   pool_free(ctx, ik.owned);
   pool_free(ctx, id.owned);
   return st;
@@ -1151,25 +1172,26 @@ adapm_status adapm_mf_step(adapm_ctx* ctx, uint32_t worker, const uint32_t* row_
   o.loss_out = loss_out ? lo.dev : nullptr;   // summed by the step kernel's last block
   o.loss_done = &ctx->dstate->loss_done;
   CK(pool_alloc(ctx, &o.dkeys, m));
-  CK(pool_alloc(ctx, &o.drows, m * ctx->s.D));
+  CK(pool_alloc(ctx, &o.x, m * ctx->s.D));
   CK(pool_alloc(ctx, &o.loss_part, o.loss_blocks));
   st = early_make(ctx, worker);
   if (st != ADAPM_OK) return st;
   {
     ProfScope ps(ctx, 5);
-    launch_mf_step(ctx->s, worker, ir.dev, ic.dev, iv.dev, n, dim, adagrad != 0, lr, eps, o,
-                   ctx->sms, ctx->stream);
+    launch_mf_step(ctx->s, worker, ir.dev, ic.dev, iv.dev, n, dim, adagrad != 0, lr, eps, o, ctx->sms, ctx->stream);
   }
   {
     ProfScope ps(ctx, 3);
-    st = push_device(ctx, worker, o.dkeys, m, o.drows, true);
+    PushArgs rows{};
+    rows.deltas = o.x;
+    st = push_device(ctx, worker, o.dkeys, m, rows, true);
   }
   if (loss_out) CK(finish_out(ctx, &lo));
   pool_free(ctx, ir.owned);
   pool_free(ctx, ic.owned);
   pool_free(ctx, iv.owned);
   pool_free(ctx, o.dkeys);
-  pool_free(ctx, o.drows);
+  pool_free(ctx, o.x);
   pool_free(ctx, o.loss_part);
   if (st != ADAPM_OK) return st;
   return check_launch(ctx, "mf_step");
@@ -1207,22 +1229,26 @@ adapm_status adapm_complex_step(adapm_ctx* ctx, uint32_t worker, const uint32_t*
   o.loss_out = loss_out ? lo.dev : nullptr;   // summed by the step kernel's last block
   o.loss_done = &ctx->dstate->loss_done;
   CK(pool_alloc(ctx, &o.dkeys, m));
-  CK(pool_alloc(ctx, &o.drows, m * ctx->s.D));
+  CK(pool_alloc(ctx, &o.coef, m));
+  CK(pool_alloc(ctx, &o.x, 3 * n * dim));
   CK(pool_alloc(ctx, &o.loss_part, o.loss_blocks));
   st = early_make(ctx, worker);
   if (st != ADAPM_OK) return st;
   {
     ProfScope ps(ctx, 5);
-    launch_complex_step(ctx->s, worker, ih.dev, ir.dev, it.dev, ineg.dev, n, n_neg, dim, lr, eps,
-                        o, ctx->sms, ctx->stream);
+    launch_complex_step(ctx->s, worker, ih.dev, ir.dev, it.dev, ineg.dev, n, n_neg, dim, o, ctx->sms, ctx->stream);
   }
   {
     ProfScope ps(ctx, 3);
-    st = push_device(ctx, worker, o.dkeys, m, o.drows, true);
+    PushArgs f = step_factors(o, kFactorsComplEx, n, n_neg);
+    f.adagrad = true;
+    f.lr = lr;
+    f.eps = eps;
+    st = push_device(ctx, worker, o.dkeys, m, f, true);
   }
   if (loss_out) CK(finish_out(ctx, &lo));
   for (void* p : {(void*)ih.owned, (void*)ir.owned, (void*)it.owned, (void*)ineg.owned,
-                  (void*)o.dkeys, (void*)o.drows, (void*)o.loss_part})
+                  (void*)o.dkeys, (void*)o.coef, (void*)o.x, (void*)o.loss_part})
     pool_free(ctx, p);
   if (st != ADAPM_OK) return st;
   return check_launch(ctx, "complex_step");
@@ -1260,7 +1286,8 @@ adapm_status adapm_sgns_step(adapm_ctx* ctx, uint32_t worker, const uint32_t* ce
   o.loss_out = loss_out ? lo.dev : nullptr;   // summed by the step kernel's last block
   o.loss_done = &ctx->dstate->loss_done;
   CK(pool_alloc(ctx, &o.dkeys, m));
-  CK(pool_alloc(ctx, &o.drows, m * ctx->s.D));
+  CK(pool_alloc(ctx, &o.coef, m));
+  CK(pool_alloc(ctx, &o.x, 2 * n * dim));
   CK(pool_alloc(ctx, &o.loss_part, o.loss_blocks));
   st = early_make(ctx, worker);
   if (st != ADAPM_OK) return st;
@@ -1273,11 +1300,11 @@ adapm_status adapm_sgns_step(adapm_ctx* ctx, uint32_t worker, const uint32_t* ce
     ProfScope ps(ctx, 3);
     // its rows follow the centres (each with its context and negative slots),
     // never an intent's key order: no plan
-    st = push_device(ctx, worker, o.dkeys, m, o.drows, true, /*plans=*/false);
+    st = push_device(ctx, worker, o.dkeys, m, step_factors(o, kFactorsSGNS, n, (uint32_t)per), true, /*plans=*/false);
   }
   if (loss_out) CK(finish_out(ctx, &lo));
   for (void* p : {(void*)ic.owned, (void*)ix.owned, (void*)ineg.owned, (void*)o.dkeys,
-                  (void*)o.drows, (void*)o.loss_part})
+                  (void*)o.coef, (void*)o.x, (void*)o.loss_part})
     pool_free(ctx, p);
   if (st != ADAPM_OK) return st;
   return check_launch(ctx, "sgns_step");

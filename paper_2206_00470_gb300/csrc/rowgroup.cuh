@@ -152,9 +152,11 @@ void dispatch_gc(uint32_t D4, F&& f) {
 // The push kernels give each lane two float4 of a row where the row allows
 // it, so every row's control work (flags, slots, addresses) is shared by
 // half as many lanes.
+// `pairs`: a lane's float4 come in pairs (AdaGrad halves), so C is even.
 template <class F>
-void dispatch_push_gc(uint32_t D4, F&& f) {
-  if (D4 <= 8) f(std::integral_constant<int, 4>{}, std::integral_constant<int, 2>{});
+void dispatch_push_gc(uint32_t D4, bool pairs, F&& f) {
+  if (D4 > 64 && D4 <= 96 && !pairs) f(std::integral_constant<int, 32>{}, std::integral_constant<int, 3>{});
+  else if (D4 <= 8) f(std::integral_constant<int, 4>{}, std::integral_constant<int, 2>{});
   else if (D4 <= 16) f(std::integral_constant<int, 8>{}, std::integral_constant<int, 2>{});
   else if (D4 <= 32) f(std::integral_constant<int, 16>{}, std::integral_constant<int, 2>{});
   else dispatch_gc(D4, f);

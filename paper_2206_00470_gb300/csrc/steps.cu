@@ -1,14 +1,23 @@
 // Fused training steps of the three sparse workloads (App. C): each reads the
 // rows a sample needs straight through the worker's slot map (replica, else
-// main copy), computes loss and gradients in fp32 from those values, and
-// writes one delta row per row occurrence for the push that follows:
+// main copy) and computes loss and gradients in fp32 from those values.  The
+// delta row of every row occurrence,
 //   AdaGrad rows [theta | a]:  delta = [-lr*g/sqrt(a + g*g + eps) | g*g]
 //   (1/sqrt evaluated with the correctly rounded __frsqrt_rn)
 //   plain SGD:                 delta = -lr*g
+// is written for the push that follows (MF), or formed by it from factors
+// written here (ComplEx, SGNS): g is a scalar of the occurrence (coef) times
+// one of a few rows (x): a triple's h*r (tails) or its head and relation
+// gradients, a centre's vector or its gradient.  So those steps write 4 bytes
+// per occurrence and these rows, not the delta rows (per worker: 8192 centres
+// of 261 rows x 300 floats: 28 MB instead of 2.5 GB; 4096 triples of 103 rows
+// x 512 floats: 14 MB instead of 864 MB), and read no accumulators.
 // Losses: MF 1/2 (v - u.w)^2; ComplEx softplus(-y phi), phi = Re(sum h r
 // conj(t)) with rows [re | im]; SGNS softplus(-u_o.v_c) + sum softplus(u_n.v_c).
-// Every sample's loss is added by one lane into a per-block fp64 partial in
-// a fixed order, so the batch loss is deterministic.
+// Every sample's loss is added into a per-block fp64 partial in a fixed order,
+// so the batch loss is deterministic.
+#include <type_traits>
+
 #include "internal.cuh"
 #include "store_launch.cuh"
 
@@ -21,9 +30,6 @@ constexpr int kThreads = 256;
 __device__ __forceinline__ float4 f4zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
 __device__ __forceinline__ float dot4(float4 a, float4 b) {
   return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w;
-}
-__device__ __forceinline__ float4 f4scale(float4 a, float s) {
-  return make_float4(a.x * s, a.y * s, a.z * s, a.w * s);
 }
 __device__ __forceinline__ float4 f4fma(float4 a, float s, float4 acc) {
   return make_float4(fmaf(a.x, s, acc.x), fmaf(a.y, s, acc.y), fmaf(a.z, s, acc.z), fmaf(a.w, s, acc.w));
@@ -45,6 +51,16 @@ __device__ __forceinline__ float4 ada_theta4(float4 g, float4 a, float lr, float
                      ada_theta(g.z, a.z, lr, eps), ada_theta(g.w, a.w, lr, eps));
 }
 __device__ __forceinline__ float4 sq4(float4 g) { return make_float4(g.x * g.x, g.y * g.y, g.z * g.z, g.w * g.w); }
+__device__ __forceinline__ float4 f4scale(float4 a, float s) {
+  return make_float4(a.x * s, a.y * s, a.z * s, a.w * s);
+}
+
+// The loss of a score x under label +1 (softplus(-x)) or -1 (softplus(x)),
+// added to *loss, and its derivative by x.
+__device__ __forceinline__ float score_coef(float x, bool positive, double* loss) {
+  *loss += (double)(positive ? softplus_f(-x) : softplus_f(x));
+  return positive ? -sigmoid_f(-x) : sigmoid_f(x);
+}
 
 template <int G>
 __device__ __forceinline__ float group_sum(float v) {
@@ -112,6 +128,12 @@ __device__ void block_loss(double v, const StepOut& o) {
 // ---------------------------------------------------------------------------
 // matrix factorisation: one cell per group of G lanes
 // ---------------------------------------------------------------------------
+// The delta rows are written here, unlike the other steps': a batch's rows
+// stay in L2 until the push, and a cell's two rows share nothing that would be
+// read once for many.  (Formed in the push from theta and accumulator halves:
+// step 395 -> 286 us, push 383 -> 536 us per clock of 8 x 65,536 cells of rank
+// 100.)  One cell per group: two in flight take the registers of a third of
+// the resident warps (step 395 -> 587 us).
 template <int G, int C>
 __global__ void __launch_bounds__(kThreads)
 mf_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ rows, const uint32_t* __restrict__ cols,
@@ -125,7 +147,7 @@ mf_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ rows, const uin
   const uint32_t dim4 = dim >> 2, D4 = s.D >> 2;
   const int32_t* mapw = s.map + (uint64_t)w * s.K;
   s.par = s.st->par;
-  float4* d4 = reinterpret_cast<float4*>(o.drows);
+  float4* d4 = reinterpret_cast<float4*>(o.x);
   double lsum = 0.0;
   // software-pipelined: a round loads the rows of its cell, the slots of the
   // next round's cell and the keys of the cell after
@@ -220,37 +242,110 @@ mf_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ rows, const uin
   block_loss(lsum, o);
 }
 
+// Rows of a sample (tails of a triple, context and negative rows of a centre)
+// are taken in batches of 32: lane t looks up row t of the batch (key, map
+// entry, where its value is) while the batches before it are being read, up
+// to the next sample's first ones, and writes its key and scalar.  The warp
+// reads the rows in order, each lane its columns, by 16-byte asynchronous
+// copies into a ring of DEPTH rows in shared memory, U rows consumed at a
+// time: a lane reads back only what it copied itself, so the ring needs no
+// barrier, and the rows in flight take no registers.  (Loaded into registers,
+// U rows at a time with two blocks per SM, the SGNS step spent most of its
+// issue slots waiting for the next U.)
+struct RowBits {   // a Row, passed between lanes; 0: the row is skipped
+  unsigned long long p, add;
+};
+__device__ __forceinline__ RowBits row_bits(const Store& s, int32_t e, uint32_t k) {
+  if (k == kNoKey) return RowBits{0ull, 0ull};
+  const Row r = row_of(s, e, k);
+  return RowBits{reinterpret_cast<unsigned long long>(r.p), reinterpret_cast<unsigned long long>(r.add)};
+}
+
+__device__ __forceinline__ void copy_async16(float4* dst, const float4* src) {
+  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() {   // all but the last N groups have landed
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // ---------------------------------------------------------------------------
 // ComplEx: one triple per warp; lane q holds float4 q of the re and im halves
 // ---------------------------------------------------------------------------
-template <int CC, int U>
-__global__ void __launch_bounds__(kThreads, CC == 1 ? 2 : 1)
+template <int CC, int U, int DEPTH>
+__global__ void __launch_bounds__(kThreads, 2)
 complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, const uint32_t* __restrict__ rels,
                     const uint32_t* __restrict__ tails, const uint32_t* __restrict__ negs, uint64_t n,
-                    uint32_t n_neg, uint32_t dim, float lr, float eps, StepOut o) {
+                    uint32_t n_neg, uint32_t dim, StepOut o) {
+  static_assert(16 % U == 0 && DEPTH <= 16 && U <= DEPTH, "see the batches' second half");
+  extern __shared__ float4 ring_all[];
   const int lane = threadIdx.x & 31;
+  float4* const ring = ring_all + (threadIdx.x >> 5) * (DEPTH * 2 * CC * 32) + lane;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   const uint32_t h4 = dim >> 3;          // float4 per half (re or im) of theta
-  const uint32_t D4 = s.D >> 2;          // = 4 * h4: [theta re | theta im | a re | a im]
+  const uint32_t T4 = 2 * h4;            // float4 of a theta row
   const int32_t* mapw = s.map + (uint64_t)w * s.K;
   s.par = s.st->par;
-  float4* d4 = reinterpret_cast<float4*>(o.drows);
-  // delta rows in the order the keys of a batch are listed: all heads, all
-  // relations, all true tails, then the negatives triple by triple
-  const uint64_t rh = 0, rrel = n, rt = 2 * n, rneg = 3 * n;
+  float4* x4 = reinterpret_cast<float4*>(o.x);   // head gradients, relation gradients, h*r, n rows each
+  // row occurrences in the order the keys of a batch are listed: all heads,
+  // all relations, all true tails, then the negatives triple by triple
+  const uint64_t rrel = n, rt = 2 * n, rneg = 3 * n;
+  // tails: j = 0 is the true tail (label +1), j >= 1 the negatives (label -1)
+  const uint32_t J = 1 + n_neg;
   double lsum = 0.0;
+  auto tail_key = [&](uint64_t i, uint32_t j) -> uint32_t {   // kNoKey: no such row, or skipped
+    if (i >= n || j >= J) return kNoKey;
+    const uint32_t k = j == 0 ? tails[i] : negs[i * n_neg + (j - 1)];
+    if (k >= s.K) {
+      set_error(s.st, ERR_KEY_RANGE);
+      return kNoKey;
+    }
+    return k;
+  };
+  auto entry = [&](uint32_t k) -> int32_t { return k != kNoKey ? mapw[k] : -1; };
+  // this batch's rows, and the next batch's keys
+  uint32_t key = 0, k1 = 0;
+  RowBits cur{0ull, 0ull};
+  auto restart = [&](uint64_t i) {
+    key = tail_key(i, lane);
+    k1 = J > 32 ? tail_key(i, 32 + lane) : tail_key(i + nwarps, lane);
+    cur = row_bits(s, entry(key), key);
+  };
+  restart(warp);
   for (uint64_t i = warp; i < n; i += nwarps) {
     const uint32_t kh = heads[i], kr = rels[i], kt = tails[i];
     if (kh >= s.K || kr >= s.K || kt >= s.K) {
       if (lane == 0) set_error(s.st, ERR_KEY_RANGE);
       if (lane < 3) o.dkeys[(uint64_t)lane * n + i] = kNoKey;
       for (uint64_t q = lane; q < n_neg; q += 32) o.dkeys[rneg + i * n_neg + q] = kNoKey;
+      restart(i + nwarps);
       continue;
     }
+    RowBits nxt{0ull, 0ull};
+    uint32_t islot = 0, cslot = 0;   // ring slots of the next row copied, consumed
+    auto issue = [&](uint32_t r, uint32_t j0) {   // row r of the triple (in the batch at j0 or the next)
+      const float4* pt = reinterpret_cast<const float4*>(__shfl_sync(0xFFFFFFFFu, r < j0 + 32 ? cur.p : nxt.p, r & 31));
+      if (r < J && pt != nullptr) {
+#pragma unroll
+        for (int c = 0; c < CC; ++c) {
+          const uint32_t q = lane + 32 * c;
+          if (q < h4) {
+            copy_async16(ring + (islot * 2 * CC + 2 * c) * 32, pt + q);
+            copy_async16(ring + (islot * 2 * CC + 2 * c + 1) * 32, pt + h4 + q);
+          }
+        }
+      }
+      copy_commit();
+      islot = islot + 1 == DEPTH ? 0 : islot + 1;
+    };
+#pragma unroll
+    for (int r = 0; r < DEPTH; ++r) issue(r, 0);
     const Row ph = row_of(s, mapw[kh], kh);
     const Row pr = row_of(s, mapw[kr], kr);
-    // float4 q of part p of a row: 0 re, 1 im (theta), 2 re, 3 im (accumulators)
+    // float4 q of half p (0 re, 1 im) of a theta row
     auto part4 = [&](const Row& row, uint32_t p, uint32_t q) {
       float4 v = q < h4 ? row.p[p * h4 + q] : f4zero();
       if (row.add && q < h4) v = f4add(v, row.add[p * h4 + q]);
@@ -268,109 +363,88 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
                            hre.z * rim.z + him.z * rre.z, hre.w * rim.w + him.w * rre.w);
       Tre[c] = f4zero();
       Tim[c] = f4zero();
-    }
-    // tails: j = 0 is the true tail (label +1), j >= 1 the negatives (label
-    // -1); software-pipelined: a round loads the tail rows of U indices, the
-    // slots of the next U and the keys of the U after
-    const uint32_t J = 1 + n_neg;
-    auto tail_key = [&](uint32_t j) -> uint32_t {   // kNoKey: skipped
-      if (j >= J) return kNoKey;
-      const uint32_t k = j == 0 ? kt : negs[i * n_neg + (j - 1)];
-      if (k >= s.K) {
-        if (lane == 0) set_error(s.st, ERR_KEY_RANGE);
-        return kNoKey;
+      if (q < h4) {
+        x4[(rt + i) * T4 + q] = xre[c];
+        x4[(rt + i) * T4 + h4 + q] = xim[c];
       }
-      return k;
-    };
-    uint32_t k0[U], k1[U];
-    int32_t s0[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      k0[u] = tail_key(u);
-      k1[u] = tail_key(U + u);
     }
-#pragma unroll
-    for (int u = 0; u < U; ++u) s0[u] = k0[u] != kNoKey ? mapw[k0[u]] : -1;
-    for (uint32_t j0 = 0; j0 < J; j0 += U) {
-      float4 tre[U][CC], tim[U][CC], are[U][CC], aim[U][CC];
-      float part[U];
-      uint32_t sums = 0;   // rows with a pending push to add
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const bool vx = k0[u] != kNoKey;
-        const Row pt = row_of(s, vx ? s0[u] : -1, k0[u]);
-        if (pt.add) sums |= 1u << u;
-#pragma unroll
-        for (int c = 0; c < CC; ++c) {
-          const uint32_t q = lane + 32 * c;
-          const bool cv = vx && q < h4;
-          tre[u][c] = cv ? pt.p[q] : f4zero();
-          tim[u][c] = cv ? pt.p[h4 + q] : f4zero();
-          are[u][c] = cv ? pt.p[2 * h4 + q] : f4zero();
-          aim[u][c] = cv ? pt.p[3 * h4 + q] : f4zero();
-        }
-      }
-      int32_t s1[U];
-      uint32_t k2[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) s1[u] = k1[u] != kNoKey ? mapw[k1[u]] : -1;
-#pragma unroll
-      for (int u = 0; u < U; ++u) k2[u] = tail_key(j0 + 2 * U + u);
-      if (sums) {
+    for (uint32_t j0 = 0; j0 < J; j0 += 32) {
+      const bool any_add = __any_sync(0xFFFFFFFFu, cur.add != 0ull);
+      // the next batch's map entries and the keys of the one after
+      const int32_t e1 = entry(k1);
+      const uint32_t k2 = j0 + 64 < J ? tail_key(i, j0 + 64 + lane)
+                          : j0 + 32 < J ? tail_key(i + nwarps, lane)
+                          : J > 32 ? tail_key(i + nwarps, 32 + lane) : tail_key(i + 2 * nwarps, lane);
+      float mycoef = 0.f;
+      const uint32_t cnt = J - j0 < 32 ? J - j0 : 32;
+#pragma unroll 1
+      for (uint32_t u0 = 0; u0 < cnt; u0 += U) {
+        if (u0 == 16) nxt = row_bits(s, e1, k1);
+        copy_wait<DEPTH - U>();
+        float4 tre[U][CC], tim[U][CC];
+        float part[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          if (!((sums >> u) & 1u)) continue;
-          const float4* pa = reinterpret_cast<const float4*>(s.acc) + (uint64_t)map_slot(s0[u]) * D4;
+          const bool v = u0 + u < cnt && __shfl_sync(0xFFFFFFFFu, cur.p, (u0 + u) & 31) != 0ull;
 #pragma unroll
           for (int c = 0; c < CC; ++c) {
-            const uint32_t q = lane + 32 * c;
-            if (q >= h4) continue;
-            tre[u][c] = f4add(tre[u][c], pa[q]);
-            tim[u][c] = f4add(tim[u][c], pa[h4 + q]);
-            are[u][c] = f4add(are[u][c], pa[2 * h4 + q]);
-            aim[u][c] = f4add(aim[u][c], pa[3 * h4 + q]);
+            const bool cv = v && lane + 32 * c < (int)h4;
+            tre[u][c] = cv ? ring[(cslot * 2 * CC + 2 * c) * 32] : f4zero();
+            tim[u][c] = cv ? ring[(cslot * 2 * CC + 2 * c + 1) * 32] : f4zero();
+          }
+          cslot = cslot + 1 == DEPTH ? 0 : cslot + 1;
+        }
+        if (any_add) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const float4* pa = reinterpret_cast<const float4*>(__shfl_sync(0xFFFFFFFFu, cur.add, (u0 + u) & 31));
+            if (pa == nullptr || u0 + u >= cnt) continue;
+#pragma unroll
+            for (int c = 0; c < CC; ++c) {
+              const uint32_t q = lane + 32 * c;
+              if (q >= h4) continue;
+              tre[u][c] = f4add(tre[u][c], pa[q]);
+              tim[u][c] = f4add(tim[u][c], pa[h4 + q]);
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          part[u] = 0.f;
+#pragma unroll
+          for (int c = 0; c < CC; ++c) part[u] += dot4(xre[c], tre[u][c]) + dot4(xim[c], tim[u][c]);
+          part[u] = group_sum<32>(part[u]);
+        }
+        // (the ring slots just read are free)
+#pragma unroll
+        for (int u = 0; u < U; ++u) issue(j0 + u0 + DEPTH + u, j0);
+        // lane u0 + u evaluates row u's loss and derivative
+        float phi = 0.f;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (lane == (int)(u0 + u)) phi = part[u];
+        const bool eval = (uint32_t)lane >= u0 && (uint32_t)lane < u0 + U && (uint32_t)lane < cnt && key != kNoKey;
+        if (eval) mycoef = score_coef(phi, j0 + lane == 0, &lsum);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const float coef = __shfl_sync(0xFFFFFFFFu, mycoef, (u0 + u) & 31);   // (0 for a skipped row)
+          if (u0 + u >= cnt) continue;
+#pragma unroll
+          for (int c = 0; c < CC; ++c) {
+            Tre[c] = f4fma(tre[u][c], coef, Tre[c]);
+            Tim[c] = f4fma(tim[u][c], coef, Tim[c]);
           }
         }
       }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        part[u] = 0.f;
-#pragma unroll
-        for (int c = 0; c < CC; ++c) part[u] += dot4(xre[c], tre[u][c]) + dot4(xim[c], tim[u][c]);
+      if ((uint32_t)lane < cnt) {
+        const uint64_t row = j0 + lane == 0 ? rt + i : rneg + i * n_neg + (j0 + lane - 1);
+        o.dkeys[row] = key;
+        o.coef[row] = mycoef;
       }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const uint32_t j = j0 + u;
-        const float phi = group_sum<32>(part[u]);
-        if (j >= J) continue;
-        const uint64_t row = j == 0 ? rt + i : rneg + i * n_neg + (j - 1);
-        if (k0[u] == kNoKey) {
-          if (lane == 0) o.dkeys[row] = kNoKey;
-          continue;
-        }
-        const float coef = j == 0 ? -sigmoid_f(-phi) : sigmoid_f(phi);
-        if (lane == 0) lsum += (double)(j == 0 ? softplus_f(-phi) : softplus_f(phi));
-#pragma unroll
-        for (int c = 0; c < CC; ++c) {
-          const uint32_t q = lane + 32 * c;
-          Tre[c] = f4fma(tre[u][c], coef, Tre[c]);
-          Tim[c] = f4fma(tim[u][c], coef, Tim[c]);
-          if (q < h4) {
-            const float4 gre = f4scale(xre[c], coef), gim = f4scale(xim[c], coef);
-            d4[row * D4 + q] = ada_theta4(gre, are[u][c], lr, eps);
-            d4[row * D4 + h4 + q] = ada_theta4(gim, aim[u][c], lr, eps);
-            d4[row * D4 + 2 * h4 + q] = sq4(gre);
-            d4[row * D4 + 3 * h4 + q] = sq4(gim);
-          }
-        }
-        if (lane == 0) o.dkeys[row] = k0[u];
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        k0[u] = k1[u];
-        s0[u] = s1[u];
-        k1[u] = k2[u];
-      }
+      if (cnt <= 16) nxt = row_bits(s, e1, k1);
+      cur = nxt;
+      key = k1;
+      k1 = k2;
     }
     // head and relation: gradients are linear in T = sum_j coef_j t_j (their
     // rows are read again, from the caches, rather than held through the tails)
@@ -379,28 +453,19 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
       const uint32_t q = lane + 32 * c;
       if (q >= h4) continue;
       const float4 hre = part4(ph, 0, q), him = part4(ph, 1, q), rre = part4(pr, 0, q), rim = part4(pr, 1, q);
-      const float4 gh_re = make_float4(rre.x * Tre[c].x + rim.x * Tim[c].x, rre.y * Tre[c].y + rim.y * Tim[c].y,
-                                       rre.z * Tre[c].z + rim.z * Tim[c].z, rre.w * Tre[c].w + rim.w * Tim[c].w);
-      const float4 gh_im = make_float4(rre.x * Tim[c].x - rim.x * Tre[c].x, rre.y * Tim[c].y - rim.y * Tre[c].y,
-                                       rre.z * Tim[c].z - rim.z * Tre[c].z, rre.w * Tim[c].w - rim.w * Tre[c].w);
-      const float4 gr_re = make_float4(hre.x * Tre[c].x + him.x * Tim[c].x, hre.y * Tre[c].y + him.y * Tim[c].y,
-                                       hre.z * Tre[c].z + him.z * Tim[c].z, hre.w * Tre[c].w + him.w * Tim[c].w);
-      const float4 gr_im = make_float4(hre.x * Tim[c].x - him.x * Tre[c].x, hre.y * Tim[c].y - him.y * Tre[c].y,
-                                       hre.z * Tim[c].z - him.z * Tre[c].z, hre.w * Tim[c].w - him.w * Tre[c].w);
-      const float4 ah_re = part4(ph, 2, q), ah_im = part4(ph, 3, q);
-      const float4 ar_re = part4(pr, 2, q), ar_im = part4(pr, 3, q);
-      d4[(rh + i) * D4 + q] = ada_theta4(gh_re, ah_re, lr, eps);
-      d4[(rh + i) * D4 + h4 + q] = ada_theta4(gh_im, ah_im, lr, eps);
-      d4[(rh + i) * D4 + 2 * h4 + q] = sq4(gh_re);
-      d4[(rh + i) * D4 + 3 * h4 + q] = sq4(gh_im);
-      d4[(rrel + i) * D4 + q] = ada_theta4(gr_re, ar_re, lr, eps);
-      d4[(rrel + i) * D4 + h4 + q] = ada_theta4(gr_im, ar_im, lr, eps);
-      d4[(rrel + i) * D4 + 2 * h4 + q] = sq4(gr_re);
-      d4[(rrel + i) * D4 + 3 * h4 + q] = sq4(gr_im);
+      x4[i * T4 + q] = make_float4(rre.x * Tre[c].x + rim.x * Tim[c].x, rre.y * Tre[c].y + rim.y * Tim[c].y,
+                                   rre.z * Tre[c].z + rim.z * Tim[c].z, rre.w * Tre[c].w + rim.w * Tim[c].w);
+      x4[i * T4 + h4 + q] = make_float4(rre.x * Tim[c].x - rim.x * Tre[c].x, rre.y * Tim[c].y - rim.y * Tre[c].y,
+                                        rre.z * Tim[c].z - rim.z * Tre[c].z, rre.w * Tim[c].w - rim.w * Tre[c].w);
+      x4[(rrel + i) * T4 + q] = make_float4(hre.x * Tre[c].x + him.x * Tim[c].x, hre.y * Tre[c].y + him.y * Tim[c].y,
+                                            hre.z * Tre[c].z + him.z * Tim[c].z, hre.w * Tre[c].w + him.w * Tim[c].w);
+      x4[(rrel + i) * T4 + h4 + q] =
+          make_float4(hre.x * Tim[c].x - him.x * Tre[c].x, hre.y * Tim[c].y - him.y * Tre[c].y,
+                      hre.z * Tim[c].z - him.z * Tre[c].z, hre.w * Tim[c].w - him.w * Tre[c].w);
     }
-    if (lane == 0) {
-      o.dkeys[rh + i] = kh;
-      o.dkeys[rrel + i] = kr;
+    if (lane < 2) {
+      o.dkeys[(uint64_t)lane * n + i] = lane == 0 ? kh : kr;
+      o.coef[(uint64_t)lane * n + i] = 1.f;
     }
   }
   block_loss(lsum, o);
@@ -410,28 +475,78 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
 // skip-gram with negative sampling: one centre per warp
 // rows per centre: [centre | for each context slot: positive, negatives...]
 // ---------------------------------------------------------------------------
-template <int C, int U>
+template <int C, int U, int DEPTH>
 __global__ void __launch_bounds__(kThreads, 2)
 sgns_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ centres, const uint32_t* __restrict__ contexts,
                  const uint32_t* __restrict__ negs, uint64_t n, uint32_t n_ctx, uint32_t n_neg, uint32_t vocab,
                  float lr, StepOut o) {
+  static_assert(16 % U == 0 && DEPTH <= 16 && U <= DEPTH, "see the batches' second half");
+  extern __shared__ float4 ring_all[];
   const int lane = threadIdx.x & 31;
+  float4* const ring = ring_all + (threadIdx.x >> 5) * (DEPTH * C * 32) + lane;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   const uint32_t D4 = s.D >> 2;
   const int32_t* mapw = s.map + (uint64_t)w * s.K;
   s.par = s.st->par;
-  float4* d4 = reinterpret_cast<float4*>(o.drows);
+  float4* x4 = reinterpret_cast<float4*>(o.x);   // the centres' vectors, then their gradients
   const uint64_t per = 1 + (uint64_t)n_ctx * (1 + n_neg);
+  // a centre's rows in one index space t = j * (1 + n_neg) + q (q = 0: the
+  // context word, q >= 1: its negatives)
+  const uint32_t per_ctx = 1 + n_neg;
+  const uint32_t T = n_ctx * per_ctx;
   double lsum = 0.0;
+  auto token = [&](uint64_t i, uint32_t t) -> uint32_t {   // the row's key; kNoKey: no such row, or skipped
+    if (i >= n || t >= T) return kNoKey;
+    const uint32_t j = t / per_ctx, q = t - j * per_ctx;
+    const uint32_t oc = contexts[i * n_ctx + j];
+    if (oc == kNoKey) return kNoKey;
+    if (oc >= vocab) {
+      if (q == 0) set_error(s.st, ERR_KEY_RANGE);
+      return kNoKey;
+    }
+    const uint32_t tok = q == 0 ? oc : negs[(i * n_ctx + j) * n_neg + (q - 1)];
+    if (tok >= vocab) {
+      set_error(s.st, ERR_KEY_RANGE);
+      return kNoKey;
+    }
+    return vocab + tok;
+  };
+  auto entry = [&](uint32_t k) -> int32_t { return k != kNoKey ? mapw[k] : -1; };
+  // this batch's rows, and the next batch's keys
+  uint32_t key = 0, k1 = 0;
+  RowBits cur{0ull, 0ull};
+  auto restart = [&](uint64_t i) {
+    key = token(i, lane);
+    k1 = T > 32 ? token(i, 32 + lane) : token(i + nwarps, lane);
+    cur = row_bits(s, entry(key), key);
+  };
+  restart(warp);
   for (uint64_t i = warp; i < n; i += nwarps) {
     const uint64_t base = i * per;
     const uint32_t kc = centres[i];
     if (kc >= vocab) {
       if (lane == 0) set_error(s.st, ERR_KEY_RANGE);
       for (uint64_t q = lane; q < per; q += 32) o.dkeys[base + q] = kNoKey;
+      restart(i + nwarps);
       continue;
     }
+    RowBits nxt{0ull, 0ull};
+    uint32_t islot = 0, cslot = 0;   // ring slots of the next row copied, consumed
+    auto issue = [&](uint32_t r, uint32_t t0) {   // row r of the centre (in the batch at t0 or the next)
+      const float4* px = reinterpret_cast<const float4*>(__shfl_sync(0xFFFFFFFFu, r < t0 + 32 ? cur.p : nxt.p, r & 31));
+      if (r < T && px != nullptr) {
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          const uint32_t col = lane + 32 * c;
+          if (col < D4) copy_async16(ring + (islot * C + c) * 32, px + col);
+        }
+      }
+      copy_commit();
+      islot = islot + 1 == DEPTH ? 0 : islot + 1;
+    };
+#pragma unroll
+    for (int r = 0; r < DEPTH; ++r) issue(r, 0);
     const Row pv = row_of(s, mapw[kc], kc);
     float4 v[C], gv[C];
 #pragma unroll
@@ -440,115 +555,101 @@ sgns_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ centres, cons
       v[c] = col < D4 ? pv.p[col] : f4zero();
       if (pv.add && col < D4) v[c] = f4add(v[c], pv.add[col]);
       gv[c] = f4zero();
+      if (col < D4) x4[i * D4 + col] = v[c];
     }
-    // the centre's rows in one index space t = j * (1 + n_neg) + q (q = 0:
-    // the context word, q >= 1: its negatives), software-pipelined: a round
-    // loads the rows of U indices, the slots of the next U and the tokens of
-    // the U after, so one memory latency per round
-    const uint32_t per_ctx = 1 + n_neg;
-    const uint32_t T = n_ctx * per_ctx;
-    auto token = [&](uint32_t t) -> uint32_t {   // the row's key, kNoKey when it is skipped
-      if (t >= T) return kNoKey;
-      const uint32_t j = t / per_ctx, q = t - j * per_ctx;
-      const uint32_t oc = contexts[i * n_ctx + j];
-      if (oc == kNoKey) return kNoKey;
-      if (oc >= vocab) {
-        if (q == 0 && lane == 0) set_error(s.st, ERR_KEY_RANGE);
-        return kNoKey;
-      }
-      const uint32_t tok = q == 0 ? oc : negs[(i * n_ctx + j) * n_neg + (q - 1)];
-      if (tok >= vocab) {
-        if (lane == 0) set_error(s.st, ERR_KEY_RANGE);
-        return kNoKey;
-      }
-      return vocab + tok;
-    };
-    uint32_t k0[U], k1[U];
-    int32_t s0[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      k0[u] = token(u);
-      k1[u] = token(U + u);
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) s0[u] = k0[u] != kNoKey ? mapw[k0[u]] : -1;
-    for (uint32_t t0 = 0; t0 < T; t0 += U) {
-      float4 x[U][C];
-      uint32_t sums = 0;   // rows with a pending push to add
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const bool vx = k0[u] != kNoKey;
-        const Row px = row_of(s, vx ? s0[u] : -1, k0[u]);
-        if (px.add) sums |= 1u << u;
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-          const uint32_t col = lane + 32 * c;
-          x[u][c] = (vx && col < D4) ? px.p[col] : f4zero();
-        }
-      }
-      if (sums) {
+    for (uint32_t t0 = 0; t0 < T; t0 += 32) {
+      const bool any_add = __any_sync(0xFFFFFFFFu, cur.add != 0ull);
+      // the next batch's map entries and the keys of the one after
+      const int32_t e1 = entry(k1);
+      const uint32_t k2 = t0 + 64 < T ? token(i, t0 + 64 + lane)
+                          : t0 + 32 < T ? token(i + nwarps, lane)
+                          : T > 32 ? token(i + nwarps, 32 + lane) : token(i + 2 * nwarps, lane);
+      const bool positive = (t0 + lane) % per_ctx == 0;
+      float mycoef = 0.f;
+      const uint32_t cnt = T - t0 < 32 ? T - t0 : 32;
+#pragma unroll 1
+      for (uint32_t u0 = 0; u0 < cnt; u0 += U) {
+        if (u0 == 16) nxt = row_bits(s, e1, k1);
+        copy_wait<DEPTH - U>();
+        float4 x[U][C];
+        float part[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          if (!((sums >> u) & 1u)) continue;
-          const float4* pa = reinterpret_cast<const float4*>(s.acc) + (uint64_t)map_slot(s0[u]) * D4;
+          const bool vx = u0 + u < cnt && __shfl_sync(0xFFFFFFFFu, cur.p, (u0 + u) & 31) != 0ull;
 #pragma unroll
-          for (int c = 0; c < C; ++c) {
-            const uint32_t col = lane + 32 * c;
-            if (col < D4) x[u][c] = f4add(x[u][c], pa[col]);
+          for (int c = 0; c < C; ++c)
+            x[u][c] = vx && lane + 32 * c < (int)D4 ? ring[(cslot * C + c) * 32] : f4zero();
+          cslot = cslot + 1 == DEPTH ? 0 : cslot + 1;
+        }
+        if (any_add) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const float4* pa = reinterpret_cast<const float4*>(__shfl_sync(0xFFFFFFFFu, cur.add, (u0 + u) & 31));
+            if (pa == nullptr || u0 + u >= cnt) continue;
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+              const uint32_t col = lane + 32 * c;
+              if (col < D4) x[u][c] = f4add(x[u][c], pa[col]);
+            }
           }
         }
-      }
-      // the next round's slots and the tokens of the round after, issued
-      // before this round's rows are used
-      int32_t s1[U];
-      uint32_t k2[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) s1[u] = k1[u] != kNoKey ? mapw[k1[u]] : -1;
+        for (int u = 0; u < U; ++u) {
+          part[u] = 0.f;
 #pragma unroll
-      for (int u = 0; u < U; ++u) k2[u] = token(t0 + 2 * U + u);
-      float part[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        part[u] = 0.f;
-#pragma unroll
-        for (int c = 0; c < C; ++c) part[u] += dot4(x[u][c], v[c]);
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const uint32_t t = t0 + u;
-        const float sc = group_sum<32>(part[u]);
-        if (t >= T) continue;
-        const uint64_t row = base + 1 + t;
-        if (k0[u] == kNoKey) {
-          if (lane == 0) o.dkeys[row] = kNoKey;
-          continue;
+          for (int c = 0; c < C; ++c) part[u] += dot4(x[u][c], v[c]);
+          part[u] = group_sum<32>(part[u]);
         }
-        const bool positive = t % per_ctx == 0;
-        const float coef = positive ? -sigmoid_f(-sc) : sigmoid_f(sc);
-        if (lane == 0) lsum += (double)(positive ? softplus_f(-sc) : softplus_f(sc));
+        // (the ring slots just read are free)
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-          const uint32_t col = lane + 32 * c;
-          gv[c] = f4fma(x[u][c], coef, gv[c]);
-          if (col < D4) d4[row * D4 + col] = f4scale(v[c], -lr * coef);
+        for (int u = 0; u < U; ++u) issue(t0 + u0 + DEPTH + u, t0);
+        // lane u0 + u evaluates row u's loss and derivative
+        float sc = 0.f;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (lane == (int)(u0 + u)) sc = part[u];
+        const bool eval = (uint32_t)lane >= u0 && (uint32_t)lane < u0 + U && (uint32_t)lane < cnt && key != kNoKey;
+        if (eval) mycoef = score_coef(sc, positive, &lsum);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const float coef = __shfl_sync(0xFFFFFFFFu, mycoef, (u0 + u) & 31);   // (0 for a skipped row)
+          if (u0 + u >= cnt) continue;
+#pragma unroll
+          for (int c = 0; c < C; ++c) gv[c] = f4fma(x[u][c], coef, gv[c]);
         }
-        if (lane == 0) o.dkeys[row] = k0[u];
       }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        k0[u] = k1[u];
-        s0[u] = s1[u];
-        k1[u] = k2[u];
+      if ((uint32_t)lane < cnt) {
+        o.dkeys[base + 1 + t0 + lane] = key;
+        o.coef[base + 1 + t0 + lane] = -lr * mycoef;
       }
+      if (cnt <= 16) nxt = row_bits(s, e1, k1);
+      cur = nxt;
+      key = k1;
+      k1 = k2;
     }
 #pragma unroll
     for (int c = 0; c < C; ++c) {
       const uint32_t col = lane + 32 * c;
-      if (col < D4) d4[base * D4 + col] = f4scale(gv[c], -lr);
+      if (col < D4) x4[(n + i) * D4 + col] = gv[c];
     }
-    if (lane == 0) o.dkeys[base] = kc;
+    if (lane == 0) {
+      o.dkeys[base] = kc;
+      o.coef[base] = -lr;
+    }
+    if (T == 0) restart(i + nwarps);   // (no batch moved the lookups on)
   }
   block_loss(lsum, o);
+}
+
+// The ring's dynamic shared memory per block; a kernel's limit is a
+// per-device attribute, set once.
+template <typename Kernel>
+void allow_smem(Kernel kernel, size_t bytes, bool (&set)[64]) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 0 && dev < 64 && set[dev]) return;
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (dev >= 0 && dev < 64) set[dev] = true;
 }
 
 }  // namespace
@@ -567,18 +668,26 @@ void launch_mf_step(const Store& s, uint32_t w, const uint32_t* rows, const uint
   else if (dim4 <= 16) mf_step_kernel<16, 1><<<grid, kThreads, 0, stream>>>(s, w, rows, cols, vals, n, dim, a, lr, eps, o);
   else if (dim4 <= 32) mf_step_kernel<32, 1><<<grid, kThreads, 0, stream>>>(s, w, rows, cols, vals, n, dim, a, lr, eps, o);
   else if (dim4 <= 64) mf_step_kernel<32, 2><<<grid, kThreads, 0, stream>>>(s, w, rows, cols, vals, n, dim, a, lr, eps, o);
-  else mf_step_kernel<32, 4><<<grid, kThreads, 0, stream>>>(s, w, rows, cols, vals, n, dim, a, lr, eps, o);
+  else if (dim4 <= 128) mf_step_kernel<32, 4><<<grid, kThreads, 0, stream>>>(s, w, rows, cols, vals, n, dim, a, lr, eps, o);
+  else mf_step_kernel<32, 8><<<grid, kThreads, 0, stream>>>(s, w, rows, cols, vals, n, dim, a, lr, eps, o);
 }
 
 void launch_complex_step(const Store& s, uint32_t w, const uint32_t* heads, const uint32_t* rels,
                          const uint32_t* tails, const uint32_t* negs, uint64_t n, uint32_t n_neg,
-                         uint32_t dim, float lr, float eps, const StepOut& o, int sms,
-                         cudaStream_t stream) {
+                         uint32_t dim, const StepOut& o, int sms, cudaStream_t stream) {
   const unsigned grid = o.loss_blocks;
   note_launches(1);
   const uint32_t h4 = dim / 8;
-  if (h4 <= 32) complex_step_kernel<1, 4><<<grid, kThreads, 0, stream>>>(s, w, heads, rels, tails, negs, n, n_neg, dim, lr, eps, o);
-  else complex_step_kernel<2, 2><<<grid, kThreads, 0, stream>>>(s, w, heads, rels, tails, negs, n, n_neg, dim, lr, eps, o);
+  auto run = [&](auto CCc, auto Uc, auto Dc) {
+    constexpr int CC = decltype(CCc)::value, U = decltype(Uc)::value, DEPTH = decltype(Dc)::value;
+    constexpr size_t smem = (size_t)kThreads * DEPTH * 2 * CC * sizeof(float4);
+    static bool set[64] = {false};
+    allow_smem(complex_step_kernel<CC, U, DEPTH>, smem, set);
+    complex_step_kernel<CC, U, DEPTH><<<grid, kThreads, smem, stream>>>(s, w, heads, rels, tails, negs, n, n_neg, dim, o);
+  };
+  // ring depths: as many rows as two blocks' rings hold per SM (96 KB each)
+  if (h4 <= 32) run(std::integral_constant<int, 1>{}, std::integral_constant<int, 4>{}, std::integral_constant<int, 12>{});
+  else run(std::integral_constant<int, 2>{}, std::integral_constant<int, 2>{}, std::integral_constant<int, 6>{});
 }
 
 void launch_sgns_step(const Store& s, uint32_t w, const uint32_t* centres, const uint32_t* contexts,
@@ -588,10 +697,18 @@ void launch_sgns_step(const Store& s, uint32_t w, const uint32_t* centres, const
   const unsigned grid = o.loss_blocks;
   note_launches(1);
   const uint32_t D4 = dim / 4;
-  if (D4 <= 32) sgns_step_kernel<1, 8><<<grid, kThreads, 0, stream>>>(s, w, centres, contexts, negs, n, n_ctx, n_neg, vocab, lr, o);
-  else if (D4 <= 64) sgns_step_kernel<2, 4><<<grid, kThreads, 0, stream>>>(s, w, centres, contexts, negs, n, n_ctx, n_neg, vocab, lr, o);
-  else if (D4 <= 96) sgns_step_kernel<3, 2><<<grid, kThreads, 0, stream>>>(s, w, centres, contexts, negs, n, n_ctx, n_neg, vocab, lr, o);
-  else sgns_step_kernel<8, 1><<<grid, kThreads, 0, stream>>>(s, w, centres, contexts, negs, n, n_ctx, n_neg, vocab, lr, o);
+  auto run = [&](auto Cc, auto Uc, auto Dc) {
+    constexpr int C = decltype(Cc)::value, U = decltype(Uc)::value, DEPTH = decltype(Dc)::value;
+    constexpr size_t smem = (size_t)kThreads * DEPTH * C * sizeof(float4);
+    static bool set[64] = {false};
+    allow_smem(sgns_step_kernel<C, U, DEPTH>, smem, set);
+    sgns_step_kernel<C, U, DEPTH><<<grid, kThreads, smem, stream>>>(s, w, centres, contexts, negs, n, n_ctx, n_neg, vocab, lr, o);
+  };
+  // ring depths: as many rows as two blocks' rings hold per SM (96 KB each), 16 at most
+  if (D4 <= 32) run(std::integral_constant<int, 1>{}, std::integral_constant<int, 4>{}, std::integral_constant<int, 16>{});
+  else if (D4 <= 64) run(std::integral_constant<int, 2>{}, std::integral_constant<int, 4>{}, std::integral_constant<int, 12>{});
+  else if (D4 <= 96) run(std::integral_constant<int, 3>{}, std::integral_constant<int, 4>{}, std::integral_constant<int, 8>{});
+  else run(std::integral_constant<int, 8>{}, std::integral_constant<int, 1>{}, std::integral_constant<int, 3>{});
 }
 
 }  // namespace adapm

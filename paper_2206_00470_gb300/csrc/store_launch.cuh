@@ -25,7 +25,22 @@ struct PushArgs {
   const uint32_t* alt_pos = nullptr;
   const uint32_t* plan_word = nullptr;
   uint32_t plan_seq = 0;
+  // A training step's push (coef set): the delta row at position p is formed
+  // from g = coef[p] * x (`deltas` holds the rows x, see factor_row): it is
+  // g, or with adagrad [-lr * g / sqrt(a + g*g + eps) | g*g], x and g half a
+  // row wide and a the accumulator half of the worker's value of the key
+  // before the push.
+  const float* coef = nullptr;
+  uint32_t x_kind = 0;
+  uint32_t x_n = 0;       // samples of the batch
+  uint32_t x_per = 1;     // negatives per triple, rows per centre
+  bool adagrad = false;
+  float lr = 0.f, eps = 0.f;
 };
+
+// Sources of a push's delta rows, and the layouts of a step's factor rows.
+constexpr int kSrcRows = 0, kSrcSgd = 1, kSrcAda = 2;
+constexpr uint32_t kFactorsComplEx = 0, kFactorsSGNS = 1;
 
 // Rows of span_parts scratch for nchunks chunks (2 per span, spans of >= 8 chunks).
 uint64_t push_span_part_rows(uint64_t nchunks);
@@ -56,6 +71,7 @@ bool pull_bulk_fits(uint32_t D, const void* out);
 void launch_pull_bulk(const Store& s, int w, const uint32_t* keys, uint64_t n, float* out, int sms,
                       cudaStream_t stream);
 void launch_push(const Store& s, const PushArgs& a, int sms, cudaStream_t stream);
+void launch_push_factors(const Store& s, const PushArgs& a, int sms, cudaStream_t stream);   // (coef set)
 // Refcount events of one advance of worker w: keys to create a replica of
 // for w go to create_list, replica slots to destroy (of w, and in relocation
 // mode of a worker the key is relocated to) to evict_list; the counters
@@ -93,11 +109,14 @@ void launch_replica_rows(const Store& s, uint32_t w, const uint32_t* keys, uint6
 void launch_init_pool(int32_t* free_stack, uint64_t S, unsigned long long* owner, cudaStream_t stream);
 
 // Fused training steps (steps.cu): read rows through the worker's slot map,
-// write one delta row per row occurrence (keys to dkeys, rows to drows) and
-// the per-block loss partials to loss_part; then the caller pushes.
+// write for every row occurrence its key (dkeys) and its delta row (MF: x), or
+// its scalar (coef) and the rows the delta rows are formed from (x; see
+// factor_row), and the per-block loss partials to loss_part; then the caller
+// pushes.
 struct StepOut {
   uint32_t* dkeys;
-  float* drows;
+  float* coef;   // null: x holds delta rows
+  float* x;
   double* loss_part;     // grid-sized partial sums
   unsigned loss_blocks;  // number of partials written
   double* loss_out;      // the batch loss (summed by the last block), or nullptr
@@ -109,8 +128,7 @@ void launch_mf_step(const Store& s, uint32_t w, const uint32_t* rows, const uint
                     const StepOut& o, int sms, cudaStream_t stream);
 void launch_complex_step(const Store& s, uint32_t w, const uint32_t* heads, const uint32_t* rels,
                          const uint32_t* tails, const uint32_t* negs, uint64_t n, uint32_t n_neg,
-                         uint32_t dim, float lr, float eps, const StepOut& o, int sms,
-                         cudaStream_t stream);
+                         uint32_t dim, const StepOut& o, int sms, cudaStream_t stream);
 void launch_sgns_step(const Store& s, uint32_t w, const uint32_t* centres, const uint32_t* contexts,
                       const uint32_t* negs, uint64_t n, uint32_t n_ctx, uint32_t n_neg,
                       uint32_t vocab, uint32_t dim, float lr, const StepOut& o, int sms,
