@@ -145,6 +145,18 @@ def _torch():
     return torch
 
 
+_torch_types = None   # (Tensor, int32, float32), once torch is needed
+
+
+def _plain_tensor(a, which):
+    """Whether `a` is a contiguous tensor of int32 (which = 1) or float32 (2): passed on as it is."""
+    global _torch_types
+    if _torch_types is None:
+        torch = _torch()
+        _torch_types = (torch.Tensor, torch.int32, torch.float32)
+    return isinstance(a, _torch_types[0]) and a.dtype is _torch_types[which] and a.is_contiguous()
+
+
 class _Arr:
     """A pointer to a contiguous array and the object that keeps it alive."""
 
@@ -157,6 +169,9 @@ class _Arr:
 def _keys(a):
     if a is None:
         return _Arr(None, None, 0)
+    if _plain_tensor(a, 1):
+        n = a.numel()
+        return _Arr(a.data_ptr() if n else None, a, n)
     if isinstance(a, np.ndarray) or isinstance(a, (list, tuple)):
         arr = np.ascontiguousarray(np.asarray(a, dtype=np.int64).astype(np.uint32))
         return _Arr(arr.ctypes.data if arr.size else None, arr, arr.size)
@@ -171,6 +186,9 @@ def _keys(a):
 def _floats(a, dtype_np=np.float32):
     if a is None:
         return _Arr(None, None, 0)
+    if _plain_tensor(a, 2):
+        n = a.numel()
+        return _Arr(a.data_ptr() if n else None, a, n)
     if isinstance(a, np.ndarray) or isinstance(a, (list, tuple)):
         arr = np.ascontiguousarray(np.asarray(a, dtype=dtype_np))
         return _Arr(arr.ctypes.data if arr.size else None, arr, arr.size)

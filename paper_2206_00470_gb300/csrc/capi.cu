@@ -16,6 +16,7 @@
 #include <new>
 #include <string>
 #include <tuple>
+#include <unordered_map>
 #include <vector>
 
 #include "adapm.h"
@@ -31,6 +32,63 @@ std::atomic<unsigned long long> g_launches{0};
 void adapm::note_launches(uint64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
 namespace {
+
+// Scratch blocks kept for reuse on one stream: a block given back is handed
+// out again to later work of the same stream, whose order makes that safe
+// (what other streams do with a block is waited for before it is given back).
+// Taking and giving back are host bookkeeping, where a pool allocation and
+// its free are two calls into the driver (0.7 to 1 us each, six pairs a push).
+// Sizes are rounded up to one of four steps per power of two.  Blocks above
+// kLargest are not kept, and not more than kKeep bytes in all; the rest goes
+// back to the pool, which the context owns and destroys.
+class BlockCache {
+ public:
+  cudaError_t take(cudaMemPool_t pool, cudaStream_t stream, size_t bytes, void** p) {
+    const size_t size = bytes <= kLargest ? round_up(bytes) : bytes;
+    auto it = size <= kLargest ? free_.find(size) : free_.end();
+    if (it != free_.end() && !it->second.empty()) {
+      *p = it->second.back();
+      it->second.pop_back();
+      kept_ -= size;
+      return cudaSuccess;
+    }
+    const cudaError_t e = cudaMallocFromPoolAsync(p, size, pool, stream);
+    if (e == cudaSuccess && size <= kLargest) size_[*p] = size;
+    return e;
+  }
+  // false: not a block of this cache (the caller frees it)
+  bool give(void* p, cudaStream_t stream) {
+    auto it = size_.find(p);
+    if (it == size_.end()) return false;
+    if (kept_ + it->second > kKeep) {
+      size_.erase(it);
+      cudaFreeAsync(p, stream);
+      return true;
+    }
+    kept_ += it->second;
+    free_[it->second].push_back(p);
+    return true;
+  }
+  void release() {   // the stream is idle
+    for (auto& f : free_)
+      for (void* p : f.second) cudaFree(p);
+    free_.clear();
+    size_.clear();
+    kept_ = 0;
+  }
+
+ private:
+  static constexpr size_t kLargest = 64u << 20, kKeep = 512u << 20;
+  static size_t round_up(size_t bytes) {
+    if (bytes <= 1024) return 1024;
+    size_t step = 256;
+    while (step * 8 < bytes) step <<= 1;   // four steps between 4 * step and 8 * step
+    return (bytes + step - 1) / step * step;
+  }
+  std::unordered_map<size_t, std::vector<void*>> free_;
+  std::unordered_map<void*, size_t> size_;
+  size_t kept_ = 0;
+};
 
 struct IntentList {
   uint32_t* keys = nullptr;   // device: cap distinct keys (no particular order), then the count word
@@ -86,6 +144,7 @@ struct adapm_ctx {
   int sms = kNumSms;
   int bits = 32;
   cudaMemPool_t pool = nullptr;
+  BlockCache blocks, plan_blocks;   // scratch of the library stream, of the plan stream
   Store s{};
   DevState* dstate = nullptr;
   std::vector<WorkerState> workers;
@@ -111,6 +170,7 @@ struct adapm_ctx {
   cudaStream_t copy_in = nullptr;
   cudaMemPool_t stage_pool = nullptr;
   cudaEvent_t staged = nullptr;
+  bool stage_wait = false;       // copies started that `stream` does not wait for yet
   std::deque<std::pair<cudaEvent_t, uint64_t>> stage_marks;
   std::vector<cudaEvent_t> spare_marks;
   uint64_t stage_unmarked = 0;   // bytes staged since the last mark
@@ -281,12 +341,11 @@ cudaError_t stage_mark(adapm_ctx* ctx, uint64_t next_bytes) {
 template <class T>
 cudaError_t pool_alloc(adapm_ctx* ctx, T** p, size_t count) {
   if (count == 0) count = 1;
-  return cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), count * sizeof(T), ctx->pool,
-                                 ctx->stream);
+  return ctx->blocks.take(ctx->pool, ctx->stream, count * sizeof(T), reinterpret_cast<void**>(p));
 }
 
 void pool_free(adapm_ctx* ctx, void* p) {
-  if (p) cudaFreeAsync(p, ctx->stream);
+  if (p && !ctx->blocks.give(p, ctx->stream)) cudaFreeAsync(p, ctx->stream);
 }
 
 // Device view of an input array; copies host arrays in.
@@ -316,8 +375,7 @@ cudaError_t stage_in(adapm_ctx* ctx, const T* p, size_t count, Input<T>* in) {
     if (e != cudaSuccess) return e;
     in->dev = in->owned;
     e = cudaMemcpyAsync(in->owned, p, bytes, cudaMemcpyHostToDevice, ctx->copy_in);
-    if (e == cudaSuccess) e = cudaEventRecord(ctx->staged, ctx->copy_in);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, ctx->staged, 0);
+    ctx->stage_wait = true;   // `stream` waits for the call's copies once (stage_join)
     ctx->stage_unmarked += bytes;
     ctx->stage_live += bytes;
     return e;   // the buffer is freed on `stream` after its consumer, like any pool buffer
@@ -326,6 +384,16 @@ cudaError_t stage_in(adapm_ctx* ctx, const T* p, size_t count, Input<T>* in) {
   if (e != cudaSuccess) return e;
   in->dev = in->owned;
   return cudaMemcpyAsync(in->owned, p, bytes, cudaMemcpyHostToDevice, ctx->stream);
+}
+
+// After a call's stage_in calls, before its kernels: `stream` waits for the
+// copies they started.
+cudaError_t stage_join(adapm_ctx* ctx) {
+  if (!ctx->stage_wait) return cudaSuccess;
+  ctx->stage_wait = false;
+  cudaError_t e = cudaEventRecord(ctx->staged, ctx->copy_in);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, ctx->staged, 0);
+  return e;
 }
 
 // Device buffer for an output array; copied out to host arrays at finish.
@@ -676,8 +744,8 @@ cudaError_t make_plan(adapm_ctx* ctx, IntentList& L, const uint32_t* keys, cudaE
   if ((e = cudaMemcpyAsync(L.px, keys, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, ps)) != cudaSuccess) return e;
   uint32_t *tk = nullptr, *tv = nullptr, *hist = nullptr, *tmp = nullptr;
   auto palloc = [&](uint32_t** p, size_t words) {
-    return cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), (words ? words : 1) * sizeof(uint32_t),
-                                   ctx->plan_pool, ps);
+    return ctx->plan_blocks.take(ctx->plan_pool, ps, (words ? words : 1) * sizeof(uint32_t),
+                                 reinterpret_cast<void**>(p));
   };
   if ((e = palloc(&tk, n)) != cudaSuccess || (e = palloc(&tv, n)) != cudaSuccess ||
       (e = palloc(&hist, sort_scratch_words(n))) != cudaSuccess ||
@@ -691,7 +759,8 @@ cudaError_t make_plan(adapm_ctx* ctx, IntentList& L, const uint32_t* keys, cudaE
                 nullptr, nullptr, 0, /*phased=*/true);
   if (e != cudaSuccess) return e;
   if (L.from_plan) compact_sorted_heads(L.psk, n, L.keys, L.count, tmp, ps);
-  for (uint32_t* p : {tk, tv, hist, tmp}) cudaFreeAsync(p, ps);
+  for (uint32_t* p : {tk, tv, hist, tmp})
+    if (!ctx->plan_blocks.give(p, ps)) cudaFreeAsync(p, ps);
   if ((e = take_ready_event(ctx, &L.ready)) != cudaSuccess) return e;
   if ((e = cudaEventRecord(L.ready, ps)) != cudaSuccess) return e;
   return cudaGetLastError();
@@ -883,6 +952,8 @@ adapm_status adapm_destroy(adapm_ctx* ctx) {
     if (kv.second.ready) cudaEventDestroy(kv.second.ready);
   }
   for (auto e : ctx->spare_ready) cudaEventDestroy(e);
+  ctx->blocks.release();
+  ctx->plan_blocks.release();
   Store& s = ctx->s;
   void* ptrs[] = {s.main, s.val, s.acc, s.map, s.rc, s.holders, s.slot_owner, s.free_stack,
                   s.stamp, s.own, s.dirty, ctx->dstate, ctx->early_counts};
@@ -931,13 +1002,14 @@ adapm_status adapm_intent(adapm_ctx* ctx, uint32_t worker, const uint32_t* keys,
   const bool plan = n > 0 && !ctx->cfg.no_push_plans &&
                     (ws.unused_plans < kPlanPatience || ws.intents % kPlanProbe == 0);
   ws.intents += 1;
-  CK(cudaMallocFromPoolAsync((void**)&L.keys, (n + 1) * sizeof(uint32_t), ctx->pool, ctx->stream));
+  CK(pool_alloc(ctx, &L.keys, n + 1));
   L.count = L.keys + n;
   if (n == 0) {
     CK(cudaMemsetAsync(L.count, 0, sizeof(uint32_t), ctx->stream));
   } else {
     Input<uint32_t> in;
     CK(stage_in(ctx, keys, n, &in));
+    CK(stage_join(ctx));
     if (plan) {
       CK(pool_alloc(ctx, &L.psk, n));
       CK(pool_alloc(ctx, &L.psp, n));
@@ -1044,6 +1116,7 @@ adapm_status adapm_pull(adapm_ctx* ctx, uint32_t worker, const uint32_t* keys, u
   ProfScope ps(ctx, 2);
   Input<uint32_t> in;
   CK(stage_in(ctx, keys, n, &in));
+  CK(stage_join(ctx));
   Output<float> o;
   CK(stage_out(ctx, out, n * ctx->s.D, &o));
   {
@@ -1070,6 +1143,7 @@ adapm_status adapm_push(adapm_ctx* ctx, uint32_t worker, const uint32_t* keys, u
   Input<float> id;
   CK(stage_in(ctx, keys, n, &ik));
   CK(stage_in(ctx, deltas, n * ctx->s.D, &id));
+  CK(stage_join(ctx));
   if (reinterpret_cast<uintptr_t>(id.dev) % 16 != 0) {
     // the push copies whole rows with the bulk-copy engine: 16-byte aligned rows
     float* aligned = nullptr;
@@ -1166,6 +1240,7 @@ adapm_status adapm_mf_step(adapm_ctx* ctx, uint32_t worker, const uint32_t* row_
   CK(stage_in(ctx, row_keys, n, &ir));
   CK(stage_in(ctx, col_keys, n, &ic));
   CK(stage_in(ctx, vals, n, &iv));
+  CK(stage_join(ctx));
   const uint64_t m = 2 * n;
   StepOut o{};
   o.loss_blocks = step_loss_blocks(ctx->sms);
@@ -1223,6 +1298,7 @@ adapm_status adapm_complex_step(adapm_ctx* ctx, uint32_t worker, const uint32_t*
   CK(stage_in(ctx, rels, n, &ir));
   CK(stage_in(ctx, tails, n, &it));
   CK(stage_in(ctx, neg_tails, n * n_neg, &ineg));
+  CK(stage_join(ctx));
   const uint64_t m = n * (3 + (uint64_t)n_neg);
   StepOut o{};
   o.loss_blocks = step_loss_blocks(ctx->sms);
@@ -1280,6 +1356,7 @@ adapm_status adapm_sgns_step(adapm_ctx* ctx, uint32_t worker, const uint32_t* ce
   CK(stage_in(ctx, centres, n, &ic));
   CK(stage_in(ctx, contexts, n * n_ctx, &ix));
   CK(stage_in(ctx, negatives, n * n_ctx * n_neg, &ineg));
+  CK(stage_join(ctx));
   const uint64_t m = n * per;
   StepOut o{};
   o.loss_blocks = step_loss_blocks(ctx->sms);
@@ -1349,6 +1426,7 @@ adapm_status adapm_replica_rows(adapm_ctx* ctx, uint32_t worker, const uint32_t*
   if (n == 0) return ADAPM_OK;
   Input<uint32_t> in;
   CK(stage_in(ctx, keys, n, &in));
+  CK(stage_join(ctx));
   Output<float> ov, oa;
   Output<uint8_t> oh;
   CK(stage_out(ctx, val_out, n * ctx->s.D, &ov));
@@ -1374,6 +1452,7 @@ adapm_status adapm_refcounts(adapm_ctx* ctx, uint32_t worker, const uint32_t* ke
   if (st != ADAPM_OK) return st;
   Input<uint32_t> in;
   CK(stage_in(ctx, keys, n, &in));
+  CK(stage_join(ctx));
   Output<uint32_t> o;
   CK(stage_out(ctx, out, n, &o));
   launch_refcounts(ctx->s, worker, in.dev, n, o.dev, ctx->stream);
@@ -1390,6 +1469,7 @@ adapm_status adapm_owners(adapm_ctx* ctx, const uint32_t* keys, uint64_t n, int3
   if (n == 0) return ADAPM_OK;
   Input<uint32_t> in;
   CK(stage_in(ctx, keys, n, &in));
+  CK(stage_join(ctx));
   Output<int32_t> o;
   CK(stage_out(ctx, out, n, &o));
   launch_owners(ctx->s, in.dev, n, o.dev, ctx->stream);
@@ -1406,6 +1486,7 @@ adapm_status adapm_read_main(adapm_ctx* ctx, const uint32_t* keys, uint64_t n, f
   if (n == 0) return ADAPM_OK;
   Input<uint32_t> in;
   CK(stage_in(ctx, keys, n, &in));
+  CK(stage_join(ctx));
   Output<float> o;
   CK(stage_out(ctx, out, n * ctx->s.D, &o));
   launch_pull(ctx->s, -1, in.dev, n, o.dev, ctx->sms, ctx->stream);
