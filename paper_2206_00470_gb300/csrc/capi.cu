@@ -102,6 +102,7 @@ struct IntentList {
   uint32_t* px = nullptr;     // the call's keys as given (what a matching push's keys equal)
   uint64_t n = 0;
   bool from_plan = false;
+  cudaEvent_t listed = nullptr;   // the distinct keys, when the early stream makes them
   bool plan_used = false;      // a push took this plan
   cudaEvent_t ready = nullptr;
   void* in_owned = nullptr;   // the call's staged copy of host keys, read by the plan stream
@@ -188,6 +189,7 @@ struct adapm_ctx {
   // advances).
   cudaStream_t early_stream = nullptr;
   AdvCounts* early_counts = nullptr;
+  cudaEvent_t early_dedup = nullptr;   // after the last intent_dedup on early_stream (they share the stamps)
   uint64_t early_advances = 0;   // advances that used their early events
   uint64_t early_undone = 0;     // early events taken back
   bool fake_launch_error = false;   // adapm_debug_fail_next_launch
@@ -459,6 +461,9 @@ adapm_status check_ctx(adapm_ctx* ctx) {
 }
 
 constexpr uint64_t kMaxN = 1ull << 31;
+// Keys of an intent that one block sorts (8 x 8000 keys per clock: 474 us so,
+// 441 us with the phased sort; 8 x 4000: 397 us, 519 us).
+constexpr uint64_t kSmallIntent = kSmallPlan;
 constexpr int kPlanPatience = 4;       // unused plans in a row after which a worker gets none ...
 constexpr uint64_t kPlanProbe = 16;    // ... but for one intent in this many
 
@@ -479,6 +484,20 @@ constexpr uint64_t kPlanProbe = 16;    // ... but for one intent in this many
 // ---------------------------------------------------------------------------
 bool early_enabled(const adapm_ctx* ctx) {
   return !ctx->cfg.no_early_events && ctx->s.own == nullptr && ctx->cfg.action_timing != ADAPM_ACT_ADAPTIVE;
+}
+
+cudaError_t ensure_early_stream(adapm_ctx* ctx) {
+  if (ctx->early_stream) return cudaSuccess;
+  cudaError_t e = cudaEventCreateWithFlags(&ctx->early_dedup, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->early_stream, cudaStreamNonBlocking);
+  return e;
+}
+
+// Where a list's distinct keys are made beside the library stream, the event
+// to wait for before they are used there.
+void add_list_wait(const IntentList& L, std::vector<cudaEvent_t>& waits) {
+  if (L.from_plan) waits.push_back(L.ready);
+  else if (L.listed) waits.push_back(L.listed);
 }
 
 // The lists of worker w's advance to clock c: opening ones, closing ones.
@@ -512,7 +531,7 @@ adapm_status early_make(adapm_ctx* ctx, uint32_t w) {
   E.clock = ws.clock + 1;
   advance_lists(ws, E.clock, E.open, E.close);
   if (E.open.empty() && E.close.empty()) return ADAPM_OK;
-  if (!ctx->early_stream) CK(cudaStreamCreateWithFlags(&ctx->early_stream, cudaStreamNonBlocking));
+  CK(ensure_early_stream(ctx));
   const std::vector<EventList> ev = event_lists(ctx, E.open, E.close);
   for (const auto& e : ev) E.cap += e.cap;
   CK(pool_alloc(ctx, &E.create_list, E.cap));
@@ -637,7 +656,7 @@ adapm_status push_device(adapm_ctx* ctx, uint32_t w, const uint32_t* dkeys, uint
   uint32_t seq = 0;
   if (plan) {
     plan->plan_used = true;
-    CK(cudaStreamWaitEvent(ctx->stream, plan->ready, 0));
+    if (plan->ready) CK(cudaStreamWaitEvent(ctx->stream, plan->ready, 0));   // (null: made on this stream)
     if (++ctx->plan_seq == 0) ctx->plan_seq = 1;
     seq = ctx->plan_seq;
     ctx->planned_pushes += 1;
@@ -717,7 +736,7 @@ adapm_status act_in_round(adapm_ctx* ctx) {
       for (int64_t id : it->second) {
         const IntentList& L = ctx->lists[id];
         ev.push_back(EventList{L.keys, L.count, L.cap, +1});
-        if (L.from_plan) waits.push_back(L.ready);
+        add_list_wait(L, waits);
       }
       it = ws.starts.erase(it);
     }
@@ -727,6 +746,21 @@ adapm_status act_in_round(adapm_ctx* ctx) {
     }
   }
   return ADAPM_OK;
+}
+
+// The sort of a small call's keys: its plan (if it gets one) and distinct keys.
+SmallSort small_plan(adapm_ctx* ctx, const IntentList& L, const uint32_t* keys) {
+  SmallSort a{};
+  a.raw = keys;
+  a.n = (uint32_t)L.n;
+  a.K = ctx->s.K;
+  a.keys_out = L.psk;
+  a.pos_out = L.psp;
+  a.copy_out = L.px;
+  a.heads_out = L.keys;
+  a.heads_count = L.count;
+  a.st = ctx->dstate;
+  return a;
 }
 
 // Sort an intent's keys with their positions on the plan stream (a phased
@@ -741,6 +775,11 @@ cudaError_t make_plan(adapm_ctx* ctx, IntentList& L, const uint32_t* keys, cudaE
   cudaStream_t ps = ctx->plan_stream;
   const uint64_t n = L.n;
   if ((e = cudaStreamWaitEvent(ps, after, 0)) != cudaSuccess) return e;
+  if (n <= kSmallIntent) {   // one launch for the sort, the copy of the keys and the distinct ones
+    if ((e = sort_small(small_plan(ctx, L, keys), ctx->bits, ps)) != cudaSuccess) return e;
+    if ((e = take_ready_event(ctx, &L.ready)) != cudaSuccess) return e;
+    return cudaEventRecord(L.ready, ps);
+  }
   if ((e = cudaMemcpyAsync(L.px, keys, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, ps)) != cudaSuccess) return e;
   uint32_t *tk = nullptr, *tv = nullptr, *hist = nullptr, *tmp = nullptr;
   auto palloc = [&](uint32_t** p, size_t words) {
@@ -778,6 +817,10 @@ cudaError_t close_list(adapm_ctx* ctx, uint32_t w, int64_t id) {
   if (L.ready) {
     e = cudaStreamWaitEvent(ctx->stream, L.ready, 0);
     ctx->spare_ready.push_back(L.ready);   // the wait has captured it; it can be recorded again
+  }
+  if (L.listed) {
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, L.listed, 0);
+    ctx->spare_ready.push_back(L.listed);
   }
   for (void* p : {(void*)L.keys, (void*)L.psk, (void*)L.psp, (void*)L.px, L.in_owned}) pool_free(ctx, p);
   auto& order = ctx->workers[w].order;
@@ -950,6 +993,7 @@ adapm_status adapm_destroy(adapm_ctx* ctx) {
                     kv.second.in_owned})
       if (p) cudaFree(p);
     if (kv.second.ready) cudaEventDestroy(kv.second.ready);
+    if (kv.second.listed) cudaEventDestroy(kv.second.listed);
   }
   for (auto e : ctx->spare_ready) cudaEventDestroy(e);
   ctx->blocks.release();
@@ -971,6 +1015,7 @@ adapm_status adapm_destroy(adapm_ctx* ctx) {
   if (ctx->copy_in) cudaStreamDestroy(ctx->copy_in);
   if (ctx->stage_pool) cudaMemPoolDestroy(ctx->stage_pool);
   if (ctx->plan_stream) cudaStreamDestroy(ctx->plan_stream);
+  if (ctx->early_dedup) cudaEventDestroy(ctx->early_dedup);
   if (ctx->early_stream) cudaStreamDestroy(ctx->early_stream);
   if (ctx->plan_pool) cudaMemPoolDestroy(ctx->plan_pool);
   if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
@@ -1015,26 +1060,56 @@ adapm_status adapm_intent(adapm_ctx* ctx, uint32_t worker, const uint32_t* keys,
       CK(pool_alloc(ctx, &L.psp, n));
       CK(pool_alloc(ctx, &L.px, n));
     }
-    // a window that opens two or more clocks ahead takes its distinct keys
-    // from the plan; one that opens at the next advance (or is active now)
-    // would wait there for the plan, so its keys come from the hash-set pass
-    // here, and the plan only serves the push a clock later
-    L.from_plan = plan && clock_start > ws.clock + 1;
-    if (!L.from_plan) {
+    // Where the distinct keys come from.  A window that opens two or more
+    // clocks ahead: the plan.  One that opens at the next advance would wait
+    // there for the plan's sort, so its keys come from the hash-set pass, on
+    // the early stream where the advance's events follow it (8 x 16,384 keys
+    // per clock 561 -> 465 us, 8 x 131,072 1072 -> 992 us, 8 x 2^20 2983 -> 2957
+    // us), or here when there are no early events.  Up to kSmallIntent keys,
+    // whose sort is one short launch, always come from that: on the plan
+    // stream, or here without a plan or when the window is active now.
+    const bool small = n <= kSmallIntent;
+    L.from_plan = plan && !now && (small || clock_start > ws.clock + 1);
+    const bool early = !small && !L.from_plan && !now && early_enabled(ctx);
+    if (L.from_plan) {
+    } else if (small) {
+      CK(sort_small(small_plan(ctx, L, in.dev), ctx->bits, ctx->stream));
+    } else {
+      if (early) CK(ensure_early_stream(ctx));
+      // (the stamps have one user at a time: a pass here waits for the last one there)
+      if (!early && ctx->early_stream) CK(cudaStreamWaitEvent(ctx->stream, ctx->early_dedup, 0));
       if (++ctx->intent_tag == 0) {   // tags wrapped: clear the stamps
+        if (ctx->early_stream) CK(cudaStreamWaitEvent(ctx->stream, ctx->early_dedup, 0));
         CK(cudaMemsetAsync(ctx->s.stamp, 0, ctx->s.K * 4, ctx->stream));
         ctx->intent_tag = 1;
       }
-      CK(cudaMemsetAsync(L.count, 0, sizeof(uint32_t), ctx->stream));
-      launch_intent_dedup(ctx->s, in.dev, n, ctx->intent_tag, L.keys, L.count, ctx->sms, ctx->stream);
+      cudaStream_t on = ctx->stream;
+      if (early) {
+        on = ctx->early_stream;
+        cudaEvent_t after = nullptr;
+        CK(take_ready_event(ctx, &after));
+        CK(cudaEventRecord(after, ctx->stream));
+        CK(cudaStreamWaitEvent(on, after, 0));
+        ctx->spare_ready.push_back(after);   // the wait has captured it
+      }
+      CK(cudaMemsetAsync(L.count, 0, sizeof(uint32_t), on));
+      launch_intent_dedup(ctx->s, in.dev, n, ctx->intent_tag, L.keys, L.count, ctx->sms, on);
+      if (early) {
+        CK(cudaEventRecord(ctx->early_dedup, on));
+        CK(take_ready_event(ctx, &L.listed));
+        CK(cudaEventRecord(L.listed, on));
+      }
     }
-    if (plan) {
+    const bool planned_here = plan && small && !L.from_plan;   // the plan was made on this stream
+    if (plan && !planned_here) {
       cudaEvent_t after = nullptr;
       CK(take_ready_event(ctx, &after));
       CK(cudaEventRecord(after, ctx->stream));
       CK(make_plan(ctx, L, in.dev, after));
       ctx->spare_ready.push_back(after);   // the plan stream's wait has captured it
       L.in_owned = in.owned;               // freed when the list closes, after the plan
+    } else if (early) {
+      L.in_owned = in.owned;               // freed when the list closes
     } else {
       pool_free(ctx, in.owned);
     }
@@ -1084,7 +1159,7 @@ adapm_status adapm_advance_clock(adapm_ctx* ctx, uint32_t worker) {
     for (int64_t id : it->second) {
       const IntentList& L = ctx->lists[id];
       ev.push_back(EventList{L.keys, L.count, L.cap, +1});
-      if (L.from_plan) waits.push_back(L.ready);
+      add_list_wait(L, waits);
     }
     ws.starts.erase(it);
   }

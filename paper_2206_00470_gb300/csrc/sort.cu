@@ -27,6 +27,7 @@
 // ERR_TIMEOUT and the kernel returns, and since all later barriers need
 // every block, the whole launch stops within one bounded wait.
 #include "internal.cuh"
+#include "radix.cuh"
 
 namespace adapm {
 
@@ -37,8 +38,6 @@ constexpr int kWarps = kSortThreads / 32;
 constexpr int kItems = 8;                          // keys per thread per sub-tile (largest)
 constexpr int kSub = kSortThreads * kItems;        // 2048 keys per sub-tile (largest)
 constexpr int kSubMin = kSortThreads * 4;          // sub-tile of small batches (4 keys per thread)
-constexpr int kRadixBits = 9;
-constexpr int kDigits = 1 << kRadixBits;           // 512
 constexpr int kDPT = kDigits / kSortThreads;       // digits per thread (2)
 constexpr uint32_t kMaxSortBlocks = 4096;
 constexpr uint32_t kSpinLimit = 1u << 21;          // polls of one barrier wait
@@ -48,72 +47,10 @@ constexpr int kScanQ = 5;                          // digit-row entries per lane
 constexpr int kCompactItems = 8;                   // compaction: keys per thread
 constexpr int kTile = kSortThreads * kCompactItems;
 
-__device__ __forceinline__ uint32_t lanemask_lt() {
-  uint32_t m;
-  asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
-  return m;
-}
-
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
-}
-
-// Lanes of the warp whose `valid` flag and low `nbits` digit bits equal this
-// lane's (one ballot per bit: a warp-level multi-split).
-__device__ __forceinline__ uint32_t digit_peers(uint32_t d, bool valid, int nbits) {
-  const uint32_t v = __ballot_sync(0xFFFFFFFFu, valid);
-  uint32_t peers = valid ? v : ~v;
-  for (int b = 0; b < nbits; ++b) {
-    const bool bit = (d >> b) & 1u;
-    const uint32_t bal = __ballot_sync(0xFFFFFFFFu, bit);
-    peers &= bit ? bal : ~bal;
-  }
-  return peers;
-}
-
-// Exclusive scan of one value per thread over a block of NT threads.
-template <int NT>
-__device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* total,
-                                                         uint32_t* sm /* NT/32 words */) {
-  const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  uint32_t x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) sm[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    uint32_t s = lane < NT / 32 ? sm[lane] : 0u;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, s, o);
-      if (lane >= o) s += y;
-    }
-    if (lane < NT / 32) sm[lane] = s;
-  }
-  __syncthreads();
-  const uint32_t before = warp > 0 ? sm[warp - 1] : 0u;
-  *total = sm[NT / 32 - 1];
-  __syncthreads();
-  return before + x - v;
-}
-
-struct PassPlan {
-  int passes;
-  int per;
-};
-
-PassPlan plan_for(int bits) {
-  PassPlan p;
-  p.passes = (bits + kRadixBits - 1) / kRadixBits;
-  if (p.passes < 1) p.passes = 1;
-  p.per = (bits + p.passes - 1) / p.passes;
-  return p;
 }
 
 struct SortArgs {
@@ -736,6 +673,25 @@ cudaError_t sort_keys(const uint32_t* raw, uint64_t n, uint64_t K, bool allow_no
                       cudaStream_t stream, uint32_t** keys_out, uint32_t** pos_out, const uint32_t* plan_keys,
                       uint32_t* plan_word, uint32_t plan_seq, bool phased) {
   const PassPlan pl = plan_for(bits);
+  // (a context whose next grid barrier was made to fail sorts with one)
+  if (n <= (plan_keys ? kSmallPlan : kSmallSort) && va && !phased && n > 0 && (*bar_base >> 40) == 0) {
+    if (keys_out) *keys_out = ka;
+    if (pos_out) *pos_out = va;
+    SmallSort a{};
+    a.raw = raw;
+    a.n = (uint32_t)n;
+    a.K = K;
+    a.allow_nokey = allow_nokey;
+    a.keys_out = ka;
+    a.pos_out = va;
+    a.st = st;
+    a.clear0 = clear0;
+    a.clear1 = clear1;
+    a.plan_keys = plan_keys && plan_word ? plan_keys : nullptr;
+    a.plan_word = plan_word;
+    a.plan_seq = plan_seq;
+    return sort_small(a, bits, stream);
+  }
   if (keys_out) *keys_out = pl.passes % 2 ? ka : kb;
   if (pos_out) *pos_out = va ? (pl.passes % 2 ? va : vb) : nullptr;
   if (n == 0) return cudaSuccess;
