@@ -353,14 +353,14 @@ __global__ void events_kernel(Store s, uint32_t w, EventBatch eb, uint32_t* out_
 // settles the advance.
 constexpr uint32_t kMany = 3u;   // a holder mask that counts as neither no holder nor one
 
-constexpr int evict_blocks_per_sm(int C) { return C >= 8 ? 2 : (C == 4 ? 3 : 4); }
+constexpr int evict_blocks_per_sm(int C) { return C >= 8 ? 2 : (C >= 3 ? 3 : 4); }
 
 template <int G, int C>
 __global__ void __launch_bounds__(kThreads, evict_blocks_per_sm(C)) evict_create_kernel(Store s, uint32_t w,
                                                                               const uint32_t* __restrict__ evict_list,
                                                                               const uint32_t* __restrict__ create_list,
                                                                               AdvCounts* early) {
-  constexpr int R = C == 4 ? 2 : (4 / C > 0 ? 4 / C : 1);
+  constexpr int R = C == 3 || C == 4 ? 2 : (4 / C > 0 ? 4 / C : 1);
   constexpr uint32_t GW = 32 / G;   // row groups per warp
   __shared__ uint2 moves[kThreads / 32][32];    // (slot, key): pending rows to add to main
   __shared__ uint2 copies[kThreads / 32][32];   // (slot, key): main rows to copy to val first

@@ -1063,14 +1063,14 @@ adapm_status adapm_intent(adapm_ctx* ctx, uint32_t worker, const uint32_t* keys,
     // Where the distinct keys come from.  A window that opens two or more
     // clocks ahead: the plan.  One that opens at the next advance would wait
     // there for the plan's sort, so its keys come from the hash-set pass, on
-    // the early stream where the advance's events follow it (8 x 16,384 keys
+    // the early stream, where early events follow it (8 x 16,384 keys
     // per clock 561 -> 465 us, 8 x 131,072 1072 -> 992 us, 8 x 2^20 2983 -> 2957
-    // us), or here when there are no early events.  Up to kSmallIntent keys,
+    // us); active now, here.  Up to kSmallIntent keys,
     // whose sort is one short launch, always come from that: on the plan
     // stream, or here without a plan or when the window is active now.
     const bool small = n <= kSmallIntent;
     L.from_plan = plan && !now && (small || clock_start > ws.clock + 1);
-    const bool early = !small && !L.from_plan && !now && early_enabled(ctx);
+    const bool early = !small && !L.from_plan && !now;
     if (L.from_plan) {
     } else if (small) {
       CK(sort_small(small_plan(ctx, L, in.dev), ctx->bits, ctx->stream));

@@ -4,16 +4,21 @@
 namespace adapm {
 
 uint64_t push_chunk_rows(uint32_t D, uint64_t n, int sms) {
-  // one span per resident block where the span fits in shared memory: rows
-  // per group = n / (groups per block x resident blocks), in [8, kPushSpan / groups]
+  // one span per resident block where the span fits in shared memory, else
+  // as few full waves of resident blocks as do: rows per group = n / (groups
+  // per block x resident blocks x waves), in [8, kPushSpan / groups].  (Spans
+  // of kPushSpan rows whatever the last wave holds: 696 blocks on 456 places
+  // at 2.1M rows of 300 floats, 475 us against 410 us for 912.)
   uint64_t ch = 0;
   dispatch_push_gc(D / 4, false, [&](auto Gc, auto Cc) {
     constexpr int G = decltype(Gc)::value, C = decltype(Cc)::value;
     constexpr uint64_t NG = kThreads / G;
     const uint64_t groups = NG * (uint64_t)sms * push_blocks_per_sm(C);
-    ch = (n + groups - 1) / groups;
+    const uint64_t most = kPushSpan / NG;
+    const uint64_t waves = (n + groups * most - 1) / (groups * most);
+    ch = waves ? (n + groups * waves - 1) / (groups * waves) : 8;
     if (ch < 8) ch = 8;
-    if (ch > kPushSpan / NG) ch = kPushSpan / NG;
+    if (ch > most) ch = most;
   });
   return ch;
 }

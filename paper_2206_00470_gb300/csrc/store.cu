@@ -19,8 +19,14 @@ namespace {
 // R rows per group and round, software-pipelined so that one round issues
 // the row loads of round i, the slot lookups of round i+1 and the key loads
 // of round i+2 together: one memory latency per round instead of three.
+// With one float4 of a row per lane, four rows per group at five blocks per SM
+// do better than eight at three (rows of 64 floats: 9 x 2^18 rows 430 -> 397
+// us, 9 x 131,072 291 -> 250 us); wider rows want the bytes in flight (8 float4
+// per lane; rows of 200 floats 538 us, with half of that 556 us).
+constexpr int pull_rows(int C) { return C == 1 ? 4 : (8 / C > 0 ? 8 / C : 1); }
+
 template <int G, int C, int R>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, C == 1 ? 5 : 1)
 pull_kernel(Store s, int w, const uint32_t* __restrict__ keys, uint64_t n, float* __restrict__ out) {
   const int lane = threadIdx.x & (G - 1);
   const uint64_t g = group_id<G>(), ng = group_count<G>();
@@ -445,7 +451,7 @@ void launch_pull(const Store& s, int w, const uint32_t* keys, uint64_t n, float*
   if (n == 0) return;
   dispatch_gc(s.D / 4, [&](auto Gc, auto Cc) {
     constexpr int G = decltype(Gc)::value, C = decltype(Cc)::value;
-    constexpr int R = 8 / C > 0 ? 8 / C : 1;
+    constexpr int R = pull_rows(C);
     note_launches(1);
     pull_kernel<G, C, R><<<grid_for((n + R - 1) / R, G, sms), kThreads, 0, stream>>>(s, w, keys, n, out);
   });
