@@ -28,28 +28,32 @@ namespace adapm {
 
 namespace {
 
-// What a push kernel needs to know before its first row, loaded together (one
-// memory latency, not one per word).  False: an earlier sort gave up, nothing
-// may be touched.  The sorted keys and positions in `a` are the plan's, unless
-// its check stored a mismatch for this push (then the sort made instead).
-// any_replica: there are replicas that may be aliases of a main row.
-__device__ __forceinline__ bool push_begin(Store& s, PushArgs& a, bool& any_replica) {
+// What a push kernel needs to know before its first row: loaded together and
+// first, used only once the loads that do not depend on it are under way.
+struct PushWords {
+  uint32_t errors, miss, live, par;
+};
+__device__ __forceinline__ PushWords push_words(const Store& s, const PushArgs& a) {
   auto ld = [](const void* p) {
     uint32_t v;
     asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
   };
-  const uint32_t errors = ld(&s.st->errors);
-  const uint32_t miss = ld(a.plan_seq != 0u ? a.plan_word : &s.st->plan_miss);
-  const uint32_t live = ld(&s.st->live);
-  s.par = ld(&s.st->par);
-  if (errors & ERR_TIMEOUT) return false;
-  if (a.plan_seq != 0u && miss == a.plan_seq) {
-    a.skeys = a.alt_keys;
-    a.spos = a.alt_pos;
-  }
-  any_replica = s.own == nullptr && (int32_t)live > 0;
-  return true;
+  return PushWords{ld(&s.st->errors), ld(a.plan_seq != 0u ? a.plan_word : &s.st->plan_miss), ld(&s.st->live),
+                   ld(&s.st->par)};
+}
+// 0: an earlier sort gave up, nothing may be touched; 1: the sorted keys and
+// positions are those in `a` (the plan's); 2: they are the sort's, which `a`
+// now names (the plan's check stored a mismatch for this push).
+// any_replica: there are replicas that may be aliases of a main row.
+__device__ __forceinline__ int push_resolve(Store& s, PushArgs& a, const PushWords& pw, bool& any_replica) {
+  any_replica = s.own == nullptr && (int32_t)pw.live > 0;
+  s.par = pw.par;
+  if (pw.errors & ERR_TIMEOUT) return 0;
+  if (a.plan_seq == 0u || pw.miss != a.plan_seq) return 1;
+  a.skeys = a.alt_keys;
+  a.spos = a.alt_pos;
+  return 2;
 }
 
 // ---------------------------------------------------------------------------
@@ -212,8 +216,8 @@ __device__ __forceinline__ uint32_t factor_row(const PushArgs& a, uint32_t pos) 
 // same ones of the accumulator half, so a gradient is loaded once for both.
 template <int G, int C, int R, int SRC>
 __global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_kernel(Store s, PushArgs a) {
-  bool any_replica;
-  if (!push_begin(s, a, any_replica)) return;
+  const PushWords pw = push_words(s, a);
+  bool any_replica = false, resolved = false;
   constexpr int NG = kThreads / G;
   const uint32_t CH = (uint32_t)a.chunk;            // rows per group, NG * CH <= kPushSpan
   const uint32_t span = NG * CH;
@@ -250,60 +254,96 @@ __global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_k
     const uint32_t len = (uint32_t)(a.n - P0 < (uint64_t)span ? a.n - P0 : span);
     __syncthreads();
     if (threadIdx.x == 0) ncopy = 0;
-    for (uint32_t i = threadIdx.x; i < len; i += kThreads) {
-      sk[1 + i] = a.skeys[P0 + i];
-      sp[i] = a.spos[P0 + i];
-    }
-    if (threadIdx.x == 0) {
-      sk[0] = P0 > 0 ? a.skeys[P0 - 1] : kNoKey;
-      sk[1 + len] = P0 + len < a.n ? a.skeys[P0 + len] : kNoKey;
+    auto stage = [&]() {
+      for (uint32_t i = threadIdx.x; i < len; i += kThreads) {
+        sk[1 + i] = a.skeys[P0 + i];
+        sp[i] = a.spos[P0 + i];
+      }
+      if (threadIdx.x == 0) {
+        sk[0] = P0 > 0 ? a.skeys[P0 - 1] : kNoKey;
+        sk[1 + len] = P0 + len < a.n ? a.skeys[P0 + len] : kNoKey;
+      }
+    };
+    stage();
+    if (!resolved) {   // (uniform over the grid)
+      resolved = true;
+      const int from = push_resolve(s, a, pw, any_replica);
+      if (from == 0) return;
+      if (from == 2) {
+        __syncthreads();
+        stage();
+      }
     }
     __syncthreads();
-    // per-row control, one thread per row, and the slot of every whole segment
-    for (uint32_t i = threadIdx.x; i < len; i += kThreads) {
-      const uint32_t k = sk[1 + i];
-      uint8_t f = 0;
-      int32_t slot = -2;
-      // (sorted keys are valid or the skip sentinel; anything else out of
-      // range, like a position outside the batch, is an internal error)
-      if (k < s.K && sp[i] < a.n) {
-        const uint32_t cs = i - i % CH;                          // first row of the chunk
-        const uint32_t ce = cs + CH < len ? cs + CH : len;        // end of the chunk
-        const bool seg_begin = (P0 + i == 0) || sk[i] != k;       // sk[i] is the key of row i-1
-        const bool seg_end = (P0 + i + 1 >= a.n) || sk[1 + i + 1] != k;
-        const bool started = (P0 + cs == 0) || sk[cs] != k;       // piece began inside the chunk
-        const bool piece_end = seg_end || i + 1 == ce;
-        f = (piece_end ? 1 : 0) | (started ? 2 : 0) | (seg_end ? 4 : 0) |
-            ((seg_begin || i == cs) ? 8 : 0) | 16;
-        if (seg_begin) ++heads;
-        if (SRC == kSrcAda && (f & 8) && (f & 7) != 7) {
-          // the accumulators of a piece's first row: where this worker's value of the key is
-          const Target t = look_target(s, a.worker, k, false);
-          slot = t.slot;
-          f |= (uint8_t)(t.state << 5);
-        }
-        if ((f & 7) == 7) {
-          const Target t = look_target(s, a.worker, k, any_replica);
-          if (SRC != kSrcAda) mark_target(s, a.worker, k, t);
-          slot = t.slot;
-          f |= (uint8_t)(t.state << 5);
-          // a main row that others replicate: its (key, holder) pairs are
-          // listed for the block (as far as the list goes)
-          if (t.holders) {
-            uint32_t at = atomicAdd(&ncopy, (uint32_t)__popc(t.holders));
-            for (uint32_t h = t.holders; h; h &= h - 1, ++at) {
-              if (at < kPushCopies) copies[at] = make_uint2(k, (uint32_t)(__ffs(h) - 1));
-              else f |= 128;
-            }
-          }
+    // per-row control, one thread per row, and the target of every whole
+    // segment; SU rows per thread and round, whose random accesses (map
+    // entries, then states or holder masks) go out together (one row after
+    // the other, nine rows per thread at 2^20 rows cost a tenth of the kernel)
+    constexpr int SU = C >= 3 ? 2 : 4;
+    for (uint32_t i0 = threadIdx.x; i0 < len; i0 += SU * kThreads) {
+      uint32_t key[SU];
+      uint8_t f[SU];
+      int32_t e[SU];
+      float coef[SU];
+#pragma unroll
+      for (int u = 0; u < SU; ++u) {
+        const uint32_t i = i0 + u * kThreads;
+        key[u] = kNoKey;
+        f[u] = 0;
+        e[u] = -1;
+        coef[u] = 0.f;
+        if (i >= len) continue;
+        const uint32_t k = sk[1 + i];
+        key[u] = k;
+        // (sorted keys are valid or the skip sentinel; anything else out of
+        // range, like a position outside the batch, is an internal error)
+        if (k < s.K && sp[i] < a.n) {
+          const uint32_t cs = i - i % CH;                          // first row of the chunk
+          const uint32_t ce = cs + CH < len ? cs + CH : len;        // end of the chunk
+          const bool seg_begin = (P0 + i == 0) || sk[i] != k;       // sk[i] is the key of row i-1
+          const bool seg_end = (P0 + i + 1 >= a.n) || sk[1 + i + 1] != k;
+          const bool started = (P0 + cs == 0) || sk[cs] != k;       // piece began inside the chunk
+          const bool piece_end = seg_end || i + 1 == ce;
+          f[u] = (piece_end ? 1 : 0) | (started ? 2 : 0) | (seg_end ? 4 : 0) |
+                 ((seg_begin || i == cs) ? 8 : 0) | 16;
+          if (seg_begin) ++heads;
+          // (AdaGrad sources: also where the accumulators of a piece's first row are)
+          if ((f[u] & 7) == 7 || (SRC == kSrcAda && (f[u] & 8))) e[u] = s.map[(uint64_t)a.worker * s.K + k];
+          if (SRC != kSrcRows) coef[u] = __ldg(a.coef + sp[i]);
+        } else if (k != kNoKey || sp[i] >= a.n) {
+          set_error(s.st, ERR_INTERNAL);
         }
       }
-      else if (k != kNoKey || sp[i] >= a.n) set_error(s.st, ERR_INTERNAL);
-      sf[i] = f;
-      ss[i] = slot;
-      if (SRC != kSrcRows) {
-        sc[i] = (f & 16) ? __ldg(a.coef + sp[i]) : 0.f;
-        sp[i] = (f & 16) ? factor_row(a, sp[i]) : 0u;
+      uint32_t state[SU], holders[SU];
+#pragma unroll
+      for (int u = 0; u < SU; ++u) {
+        const bool whole = (f[u] & 7) == 7;
+        state[u] = map_none(e[u]) ? REP_ALIAS : rep_state(s, e[u]);
+        holders[u] = whole && map_none(e[u]) && any_replica ? s.holders[key[u]] : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < SU; ++u) {
+        const uint32_t i = i0 + u * kThreads;
+        if (i >= len) continue;
+        const Target t{map_none(e[u]) ? -1 : map_slot(e[u]), state[u], holders[u]};
+        const bool whole = (f[u] & 7) == 7;
+        if (whole && SRC != kSrcAda) mark_target(s, a.worker, key[u], t);
+        f[u] |= (uint8_t)(state[u] << 5);
+        // a main row that others replicate: its (key, holder) pairs are
+        // listed for the block (as far as the list goes)
+        if (t.holders) {
+          uint32_t at = atomicAdd(&ncopy, (uint32_t)__popc(t.holders));
+          for (uint32_t h = t.holders; h; h &= h - 1, ++at) {
+            if (at < kPushCopies) copies[at] = make_uint2(key[u], (uint32_t)(__ffs(h) - 1));
+            else f[u] |= 128;
+          }
+        }
+        sf[i] = f[u];
+        ss[i] = whole || (SRC == kSrcAda && (f[u] & 8)) ? t.slot : -2;
+        if (SRC != kSrcRows) {
+          sc[i] = coef[u];
+          sp[i] = (f[u] & 16) ? factor_row(a, sp[i]) : 0u;
+        }
       }
     }
     __syncthreads();
@@ -529,8 +569,8 @@ __global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_k
 template <int G, int C>
 __global__ void __launch_bounds__(kThreads) push_combine_kernel(Store s, PushArgs a, uint64_t span,
                                                                 uint64_t nspans) {
-  bool any_replica;
-  if (!push_begin(s, a, any_replica)) return;
+  const PushWords pw = push_words(s, a);
+  bool any_replica = false, resolved = false;
   constexpr int NG = kThreads / G;
   __shared__ float4 part[NG][G * C];
   const int lane = threadIdx.x & (G - 1);
@@ -541,16 +581,34 @@ __global__ void __launch_bounds__(kThreads) push_combine_kernel(Store s, PushArg
   for (uint64_t b = blockIdx.x; b < nspans; b += gridDim.x) {   // block-uniform
     const uint64_t st = b * span;
     const uint64_t en = st + span < a.n ? st + span : a.n;
-    const uint32_t kl = a.skeys[en - 1];
-    if (en >= a.n || kl >= s.K || a.skeys[en] != kl) continue;
-    if (st > 0 && a.skeys[st - 1] == kl) continue;             // it began in an earlier span
+    // the keys around the span's end and before its start, and the first keys
+    // of the spans after it, in one latency
+    uint32_t kl, kn, kb, kf;
+    auto look = [&]() {
+      kl = a.skeys[en - 1];
+      kn = en < a.n ? a.skeys[en] : kNoKey;
+      kb = st > 0 ? a.skeys[st - 1] : kNoKey;
+      kf = b + 1 + threadIdx.x < nspans ? a.skeys[(b + 1 + threadIdx.x) * span] : kNoKey;
+    };
+    look();
+    if (!resolved) {   // (uniform over the grid)
+      resolved = true;
+      const int from = push_resolve(s, a, pw, any_replica);
+      if (from == 0) return;
+      if (from == 2) look();
+    }
+    if (kl >= s.K || kn != kl) continue;
+    if (st > 0 && kb == kl) continue;             // it began in an earlier span
+    Target target{-1, REP_ALIAS, 0u};
+    if (threadIdx.x == 0) target = look_target(s, a.worker, kl, any_replica);
     // the last span whose first row holds kl: the spans after b that do form
     // a prefix (the keys are sorted), so the block tests kThreads of them at
     // once and counts
     uint64_t lo = b;
     for (uint64_t m0 = b + 1; m0 < nspans; m0 += kThreads) {   // block-uniform
       const uint64_t m = m0 + threadIdx.x;
-      const int cnt = __syncthreads_count(m < nspans && a.skeys[m * span] == kl);
+      if (m0 > b + 1) kf = m < nspans ? a.skeys[m * span] : kNoKey;
+      const int cnt = __syncthreads_count(m < nspans && kf == kl);
       lo += (uint64_t)cnt;
       if (cnt < kThreads) break;
     }
@@ -584,7 +642,11 @@ __global__ void __launch_bounds__(kThreads) push_combine_kernel(Store s, PushArg
         tot[c] = col < D4 ? __ldcg(sp4 + (2 * b + 1) * D4 + col) : f4zero();
         for (int g2 = 0; g2 < NG; ++g2) tot[c] = f4add(tot[c], part[g2][lane + c * G]);
       }
-      take_and_apply<G, C, kSrcRows>(s, a.worker, kl, tot, lane, gmask, any_replica);
+      if (lane == 0) mark_target(s, a.worker, kl, target);
+      target.slot = __shfl_sync(gmask, target.slot, 0, G);
+      target.state = __shfl_sync(gmask, target.state, 0, G);
+      target.holders = __shfl_sync(gmask, target.holders, 0, G);
+      apply_sum<G, C, kSrcRows>(s, kl, target, tot, lane, gmask);
     }
     __syncthreads();
   }
