@@ -780,25 +780,23 @@ cudaError_t make_plan(adapm_ctx* ctx, IntentList& L, const uint32_t* keys, cudaE
     if ((e = take_ready_event(ctx, &L.ready)) != cudaSuccess) return e;
     return cudaEventRecord(L.ready, ps);
   }
-  if ((e = cudaMemcpyAsync(L.px, keys, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, ps)) != cudaSuccess) return e;
-  uint32_t *tk = nullptr, *tv = nullptr, *hist = nullptr, *tmp = nullptr;
+  uint32_t *tk = nullptr, *tv = nullptr, *hist = nullptr;
   auto palloc = [&](uint32_t** p, size_t words) {
     return ctx->plan_blocks.take(ctx->plan_pool, ps, (words ? words : 1) * sizeof(uint32_t),
                                  reinterpret_cast<void**>(p));
   };
   if ((e = palloc(&tk, n)) != cudaSuccess || (e = palloc(&tv, n)) != cudaSuccess ||
-      (e = palloc(&hist, sort_scratch_words(n))) != cudaSuccess ||
-      (e = palloc(&tmp, compact_tmp_words(n))) != cudaSuccess)
+      (e = palloc(&hist, plan_scratch_words(n, ctx->bits))) != cudaSuccess)
     return e;
   const bool odd = sort_passes(ctx->bits) % 2 == 1;   // the sort ends in ka / va after odd passes
   unsigned long long no_barriers = 0;
   uint32_t *sk = nullptr, *sp = nullptr;
   e = sort_keys(keys, n, ctx->s.K, false, ctx->bits, odd ? L.psk : tk, odd ? tk : L.psk, odd ? L.psp : tv,
-                odd ? tv : L.psp, hist, ctx->sms, ctx->dstate, &no_barriers, nullptr, nullptr, ps, &sk, &sp,
-                nullptr, nullptr, 0, /*phased=*/true);
+                odd ? tv : L.psp, hist, ctx->sms, ctx->dstate, &no_barriers, L.from_plan ? L.count : nullptr, nullptr,
+                ps, &sk, &sp, nullptr, nullptr, 0, /*phased=*/true, L.px);
   if (e != cudaSuccess) return e;
-  if (L.from_plan) compact_sorted_heads(L.psk, n, L.keys, L.count, tmp, ps);
-  for (uint32_t* p : {tk, tv, hist, tmp})
+  if (L.from_plan) list_sorted_heads(L.psk, n, L.keys, L.count, ps);   // (the sort zeroed the count)
+  for (uint32_t* p : {tk, tv, hist})
     if (!ctx->plan_blocks.give(p, ps)) cudaFreeAsync(p, ps);
   if ((e = take_ready_event(ctx, &L.ready)) != cudaSuccess) return e;
   if ((e = cudaEventRecord(L.ready, ps)) != cudaSuccess) return e;

@@ -248,18 +248,22 @@ __device__ __forceinline__ bool sort_failed(const DevState* st) {
 // otherwise its blocks account their remaining barriers and return, leaving
 // ka/kb/va/vb as they are (the plan holds the result).  Out-of-range keys
 // are reported by the check as the sort would.
-// phased = true runs the sort as 1 + 2 * passes ordinary launches (kernel
-// boundaries instead of grid barriers, *bar_base untouched): for a stream
-// that runs beside other work, where a cooperative launch would wait for
-// the whole GPU.
+// phased = true runs the sort as ordinary launches (kernel boundaries instead
+// of grid barriers, *bar_base untouched): for a stream that runs beside other
+// work, where a cooperative launch would wait for the whole GPU.  One for the
+// count and two per pass, or one per pass when the blocks are few enough that
+// each scans the digit table itself.  `scratch` then holds
+// plan_scratch_words(n, bits) words, and copy_out (may be null) receives the
+// keys as given.
 size_t sort_scratch_words(uint64_t n);
+size_t plan_scratch_words(uint64_t n, int bits);
 int sort_passes(int bits);
 cudaError_t sort_keys(const uint32_t* raw, uint64_t n, uint64_t K, bool allow_nokey, int bits,
                       uint32_t* ka, uint32_t* kb, uint32_t* va, uint32_t* vb, uint32_t* scratch, int sms,
                       DevState* st, unsigned long long* bar_base, uint32_t* clear0, uint32_t* clear1,
                       cudaStream_t stream, uint32_t** keys_out, uint32_t** pos_out,
                       const uint32_t* plan_keys = nullptr, uint32_t* plan_word = nullptr, uint32_t plan_seq = 0,
-                      bool phased = false);
+                      bool phased = false, uint32_t* copy_out = nullptr);
 
 // Up to kSmallSort keys are sorted by one block in one ordinary launch
 // (sort_small.cu; sort_keys calls it for a push).  keys_out / pos_out: the
@@ -289,9 +293,9 @@ struct SmallSort {
 };
 cudaError_t sort_small(const SmallSort& a, int bits, cudaStream_t stream);
 
-// The distinct valid keys of a sorted array, ascending, into out; count to *count.
-void compact_sorted_heads(const uint32_t* sk, uint64_t n, uint32_t* out, uint32_t* count, uint32_t* tmp,
-                          cudaStream_t stream);
+// The distinct valid keys of a sorted array, in no particular order, into out;
+// their number is added to *count.
+void list_sorted_heads(const uint32_t* sk, uint64_t n, uint32_t* out, uint32_t* count, cudaStream_t stream);
 
 // Stream compaction (a count / scan / write pass), tmp of compact_tmp_words(n).
 size_t compact_tmp_words(uint64_t n);

@@ -75,6 +75,8 @@ struct SortArgs {
   uint32_t plan_seq;
   int phase;                     // -1: every phase, grid barriers between (cooperative launch);
                                  // k >= 0: phase k alone (0 count, 1 + 2p scan, 2 + 2p scatter of pass p)
+  int fused;                     // phased: the scatters scan (a table per pass)
+  uint32_t* copy_out;            // phased: a copy of raw (nullptr: none)
   int allow_nokey;
   int passes;
   int per;
@@ -191,7 +193,13 @@ __host__ __device__ constexpr uint32_t sort_barriers(int passes) { return 2u * (
 // What one sort launch runs: every phase with grid barriers between
 // (cooperative), or one phase of a phased sort.  A phased launch is compiled
 // with its own phase's code alone (registers, occupancy).
-enum SortKind { kSortAll = 0, kSortCount = 1, kSortScan = 2, kSortScatter = 3 };
+// With few blocks (kFusedBlocks) a scatter also scans: every block sums the
+// rows of the digit table itself, a warp per row, which takes less than the
+// scan launch and its gap (a clock of 8 x 16,384 keys by itself 574 -> 470 us;
+// with 128 blocks the table's reads cost more: 8 x 131,072 keys 1167 -> 1200
+// us).
+enum SortKind { kSortAll = 0, kSortCount = 1, kSortScan = 2, kSortScatter = 3, kSortScanScatter = 4 };
+constexpr uint32_t kFusedBlocks = 32;
 
 template <bool POS, int ITEMS, int KIND>
 __global__ void __launch_bounds__(kSortThreads, 4) sort_kernel(SortArgs a) {
@@ -254,7 +262,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) sort_kernel(SortArgs a) {
   auto run = [&](int ph) { return coop || a.phase == ph; };
   constexpr bool has_count = KIND == kSortAll || KIND == kSortCount;
   constexpr bool has_scan = KIND == kSortAll || KIND == kSortScan;
-  constexpr bool has_scatter = KIND == kSortAll || KIND == kSortScatter;
+  constexpr bool has_scatter = KIND == kSortAll || KIND == kSortScatter || KIND == kSortScanScatter;
     const uint64_t chunk = (a.n + B - 1) / B;
   const uint64_t c0 = a.n < b * chunk ? a.n : b * chunk;
   const uint64_t c1 = a.n < c0 + chunk ? a.n : c0 + chunk;
@@ -289,6 +297,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) sort_kernel(SortArgs a) {
         for (int it = 0; it < ITEMS; ++it) {
           if (i0 + (uint64_t)it * kSortThreads >= c1) continue;
           uint32_t k = kk[it];
+          if (a.copy_out) a.copy_out[i0 + (uint64_t)it * kSortThreads] = k;
           if (k >= a.K) {
             if (!(a.allow_nokey && k == kNoKey)) bad = true;
             k = kNoKey;
@@ -299,6 +308,10 @@ __global__ void __launch_bounds__(kSortThreads, 4) sort_kernel(SortArgs a) {
       __syncthreads();
     }
     for (uint32_t d = threadIdx.x; d <= mask; d += kSortThreads) table0[(uint64_t)d * B + b] = sm.cnt[d];
+    if (!coop && a.fused) {   // the later passes' tables
+      for (uint32_t d = threadIdx.x; d < (uint32_t)(a.passes - 1) * kDigits; d += kSortThreads)
+        table1[(uint64_t)d * B + b] = 0u;
+    }
     if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) set_error(a.st, ERR_KEY_RANGE);
   }
   if (coop && !grid_barrier(a, nbar, sm)) return;
@@ -313,6 +326,10 @@ __global__ void __launch_bounds__(kSortThreads, 4) sort_kernel(SortArgs a) {
     const uint32_t nmask = (1u << nnbits) - 1u;
     uint32_t* tcur = (p & 1) ? table1 : table0;
     uint32_t* tnext = (p & 1) ? table0 : table1;
+    if (KIND == kSortScanScatter) {
+      tcur = a.table + (uint64_t)p * kDigits * B;
+      tnext = tcur + (uint64_t)kDigits * B;
+    }
     // 1. exclusive prefix of each digit over the chunks and digit totals.
     // Up to 16 chunks: one thread per digit (its row in one round of
     // loads); 129 to 640: four warps per digit row, a quarter each in one
@@ -411,7 +428,51 @@ __global__ void __launch_bounds__(kSortThreads, 4) sort_kernel(SortArgs a) {
     // 2. scatter: digit bases, then the chunk's sub-tiles in order; each
     // written key is counted for the next pass in the chunk it lands in
     if (has_scatter && run(2 + 2 * p)) {
-    {
+    if (KIND == kSortScanScatter) {
+      // chunk b's exclusive prefix of every digit, and the digits' totals
+      constexpr int RQ = 4, JQ = (kFusedBlocks + 31) / 32;
+      for (uint32_t d0 = warp; d0 <= mask; d0 += kWarps * RQ) {
+        uint32_t pre[RQ], tot[RQ];
+#pragma unroll
+        for (int q = 0; q < RQ; ++q) {
+          const uint32_t d = d0 + q * kWarps;
+          pre[q] = 0u;
+          tot[q] = 0u;
+#pragma unroll
+          for (int jj = 0; jj < JQ; ++jj) {
+            const uint32_t j = jj * 32 + lane;
+            const uint32_t v = d <= mask && j < B ? __ldcg(tcur + (uint64_t)d * B + j) : 0u;
+            tot[q] += v;
+            pre[q] += j < b ? v : 0u;
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < RQ; ++q) {
+          const uint32_t d = d0 + q * kWarps;
+          const uint32_t ps = __reduce_add_sync(0xFFFFFFFFu, pre[q]), ts = __reduce_add_sync(0xFFFFFFFFu, tot[q]);
+          if (lane == 0 && d < (uint32_t)kDigits) {
+            sm.base[d] = ps;
+            sm.cnt[d] = ts;
+          }
+        }
+      }
+      __syncthreads();
+      uint32_t v[kDPT], local = 0;
+#pragma unroll
+      for (int q = 0; q < kDPT; ++q) {
+        const uint32_t d = threadIdx.x * kDPT + q;
+        v[q] = d <= mask ? sm.cnt[d] : 0u;
+        local += v[q];
+      }
+      uint32_t total;
+      uint32_t before = block_exclusive_scan<kSortThreads>(local, &total, sm.scan);
+#pragma unroll
+      for (int q = 0; q < kDPT; ++q) {
+        const uint32_t d = threadIdx.x * kDPT + q;
+        if (d <= mask) sm.base[d] += before;
+        before += v[q];
+      }
+    } else {
       uint32_t v[kDPT], local = 0;
 #pragma unroll
       for (int q = 0; q < kDPT; ++q) {
@@ -512,16 +573,32 @@ struct MapSel {
   __device__ uint32_t value(uint64_t i) const { return (uint32_t)i; }
 };
 
-// the first copy of every valid key of a sorted array (the distinct keys, ascending)
-struct HeadSel {
-  const uint32_t* sk;
-  uint64_t n;
-  __device__ bool flag(uint64_t i) const {
-    const uint32_t k = sk[i];
-    return k != kNoKey && (i == 0 || sk[i - 1] != k);
+// The first copy of every valid key of a sorted array, a tile per block, the
+// tiles in no particular order: *count (zero before) hands out their places.
+__global__ void __launch_bounds__(kSortThreads) list_heads_kernel(const uint32_t* __restrict__ sk, uint64_t n,
+                                                                  uint32_t* __restrict__ out, uint32_t* count) {
+  __shared__ uint32_t sm[kWarps];
+  __shared__ uint32_t base;
+  const uint64_t start = (uint64_t)blockIdx.x * kTile + threadIdx.x;
+  uint32_t k[kCompactItems];
+  bool f[kCompactItems];
+  uint32_t c = 0;
+#pragma unroll
+  for (int j = 0; j < kCompactItems; ++j) {
+    const uint64_t i = start + (uint64_t)j * kSortThreads;
+    k[j] = i < n ? sk[i] : kNoKey;
+    f[j] = k[j] != kNoKey && (i == 0 || sk[i - 1] != k[j]);
+    c += f[j] ? 1u : 0u;
   }
-  __device__ uint32_t value(uint64_t i) const { return sk[i]; }
-};
+  uint32_t tot;
+  uint32_t at = block_exclusive_scan<kSortThreads>(c, &tot, sm);
+  if (threadIdx.x == 0) base = tot ? atomicAdd(count, tot) : 0u;
+  __syncthreads();
+  at += base;
+#pragma unroll
+  for (int j = 0; j < kCompactItems; ++j)
+    if (f[j]) out[at++] = k[j];
+}
 
 template <class Sel>
 __global__ void __launch_bounds__(kSortThreads) compact_count_kernel(Sel sel, uint32_t* tile_cnt) {
@@ -636,11 +713,14 @@ cudaError_t launch_sort_phased(SortArgs& a, cudaStream_t stream) {
   if (B > kMaxSortBlocks) B = kMaxSortBlocks;
   if (B < 1) B = 1;
   a.bar_base = 0;
+  a.fused = B <= kFusedBlocks ? 1 : 0;
   const int phases = 1 + 2 * a.passes;
-  note_launches((uint64_t)phases);
+  note_launches((uint64_t)(a.fused ? 1 + a.passes : phases));
   for (int ph = 0; ph < phases; ++ph) {
     a.phase = ph;
-    if (ph == 0)
+    if (a.fused && ph > 0) {
+      if (!(ph & 1)) sort_kernel<POS, ITEMS, kSortScanScatter><<<(unsigned)B, kSortThreads, 0, stream>>>(a);
+    } else if (ph == 0)
       sort_kernel<POS, ITEMS, kSortCount><<<(unsigned)B, kSortThreads, 0, stream>>>(a);
     else if (ph & 1)
       sort_kernel<POS, ITEMS, kSortScan><<<(unsigned)B, kSortThreads, 0, stream>>>(a);
@@ -658,6 +738,16 @@ int bits_for(uint64_t num_keys) {
   return b;
 }
 
+size_t plan_scratch_words(uint64_t n, int bits) {
+  uint64_t rows = (n + kSubMin - 1) / kSubMin;
+  if (rows > kMaxSortBlocks) rows = kMaxSortBlocks;
+  if (rows < 1) rows = 1;
+  // totals, and two tables or (few blocks) one per pass
+  uint64_t columns = (uint64_t)plan_for(bits).passes * (rows < kFusedBlocks ? rows : kFusedBlocks);
+  if (columns < 2 * rows) columns = 2 * rows;
+  return (size_t)(kScratchHead + kDigits + columns * kDigits);
+}
+
 size_t sort_scratch_words(uint64_t n) {
   uint64_t rows = (n + kSubMin - 1) / kSubMin;
   if (rows > kMaxSortBlocks) rows = kMaxSortBlocks;
@@ -671,7 +761,7 @@ cudaError_t sort_keys(const uint32_t* raw, uint64_t n, uint64_t K, bool allow_no
                       uint32_t* ka, uint32_t* kb, uint32_t* va, uint32_t* vb, uint32_t* scratch, int sms,
                       DevState* st, unsigned long long* bar_base, uint32_t* clear0, uint32_t* clear1,
                       cudaStream_t stream, uint32_t** keys_out, uint32_t** pos_out, const uint32_t* plan_keys,
-                      uint32_t* plan_word, uint32_t plan_seq, bool phased) {
+                      uint32_t* plan_word, uint32_t plan_seq, bool phased, uint32_t* copy_out) {
   const PassPlan pl = plan_for(bits);
   // (a context whose next grid barrier was made to fail sorts with one)
   if (n <= (plan_keys ? kSmallPlan : kSmallSort) && va && !phased && n > 0 && (*bar_base >> 40) == 0) {
@@ -700,6 +790,8 @@ cudaError_t sort_keys(const uint32_t* raw, uint64_t n, uint64_t K, bool allow_no
   a.plan_word = plan_word;
   a.plan_seq = plan_seq;
   a.phase = -1;
+  a.fused = 0;
+  a.copy_out = phased ? copy_out : nullptr;
   a.raw = raw;
   a.n = n;
   a.K = K;
@@ -735,9 +827,10 @@ void compact_replica_keys(const int32_t* map_w, uint64_t K, uint32_t* out, uint3
   compact(MapSel{map_w, K}, out, count, tmp, stream);
 }
 
-void compact_sorted_heads(const uint32_t* sk, uint64_t n, uint32_t* out, uint32_t* count, uint32_t* tmp,
-                          cudaStream_t stream) {
-  compact(HeadSel{sk, n}, out, count, tmp, stream);
+void list_sorted_heads(const uint32_t* sk, uint64_t n, uint32_t* out, uint32_t* count, cudaStream_t stream) {
+  if (n == 0) return;
+  note_launches(1);
+  list_heads_kernel<<<(unsigned)((n + kTile - 1) / kTile), kSortThreads, 0, stream>>>(sk, n, out, count);
 }
 
 }  // namespace adapm
