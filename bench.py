@@ -456,6 +456,14 @@ class ComplEx:
         # keys in (4 B per row), every row read once and one delta row + key written per row
         return self.W * rows * (2 * self.row + 8)
 
+    push_rows_per_key = 1.5   # its accumulators read, its pending row written
+
+    def step_moved_bytes(self):
+        c = self.cfg
+        rows = c.batch * (3 + c.negatives)
+        # keys in, the theta half of every row read, a key and a scalar written per row, three theta rows per triple
+        return self.W * (rows * (4 + self.row / 2 + 8) + c.batch * 3 * self.row / 2)
+
     def prepare_host(self, clocks):
         self.hdata = {(w, cc): tuple(x.cpu().pin_memory() for x in self.data[(w, cc)]) for cc in clocks
                       for w in range(self.W) if (w, cc) in self.data}
@@ -534,6 +542,13 @@ class SGNS:
         # per centre: its rows read once, one delta row + key written per row
         return self.W * self.cfg.batch * self.per * (2 * self.row + 8)
 
+    push_rows_per_key = 1     # its pending row written
+
+    def step_moved_bytes(self):
+        c = self.cfg
+        # keys in, every row read, a key and a scalar written per row, two rows per centre
+        return self.W * c.batch * (self.per * (4 + self.row + 8) + 2 * self.row)
+
     def prepare_host(self, clocks):
         self.hdata = {(w, cc): tuple(x.cpu().pin_memory() for x in self.data[(w, cc)]) for cc in clocks
                       for w in range(self.W) if (w, cc) in self.data}
@@ -582,6 +597,34 @@ def alg_bytes_per_step(wk, d, steps, relocate=False):
     else:
         out["step"] = wk.step_alg_bytes()
         out["intent"] = R * 4 + U * 4
+    return out
+
+
+def moved_bytes_per_step(wk, d, steps, relocate=False):
+    """The least bytes the kernels move per step, which the roofline fractions are taken of.
+
+    Replicas are aliases of their main rows until somebody writes (see the replica states in internal.cuh), so
+    always replicating a push stores one row per distinct key, a destroyed replica moves three (its pending row
+    read, main read and written), a created one none and a sync reads 8 bytes per replica (the pending rows it
+    merges are not counted by the library).  The ComplEx and SGNS steps write a key and a scalar per row
+    occurrence and a few rows per sample, which their push reads instead of delta rows.  With relocation replicas
+    are copies and alg_bytes_per_step holds."""
+    out = alg_bytes_per_step(wk, d, steps, relocate)
+    row = wk.row
+    per = {k: v / steps for k, v in d.items()}
+    R, U = per["push_rows"], per["push_unique"]
+    rows_in, rows_out = R * row, row        # delta rows read; rows touched per distinct key
+    if hasattr(wk, "step_moved_bytes"):
+        out["step"] = wk.step_moved_bytes()
+        rows_in, rows_out = R * 4, wk.push_rows_per_key * row
+    if not relocate:
+        out["push"] = R * 4 + rows_in + U * (4 + rows_out)
+        out["push_kernel"] = R * 8 + rows_in + U * (4 + rows_out)
+        out["sync"] = per["sync_replicas"] * 8
+        out["advance"] = per["destroyed"] * 3 * row
+    elif hasattr(wk, "step_moved_bytes"):
+        out["push"] = R * 4 + rows_in + U * (4 + 2 * row)
+        out["push_kernel"] = R * 8 + rows_in + U * (4 + 2 * row)
     return out
 
 
@@ -677,7 +720,7 @@ def run_ours(args, ws, rank, local, workload=None):
 
     steps = args.steps
     delta = {k: s1[k] - s0[k] for k in COUNTERS}
-    alg = alg_bytes_per_step(wk, delta, steps, args.relocate)
+    alg = moved_bytes_per_step(wk, delta, steps, args.relocate)
     ops = {}
     for name, (t_ms, calls) in prof.items():
         if calls == 0:

@@ -151,7 +151,9 @@ adapm_status adapm_destroy(adapm_ctx* ctx);
  * when it builds the batch).  So the call also sorts its keys, with their
  * positions, on a stream of the library's own that runs beside the library
  * stream at low priority; the de-duplicated keys of a window that opens two
- * or more clocks ahead come from that sort.  A push (or training step) of the worker with as many keys
+ * or more clocks ahead (or of a few thousand keys) come from that sort, those
+ * of one that opens at the next advance from a pass beside the library
+ * stream.  A push (or training step) of the worker with as many keys
  * as its newest intent whose window holds the current clock checks on the
  * device that its keys equal that intent's, position by position, and then
  * groups its rows by the stored sort instead of sorting again; otherwise it
