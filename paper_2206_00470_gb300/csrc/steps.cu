@@ -55,11 +55,46 @@ __device__ __forceinline__ float4 f4scale(float4 a, float s) {
   return make_float4(a.x * s, a.y * s, a.z * s, a.w * s);
 }
 
-// The loss of a score x under label +1 (softplus(-x)) or -1 (softplus(x)),
-// added to *loss, and its derivative by x.
-__device__ __forceinline__ float score_coef(float x, bool positive, double* loss) {
-  *loss += (double)(positive ? softplus_f(-x) : softplus_f(x));
+// The derivative of a score's loss: softplus(-x) under label +1, softplus(x)
+// under label -1 (softplus_f of the same argument is the loss).
+__device__ __forceinline__ float score_coef(float x, bool positive) {
   return positive ? -sigmoid_f(-x) : sigmoid_f(x);
+}
+
+// Sums over the warp of U values per lane (U = 1, 2, 4), in 5 + U - 1 shuffles:
+// the lanes halve the values they carry before they halve the warp.  The
+// caller's lane gets the sum of value summed_row<U>(lane), which lane
+// summing_lane<U>(u) has for value u.
+template <int U>
+__device__ __forceinline__ int summed_row(int lane) {
+  return U == 1 ? 0 : (U == 2 ? (lane >> 4) & 1 : ((lane >> 4) & 1) | ((lane >> 2) & 2));
+}
+template <int U>
+__device__ __forceinline__ int summing_lane(int u) {
+  return U == 1 ? 0 : (U == 2 ? u << 4 : ((u & 1) << 4) | ((u & 2) << 2));
+}
+template <int U>
+__device__ __forceinline__ float sum_rows(const float (&part)[U], int lane) {
+  static_assert(U == 1 || U == 2 || U == 4, "values per lane");
+  float v[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) v[u] = part[u];
+  if (U >= 2) {
+    const bool hi = lane & 16;
+#pragma unroll
+    for (int u = 0; u < U / 2; ++u) {
+      const float keep = hi ? v[2 * u + 1] : v[2 * u], give = hi ? v[2 * u] : v[2 * u + 1];
+      v[u] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, 16);
+    }
+  }
+  if (U == 4) {
+    const bool hi = lane & 8;
+    const float keep = hi ? v[1 % U] : v[0], give = hi ? v[0] : v[1 % U];
+    v[0] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, 8);
+  }
+#pragma unroll
+  for (int o = U == 4 ? 4 : (U == 2 ? 8 : 16); o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], o);
+  return v[0];
 }
 
 template <int G>
@@ -314,6 +349,7 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
     k1 = J > 32 ? tail_key(i, 32 + lane) : tail_key(i + nwarps, lane);
     cur = row_bits(s, entry(key), key);
   };
+  for (int t = 0; t < DEPTH * 2 * CC; ++t) ring[t * 32] = f4zero();   // (columns no copy writes stay zero)
   restart(warp);
   for (uint64_t i = warp; i < n; i += nwarps) {
     const uint32_t kh = heads[i], kr = rels[i], kt = tails[i];
@@ -327,7 +363,8 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
     RowBits nxt{0ull, 0ull};
     uint32_t islot = 0, cslot = 0;   // ring slots of the next row copied, consumed
     auto issue = [&](uint32_t r, uint32_t j0) {   // row r of the triple (in the batch at j0 or the next)
-      const float4* pt = reinterpret_cast<const float4*>(__shfl_sync(0xFFFFFFFFu, r < j0 + 32 ? cur.p : nxt.p, r & 31));
+      const float4* pt = reinterpret_cast<const float4*>(
+          r < j0 + 32 ? __shfl_sync(0xFFFFFFFFu, cur.p, r & 31) : __shfl_sync(0xFFFFFFFFu, nxt.p, r & 31));
       if (r < J && pt != nullptr) {
 #pragma unroll
         for (int c = 0; c < CC; ++c) {
@@ -375,7 +412,8 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
       const uint32_t k2 = j0 + 64 < J ? tail_key(i, j0 + 64 + lane)
                           : j0 + 32 < J ? tail_key(i + nwarps, lane)
                           : J > 32 ? tail_key(i + nwarps, 32 + lane) : tail_key(i + 2 * nwarps, lane);
-      float mycoef = 0.f;
+      const unsigned there = __ballot_sync(0xFFFFFFFFu, cur.p != 0ull);   // rows of the batch that are not skipped
+      float mycoef = 0.f, myphi = 0.f;
       const uint32_t cnt = J - j0 < 32 ? J - j0 : 32;
 #pragma unroll 1
       for (uint32_t u0 = 0; u0 < cnt; u0 += U) {
@@ -385,12 +423,15 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
         float part[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const bool v = u0 + u < cnt && __shfl_sync(0xFFFFFFFFu, cur.p, (u0 + u) & 31) != 0ull;
+          const bool v = (there >> (u0 + u)) & 1u;   // (uniform; no bit at or above cnt is set)
 #pragma unroll
           for (int c = 0; c < CC; ++c) {
-            const bool cv = v && lane + 32 * c < (int)h4;
-            tre[u][c] = cv ? ring[(cslot * 2 * CC + 2 * c) * 32] : f4zero();
-            tim[u][c] = cv ? ring[(cslot * 2 * CC + 2 * c + 1) * 32] : f4zero();
+            tre[u][c] = f4zero();
+            tim[u][c] = f4zero();
+            if (v) {
+              tre[u][c] = ring[(cslot * 2 * CC + 2 * c) * 32];
+              tim[u][c] = ring[(cslot * 2 * CC + 2 * c + 1) * 32];
+            }
           }
           cslot = cslot + 1 == DEPTH ? 0 : cslot + 1;
         }
@@ -413,22 +454,24 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
           part[u] = 0.f;
 #pragma unroll
           for (int c = 0; c < CC; ++c) part[u] += dot4(xre[c], tre[u][c]) + dot4(xim[c], tim[u][c]);
-          part[u] = group_sum<32>(part[u]);
         }
+        const float phi = sum_rows<U>(part, lane);
         // (the ring slots just read are free)
 #pragma unroll
         for (int u = 0; u < U; ++u) issue(j0 + u0 + DEPTH + u, j0);
-        // lane u0 + u evaluates row u's loss and derivative
-        float phi = 0.f;
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (lane == (int)(u0 + u)) phi = part[u];
-        const bool eval = (uint32_t)lane >= u0 && (uint32_t)lane < u0 + U && (uint32_t)lane < cnt && key != kNoKey;
-        if (eval) mycoef = score_coef(phi, j0 + lane == 0, &lsum);
+        // every lane evaluates the derivative of the row it has the score of;
+        // lane u0 + u keeps row u's
+        const uint32_t ru = u0 + summed_row<U>(lane);
+        const float dphi = (there >> ru) & 1u ? score_coef(phi, j0 + ru == 0u) : 0.f;
+        const int from = summing_lane<U>((lane - (int)u0) & (U - 1));
+        const float s_phi = __shfl_sync(0xFFFFFFFFu, phi, from), s_coef = __shfl_sync(0xFFFFFFFFu, dphi, from);
+        if ((uint32_t)lane - u0 < (uint32_t)U) {
+          myphi = s_phi;
+          mycoef = s_coef;
+        }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const float coef = __shfl_sync(0xFFFFFFFFu, mycoef, (u0 + u) & 31);   // (0 for a skipped row)
-          if (u0 + u >= cnt) continue;
+          const float coef = __shfl_sync(0xFFFFFFFFu, dphi, summing_lane<U>(u));   // (0 for a skipped row)
 #pragma unroll
           for (int c = 0; c < CC; ++c) {
             Tre[c] = f4fma(tre[u][c], coef, Tre[c]);
@@ -436,6 +479,7 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
           }
         }
       }
+      if ((there >> lane) & 1u) lsum += (double)softplus_f(j0 + lane == 0 ? -myphi : myphi);
       if ((uint32_t)lane < cnt) {
         const uint64_t row = j0 + lane == 0 ? rt + i : rneg + i * n_neg + (j0 + lane - 1);
         o.dkeys[row] = key;
@@ -521,6 +565,7 @@ sgns_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ centres, cons
     k1 = T > 32 ? token(i, 32 + lane) : token(i + nwarps, lane);
     cur = row_bits(s, entry(key), key);
   };
+  for (int t = 0; t < DEPTH * C; ++t) ring[t * 32] = f4zero();   // (columns no copy writes stay zero)
   restart(warp);
   for (uint64_t i = warp; i < n; i += nwarps) {
     const uint64_t base = i * per;
@@ -534,7 +579,8 @@ sgns_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ centres, cons
     RowBits nxt{0ull, 0ull};
     uint32_t islot = 0, cslot = 0;   // ring slots of the next row copied, consumed
     auto issue = [&](uint32_t r, uint32_t t0) {   // row r of the centre (in the batch at t0 or the next)
-      const float4* px = reinterpret_cast<const float4*>(__shfl_sync(0xFFFFFFFFu, r < t0 + 32 ? cur.p : nxt.p, r & 31));
+      const float4* px = reinterpret_cast<const float4*>(
+          r < t0 + 32 ? __shfl_sync(0xFFFFFFFFu, cur.p, r & 31) : __shfl_sync(0xFFFFFFFFu, nxt.p, r & 31));
       if (r < T && px != nullptr) {
 #pragma unroll
         for (int c = 0; c < C; ++c) {
@@ -565,7 +611,9 @@ sgns_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ centres, cons
                           : t0 + 32 < T ? token(i + nwarps, lane)
                           : T > 32 ? token(i + nwarps, 32 + lane) : token(i + 2 * nwarps, lane);
       const bool positive = (t0 + lane) % per_ctx == 0;
-      float mycoef = 0.f;
+      const unsigned pos = __ballot_sync(0xFFFFFFFFu, positive);
+      const unsigned there = __ballot_sync(0xFFFFFFFFu, cur.p != 0ull);   // rows of the batch that are not skipped
+      float mycoef = 0.f, mysc = 0.f;
       const uint32_t cnt = T - t0 < 32 ? T - t0 : 32;
 #pragma unroll 1
       for (uint32_t u0 = 0; u0 < cnt; u0 += U) {
@@ -575,10 +623,12 @@ sgns_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ centres, cons
         float part[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const bool vx = u0 + u < cnt && __shfl_sync(0xFFFFFFFFu, cur.p, (u0 + u) & 31) != 0ull;
+          const bool vx = (there >> (u0 + u)) & 1u;   // (uniform; no bit at or above cnt is set)
 #pragma unroll
-          for (int c = 0; c < C; ++c)
-            x[u][c] = vx && lane + 32 * c < (int)D4 ? ring[(cslot * C + c) * 32] : f4zero();
+          for (int c = 0; c < C; ++c) {
+            x[u][c] = f4zero();
+            if (vx) x[u][c] = ring[(cslot * C + c) * 32];
+          }
           cslot = cslot + 1 == DEPTH ? 0 : cslot + 1;
         }
         if (any_add) {
@@ -598,26 +648,29 @@ sgns_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ centres, cons
           part[u] = 0.f;
 #pragma unroll
           for (int c = 0; c < C; ++c) part[u] += dot4(x[u][c], v[c]);
-          part[u] = group_sum<32>(part[u]);
         }
+        const float sc = sum_rows<U>(part, lane);
         // (the ring slots just read are free)
 #pragma unroll
         for (int u = 0; u < U; ++u) issue(t0 + u0 + DEPTH + u, t0);
-        // lane u0 + u evaluates row u's loss and derivative
-        float sc = 0.f;
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (lane == (int)(u0 + u)) sc = part[u];
-        const bool eval = (uint32_t)lane >= u0 && (uint32_t)lane < u0 + U && (uint32_t)lane < cnt && key != kNoKey;
-        if (eval) mycoef = score_coef(sc, positive, &lsum);
+        // every lane evaluates the derivative of the row it has the score of;
+        // lane u0 + u keeps row u's
+        const uint32_t ru = u0 + summed_row<U>(lane);
+        const float dsc = (there >> ru) & 1u ? score_coef(sc, (pos >> ru) & 1u) : 0.f;
+        const int from = summing_lane<U>((lane - (int)u0) & (U - 1));
+        const float s_sc = __shfl_sync(0xFFFFFFFFu, sc, from), s_coef = __shfl_sync(0xFFFFFFFFu, dsc, from);
+        if ((uint32_t)lane - u0 < (uint32_t)U) {
+          mysc = s_sc;
+          mycoef = s_coef;
+        }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const float coef = __shfl_sync(0xFFFFFFFFu, mycoef, (u0 + u) & 31);   // (0 for a skipped row)
-          if (u0 + u >= cnt) continue;
+          const float coef = __shfl_sync(0xFFFFFFFFu, dsc, summing_lane<U>(u));   // (0 for a skipped row)
 #pragma unroll
           for (int c = 0; c < C; ++c) gv[c] = f4fma(x[u][c], coef, gv[c]);
         }
       }
+      if ((there >> lane) & 1u) lsum += (double)softplus_f(positive ? -mysc : mysc);
       if ((uint32_t)lane < cnt) {
         o.dkeys[base + 1 + t0 + lane] = key;
         o.coef[base + 1 + t0 + lane] = -lr * mycoef;
