@@ -561,7 +561,27 @@ __global__ void events_undo_kernel(Store s, uint32_t w, EventBatch eb, int sign)
   }
 }
 
+// The caller's keys, copied in the library stream's order for the streams
+// that read them beside it; `zero` (may be null) is cleared with them.  A
+// kernel: a device-to-device copy and a clearing of the count are two
+// operations of the copy path, whose hand-over the next kernel waits for.
+__global__ void __launch_bounds__(kThreads)
+copy_keys_kernel(const uint32_t* __restrict__ keys, uint64_t n, uint32_t* __restrict__ out, uint32_t* zero) {
+  if (zero && blockIdx.x == 0 && threadIdx.x == 0) *zero = 0;
+  const uint64_t i = 4 * ((uint64_t)blockIdx.x * kThreads + threadIdx.x);
+  if (i + 4 <= n && (reinterpret_cast<uintptr_t>(keys) & 15) == 0) {   // out is the library's own: aligned
+    reinterpret_cast<uint4*>(out)[i / 4] = __ldg(reinterpret_cast<const uint4*>(keys) + i / 4);
+  } else {
+    for (uint64_t j = i; j < i + 4 && j < n; ++j) out[j] = __ldg(keys + j);
+  }
+}
+
 }  // namespace
+
+void launch_copy_keys(const uint32_t* keys, uint64_t n, uint32_t* out, uint32_t* zero, cudaStream_t stream) {
+  note_launches(1);
+  copy_keys_kernel<<<(unsigned)((n + 4 * kThreads - 1) / (4 * kThreads)), kThreads, 0, stream>>>(keys, n, out, zero);
+}
 
 void launch_intent_dedup(const Store& s, const uint32_t* keys, uint64_t n, uint32_t tag, uint32_t* out,
                          uint32_t* count, int sms, cudaStream_t stream) {

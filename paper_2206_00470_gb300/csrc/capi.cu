@@ -105,7 +105,6 @@ struct IntentList {
   cudaEvent_t listed = nullptr;   // the distinct keys, when the early stream makes them
   bool plan_used = false;      // a push took this plan
   cudaEvent_t ready = nullptr;
-  void* in_owned = nullptr;   // the call's staged copy of host keys, read by the plan stream
   int64_t start = 0, end = 0; // the window as signalled
 };
 
@@ -756,27 +755,27 @@ SmallSort small_plan(adapm_ctx* ctx, const IntentList& L, const uint32_t* keys) 
   a.K = ctx->s.K;
   a.keys_out = L.psk;
   a.pos_out = L.psp;
-  a.copy_out = L.px;
+  a.copy_out = keys == L.px ? nullptr : L.px;   // (a plan made in the library stream's order)
   a.heads_out = L.keys;
   a.heads_count = L.count;
   a.st = ctx->dstate;
   return a;
 }
 
-// Sort an intent's keys with their positions on the plan stream (a phased
+// Sort an intent's keys (L.px) with their positions on the plan stream (a phased
 // sort: no block waits for another, so it runs in whatever the library
 // stream leaves of the GPU), into L.psk / L.psp; with from_plan the distinct
 // keys follow from the sorted ones (ascending) into L.keys / L.count.
 // L.ready is recorded on the plan stream after all of it.  The library
 // stream must have enqueued the keys (and L's arrays) before `after`.
-cudaError_t make_plan(adapm_ctx* ctx, IntentList& L, const uint32_t* keys, cudaEvent_t after) {
+cudaError_t make_plan(adapm_ctx* ctx, IntentList& L, cudaEvent_t after) {
   cudaError_t e = ensure_plan_stream(ctx);
   if (e != cudaSuccess) return e;
   cudaStream_t ps = ctx->plan_stream;
   const uint64_t n = L.n;
   if ((e = cudaStreamWaitEvent(ps, after, 0)) != cudaSuccess) return e;
-  if (n <= kSmallIntent) {   // one launch for the sort, the copy of the keys and the distinct ones
-    if ((e = sort_small(small_plan(ctx, L, keys), ctx->bits, ps)) != cudaSuccess) return e;
+  if (n <= kSmallIntent) {   // one launch for the sort and the distinct keys
+    if ((e = sort_small(small_plan(ctx, L, L.px), ctx->bits, ps)) != cudaSuccess) return e;
     if ((e = take_ready_event(ctx, &L.ready)) != cudaSuccess) return e;
     return cudaEventRecord(L.ready, ps);
   }
@@ -791,9 +790,9 @@ cudaError_t make_plan(adapm_ctx* ctx, IntentList& L, const uint32_t* keys, cudaE
   const bool odd = sort_passes(ctx->bits) % 2 == 1;   // the sort ends in ka / va after odd passes
   unsigned long long no_barriers = 0;
   uint32_t *sk = nullptr, *sp = nullptr;
-  e = sort_keys(keys, n, ctx->s.K, false, ctx->bits, odd ? L.psk : tk, odd ? tk : L.psk, odd ? L.psp : tv,
+  e = sort_keys(L.px, n, ctx->s.K, false, ctx->bits, odd ? L.psk : tk, odd ? tk : L.psk, odd ? L.psp : tv,
                 odd ? tv : L.psp, hist, ctx->sms, ctx->dstate, &no_barriers, L.from_plan ? L.count : nullptr, nullptr,
-                ps, &sk, &sp, nullptr, nullptr, 0, /*phased=*/true, L.px);
+                ps, &sk, &sp, nullptr, nullptr, 0, /*phased=*/true);
   if (e != cudaSuccess) return e;
   if (L.from_plan) list_sorted_heads(L.psk, n, L.keys, L.count, ps);   // (the sort zeroed the count)
   for (uint32_t* p : {tk, tv, hist})
@@ -820,7 +819,7 @@ cudaError_t close_list(adapm_ctx* ctx, uint32_t w, int64_t id) {
     if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, L.listed, 0);
     ctx->spare_ready.push_back(L.listed);
   }
-  for (void* p : {(void*)L.keys, (void*)L.psk, (void*)L.psp, (void*)L.px, L.in_owned}) pool_free(ctx, p);
+  for (void* p : {(void*)L.keys, (void*)L.psk, (void*)L.psp, (void*)L.px}) pool_free(ctx, p);
   auto& order = ctx->workers[w].order;
   order.erase(std::remove(order.begin(), order.end(), id), order.end());
   ctx->lists.erase(id);
@@ -987,8 +986,7 @@ adapm_status adapm_destroy(adapm_ctx* ctx) {
     if (ws.early.done) cudaEventDestroy(ws.early.done);
   }
   for (auto& kv : ctx->lists) {
-    for (void* p : {(void*)kv.second.keys, (void*)kv.second.psk, (void*)kv.second.psp, (void*)kv.second.px,
-                    kv.second.in_owned})
+    for (void* p : {(void*)kv.second.keys, (void*)kv.second.psk, (void*)kv.second.psp, (void*)kv.second.px})
       if (p) cudaFree(p);
     if (kv.second.ready) cudaEventDestroy(kv.second.ready);
     if (kv.second.listed) cudaEventDestroy(kv.second.listed);
@@ -1056,7 +1054,6 @@ adapm_status adapm_intent(adapm_ctx* ctx, uint32_t worker, const uint32_t* keys,
     if (plan) {
       CK(pool_alloc(ctx, &L.psk, n));
       CK(pool_alloc(ctx, &L.psp, n));
-      CK(pool_alloc(ctx, &L.px, n));
     }
     // Where the distinct keys come from.  A window that opens two or more
     // clocks ahead: the plan.  One that opens at the next advance would wait
@@ -1069,6 +1066,16 @@ adapm_status adapm_intent(adapm_ctx* ctx, uint32_t worker, const uint32_t* keys,
     const bool small = n <= kSmallIntent;
     L.from_plan = plan && !now && (small || clock_start > ws.clock + 1);
     const bool early = !small && !L.from_plan && !now;
+    const bool planned_here = plan && small && !L.from_plan;   // the plan is made on this stream
+    // What the other streams read is the library's own: the staged copy of
+    // host keys, or a copy of device keys made in this stream's order (the
+    // array may be changed or reused in that order after the call).  A push
+    // compares its keys with it, too.
+    const bool kept = plan || early;
+    if (kept && in.owned) L.px = in.owned;
+    if (kept && !in.owned) CK(pool_alloc(ctx, &L.px, n));
+    if (kept && !in.owned && !planned_here)
+      launch_copy_keys(in.dev, n, L.px, early ? L.count : nullptr, ctx->stream);
     if (L.from_plan) {
     } else if (small) {
       CK(sort_small(small_plan(ctx, L, in.dev), ctx->bits, ctx->stream));
@@ -1090,27 +1097,22 @@ adapm_status adapm_intent(adapm_ctx* ctx, uint32_t worker, const uint32_t* keys,
         CK(cudaStreamWaitEvent(on, after, 0));
         ctx->spare_ready.push_back(after);   // the wait has captured it
       }
-      CK(cudaMemsetAsync(L.count, 0, sizeof(uint32_t), on));
-      launch_intent_dedup(ctx->s, in.dev, n, ctx->intent_tag, L.keys, L.count, ctx->sms, on);
+      if (!early || in.owned) CK(cudaMemsetAsync(L.count, 0, sizeof(uint32_t), on));
+      launch_intent_dedup(ctx->s, early ? L.px : in.dev, n, ctx->intent_tag, L.keys, L.count, ctx->sms, on);
       if (early) {
         CK(cudaEventRecord(ctx->early_dedup, on));
         CK(take_ready_event(ctx, &L.listed));
         CK(cudaEventRecord(L.listed, on));
       }
     }
-    const bool planned_here = plan && small && !L.from_plan;   // the plan was made on this stream
     if (plan && !planned_here) {
       cudaEvent_t after = nullptr;
       CK(take_ready_event(ctx, &after));
       CK(cudaEventRecord(after, ctx->stream));
-      CK(make_plan(ctx, L, in.dev, after));
+      CK(make_plan(ctx, L, after));
       ctx->spare_ready.push_back(after);   // the plan stream's wait has captured it
-      L.in_owned = in.owned;               // freed when the list closes, after the plan
-    } else if (early) {
-      L.in_owned = in.owned;               // freed when the list closes
-    } else {
-      pool_free(ctx, in.owned);
     }
+    if (!kept) pool_free(ctx, in.owned);   // (else freed when the list closes, after its plan)
   }
   const int64_t id = ctx->next_list++;
   ctx->lists[id] = L;

@@ -3,7 +3,7 @@
 // Device data layout (all in HBM, owned by the context):
 //   main        [K][D] fp32     main copy of every parameter
 //   val, acc    [S][D] fp32     replica pool: local value and pending updates
-//                               (rows are written only when needed, see RepState)
+//                               (rows are written only when needed, see the replica states)
 //   map         [W][K] int32    worker w's replica of key k: -1 if none, else its
 //                               slot, with bit 31 set when slot_owner may hold
 //                               a state other than REP_ALIAS (see map_touched)
@@ -253,8 +253,7 @@ __device__ __forceinline__ bool sort_failed(const DevState* st) {
 // work, where a cooperative launch would wait for the whole GPU.  One for the
 // count and two per pass, or one per pass when the blocks are few enough that
 // each scans the digit table itself.  `scratch` then holds
-// plan_scratch_words(n, bits) words, and copy_out (may be null) receives the
-// keys as given.
+// plan_scratch_words(n, bits) words.
 size_t sort_scratch_words(uint64_t n);
 size_t plan_scratch_words(uint64_t n, int bits);
 int sort_passes(int bits);
@@ -263,7 +262,7 @@ cudaError_t sort_keys(const uint32_t* raw, uint64_t n, uint64_t K, bool allow_no
                       DevState* st, unsigned long long* bar_base, uint32_t* clear0, uint32_t* clear1,
                       cudaStream_t stream, uint32_t** keys_out, uint32_t** pos_out,
                       const uint32_t* plan_keys = nullptr, uint32_t* plan_word = nullptr, uint32_t plan_seq = 0,
-                      bool phased = false, uint32_t* copy_out = nullptr);
+                      bool phased = false);
 
 // Up to kSmallSort keys are sorted by one block in one ordinary launch
 // (sort_small.cu; sort_keys calls it for a push).  keys_out / pos_out: the

@@ -76,7 +76,6 @@ struct SortArgs {
   int phase;                     // -1: every phase, grid barriers between (cooperative launch);
                                  // k >= 0: phase k alone (0 count, 1 + 2p scan, 2 + 2p scatter of pass p)
   int fused;                     // phased: the scatters scan (a table per pass)
-  uint32_t* copy_out;            // phased: a copy of raw (nullptr: none)
   int allow_nokey;
   int passes;
   int per;
@@ -297,7 +296,6 @@ __global__ void __launch_bounds__(kSortThreads, 4) sort_kernel(SortArgs a) {
         for (int it = 0; it < ITEMS; ++it) {
           if (i0 + (uint64_t)it * kSortThreads >= c1) continue;
           uint32_t k = kk[it];
-          if (a.copy_out) a.copy_out[i0 + (uint64_t)it * kSortThreads] = k;
           if (k >= a.K) {
             if (!(a.allow_nokey && k == kNoKey)) bad = true;
             k = kNoKey;
@@ -761,7 +759,7 @@ cudaError_t sort_keys(const uint32_t* raw, uint64_t n, uint64_t K, bool allow_no
                       uint32_t* ka, uint32_t* kb, uint32_t* va, uint32_t* vb, uint32_t* scratch, int sms,
                       DevState* st, unsigned long long* bar_base, uint32_t* clear0, uint32_t* clear1,
                       cudaStream_t stream, uint32_t** keys_out, uint32_t** pos_out, const uint32_t* plan_keys,
-                      uint32_t* plan_word, uint32_t plan_seq, bool phased, uint32_t* copy_out) {
+                      uint32_t* plan_word, uint32_t plan_seq, bool phased) {
   const PassPlan pl = plan_for(bits);
   // (a context whose next grid barrier was made to fail sorts with one)
   if (n <= (plan_keys ? kSmallPlan : kSmallSort) && va && !phased && n > 0 && (*bar_base >> 40) == 0) {
@@ -791,7 +789,6 @@ cudaError_t sort_keys(const uint32_t* raw, uint64_t n, uint64_t K, bool allow_no
   a.plan_seq = plan_seq;
   a.phase = -1;
   a.fused = 0;
-  a.copy_out = phased ? copy_out : nullptr;
   a.raw = raw;
   a.n = n;
   a.K = K;

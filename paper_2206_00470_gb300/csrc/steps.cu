@@ -104,7 +104,7 @@ __device__ __forceinline__ float group_sum(float v) {
   return v;
 }
 
-// Where a worker's value of a key is read (see RepState): the row, and the
+// Where a worker's value of a key is read (see the replica states): the row, and the
 // pending row to add to it when one push is pending on an alias (few have
 // one at a step: a null pointer otherwise).
 struct Row {

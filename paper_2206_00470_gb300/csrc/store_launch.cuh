@@ -61,6 +61,7 @@ struct EventList {
 // dropped), in no particular order, appended to out; *count (zeroed by the
 // caller) receives their number.  `tag` must differ from every stamp left
 // by earlier calls.
+void launch_copy_keys(const uint32_t* keys, uint64_t n, uint32_t* out, uint32_t* zero, cudaStream_t stream);
 void launch_intent_dedup(const Store& s, const uint32_t* keys, uint64_t n, uint32_t tag, uint32_t* out,
                          uint32_t* count, int sms, cudaStream_t stream);
 void launch_pull(const Store& s, int w, const uint32_t* keys, uint64_t n, float* out, int sms,

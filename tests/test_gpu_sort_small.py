@@ -75,3 +75,34 @@ def test_keys_out_of_range(gpu_lib, n):
     pm.advance_clock(0)
     assert np.array_equal(pm.replica_keys(0), np.unique(good))
     pm.close()
+
+
+# 32,768 keys: the last size whose plan scans in its scatter (its blocks' digit counts fit one pass), 32,769 the next
+@pytest.mark.parametrize("n,ahead", [(100, 1), (4097, 1), (4097, 2), (32_768, 2), (32_769, 2)])
+def test_device_keys_may_change_behind_an_intent(gpu_lib, n, ahead):
+    """An intent reads device keys in stream order, whichever stream sorts or lists them."""
+    K, D = 70_000, 4
+    rng = np.random.default_rng(n + ahead)
+    stream = torch.cuda.Stream()
+    pm = gpu_lib.ParameterManager(K, D, 1, stream=stream)
+    keys = rng.integers(0, K, size=n)
+    with torch.cuda.stream(stream):
+        d = torch.from_numpy(keys.astype(np.int32)).cuda()
+        for _ in range(20):                # (many, so that the side streams lag)
+            pm.intent(0, d, ahead, ahead + 1)
+        d.fill_(5)
+    for _ in range(ahead):
+        pm.advance_clock(0)
+    stream.synchronize()
+    pm.wait()
+    assert np.array_equal(pm.replica_keys(0), np.unique(keys))
+    assert pm.refcounts(0, np.unique(keys)).tolist() == [20] * len(np.unique(keys))
+    with torch.cuda.stream(stream):
+        pm.push(0, dev(keys), torch.ones(n, D, device="cuda"))
+    pm.wait()
+    pm.sync()
+    pm.wait()
+    assert np.array_equal(pm.read_main(np.arange(K)), np.bincount(keys, minlength=K)[:, None] * np.ones(D))
+    st = pm.stats()
+    assert (st["planned_pushes"], st["plan_misses"]) == (1, 0)
+    pm.close()
