@@ -43,9 +43,13 @@ namespace {
 // back to the pool, which the context owns and destroys.
 class BlockCache {
  public:
-  cudaError_t take(cudaMemPool_t pool, cudaStream_t stream, size_t bytes, void** p) {
-    const size_t size = bytes <= kLargest ? round_up(bytes) : bytes;
-    auto it = size <= kLargest ? free_.find(size) : free_.end();
+  // capturing: the stream records a graph.  Its blocks come from the pool and
+  // go back to it inside the graph (a kept block would outlive its allocation
+  // node, or be handed to other work while the graph runs).
+  cudaError_t take(cudaMemPool_t pool, cudaStream_t stream, size_t bytes, bool capturing, void** p) {
+    const bool keep = bytes <= kLargest && !capturing;
+    const size_t size = keep ? round_up(bytes) : bytes;
+    auto it = keep ? free_.find(size) : free_.end();
     if (it != free_.end() && !it->second.empty()) {
       *p = it->second.back();
       it->second.pop_back();
@@ -53,21 +57,26 @@ class BlockCache {
       return cudaSuccess;
     }
     const cudaError_t e = cudaMallocFromPoolAsync(p, size, pool, stream);
-    if (e == cudaSuccess && size <= kLargest) size_[*p] = size;
+    if (e == cudaSuccess && keep) {
+      try {
+        size_[*p] = size;
+      } catch (...) {   // no host memory to remember it by: given back like any other
+      }
+    }
     return e;
   }
-  // false: not a block of this cache (the caller frees it)
-  bool give(void* p, cudaStream_t stream) {
+  void give(void* p, cudaStream_t stream) {
     auto it = size_.find(p);
-    if (it == size_.end()) return false;
-    if (kept_ + it->second > kKeep) {
-      size_.erase(it);
-      cudaFreeAsync(p, stream);
-      return true;
+    if (it != size_.end() && kept_ + it->second <= kKeep) {
+      try {
+        free_[it->second].push_back(p);
+        kept_ += it->second;
+        return;
+      } catch (...) {
+      }
     }
-    kept_ += it->second;
-    free_[it->second].push_back(p);
-    return true;
+    if (it != size_.end()) size_.erase(it);
+    cudaFreeAsync(p, stream);
   }
   void release() {   // the stream is idle
     for (auto& f : free_)
@@ -145,6 +154,7 @@ struct adapm_ctx {
   int bits = 32;
   cudaMemPool_t pool = nullptr;
   BlockCache blocks, plan_blocks;   // scratch of the library stream, of the plan stream
+  bool capturing = false;           // this call's work goes into a graph (check_ctx)
   Store s{};
   DevState* dstate = nullptr;
   std::vector<WorkerState> workers;
@@ -342,11 +352,11 @@ cudaError_t stage_mark(adapm_ctx* ctx, uint64_t next_bytes) {
 template <class T>
 cudaError_t pool_alloc(adapm_ctx* ctx, T** p, size_t count) {
   if (count == 0) count = 1;
-  return ctx->blocks.take(ctx->pool, ctx->stream, count * sizeof(T), reinterpret_cast<void**>(p));
+  return ctx->blocks.take(ctx->pool, ctx->stream, count * sizeof(T), ctx->capturing, reinterpret_cast<void**>(p));
 }
 
 void pool_free(adapm_ctx* ctx, void* p) {
-  if (p && !ctx->blocks.give(p, ctx->stream)) cudaFreeAsync(p, ctx->stream);
+  if (p) ctx->blocks.give(p, ctx->stream);
 }
 
 // Device view of an input array; copies host arrays in.
@@ -456,6 +466,12 @@ adapm_status check_ctx(adapm_ctx* ctx) {
   if (ctx->broken) return fail(ctx, ADAPM_ECUDA, "context unusable after an earlier CUDA error");
   ctx->err.clear();
   if (cudaSetDevice(ctx->device) != cudaSuccess) return fail(ctx, ADAPM_ECUDA, "cudaSetDevice");
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess) {
+    cudaGetLastError();   // (not answered, e.g. while another thread captures: this stream does not)
+    cap = cudaStreamCaptureStatusNone;
+  }
+  ctx->capturing = cap != cudaStreamCaptureStatusNone;
   return ADAPM_OK;
 }
 
@@ -781,7 +797,7 @@ cudaError_t make_plan(adapm_ctx* ctx, IntentList& L, cudaEvent_t after) {
   }
   uint32_t *tk = nullptr, *tv = nullptr, *hist = nullptr;
   auto palloc = [&](uint32_t** p, size_t words) {
-    return ctx->plan_blocks.take(ctx->plan_pool, ps, (words ? words : 1) * sizeof(uint32_t),
+    return ctx->plan_blocks.take(ctx->plan_pool, ps, (words ? words : 1) * sizeof(uint32_t), ctx->capturing,
                                  reinterpret_cast<void**>(p));
   };
   if ((e = palloc(&tk, n)) != cudaSuccess || (e = palloc(&tv, n)) != cudaSuccess ||
@@ -795,8 +811,7 @@ cudaError_t make_plan(adapm_ctx* ctx, IntentList& L, cudaEvent_t after) {
                 ps, &sk, &sp, nullptr, nullptr, 0, /*phased=*/true);
   if (e != cudaSuccess) return e;
   if (L.from_plan) list_sorted_heads(L.psk, n, L.keys, L.count, ps);   // (the sort zeroed the count)
-  for (uint32_t* p : {tk, tv, hist})
-    if (!ctx->plan_blocks.give(p, ps)) cudaFreeAsync(p, ps);
+  for (uint32_t* p : {tk, tv, hist}) ctx->plan_blocks.give(p, ps);
   if ((e = take_ready_event(ctx, &L.ready)) != cudaSuccess) return e;
   if ((e = cudaEventRecord(L.ready, ps)) != cudaSuccess) return e;
   return cudaGetLastError();
