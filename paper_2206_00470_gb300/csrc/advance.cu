@@ -182,6 +182,7 @@ __device__ void settle_advance(DevState* st, int32_t S) {
 template <bool START>
 __global__ void events_kernel(Store s, uint32_t w, EventBatch eb, uint32_t* out_list, int settle,
                               AdvCounts* early) {
+  after_previous();
   if (sort_failed(s.st)) return;
   constexpr int Q = 4;
   __shared__ uint32_t base_s;
@@ -362,6 +363,7 @@ __global__ void __launch_bounds__(kThreads, evict_blocks_per_sm(C)) evict_create
                                                                               const uint32_t* __restrict__ evict_list,
                                                                               const uint32_t* __restrict__ create_list,
                                                                               AdvCounts* early) {
+  after_previous();
   constexpr int R = C == 3 || C == 4 ? 2 : (4 / C > 0 ? 4 / C : 1);
   constexpr uint32_t GW = 32 / G;   // row groups per warp
   __shared__ uint2 moves[kThreads / 32][32];    // (slot, key): pending rows to add to main
@@ -567,6 +569,7 @@ __global__ void events_undo_kernel(Store s, uint32_t w, EventBatch eb, int sign)
 // operations of the copy path, whose hand-over the next kernel waits for.
 __global__ void __launch_bounds__(kThreads)
 copy_keys_kernel(const uint32_t* __restrict__ keys, uint64_t n, uint32_t* __restrict__ out, uint32_t* zero) {
+  after_previous();
   if (zero && blockIdx.x == 0 && threadIdx.x == 0) *zero = 0;
   const uint64_t i = 4 * ((uint64_t)blockIdx.x * kThreads + threadIdx.x);
   if (i + 4 <= n && (reinterpret_cast<uintptr_t>(keys) & 15) == 0) {   // out is the library's own: aligned
@@ -580,7 +583,8 @@ copy_keys_kernel(const uint32_t* __restrict__ keys, uint64_t n, uint32_t* __rest
 
 void launch_copy_keys(const uint32_t* keys, uint64_t n, uint32_t* out, uint32_t* zero, cudaStream_t stream) {
   note_launches(1);
-  copy_keys_kernel<<<(unsigned)((n + 4 * kThreads - 1) / (4 * kThreads)), kThreads, 0, stream>>>(keys, n, out, zero);
+  const unsigned grid = (unsigned)((n + 4 * kThreads - 1) / (4 * kThreads));
+  launch_after(copy_keys_kernel, grid, kThreads, 0, stream, keys, n, out, zero);
 }
 
 void launch_intent_dedup(const Store& s, const uint32_t* keys, uint64_t n, uint32_t tag, uint32_t* out,
@@ -629,6 +633,7 @@ void launch_events(const Store& s, uint32_t w, const EventList* lists, int nlist
   const uint64_t cap_blocks = (uint64_t)sms * 8;
   std::vector<std::pair<EventBatch, uint64_t>> batches[2];
   event_batches(lists, nlists, early == nullptr, batches);
+  bool follows = !early;   // (the early stream has just waited for the library stream)
   for (int pass = 0; pass < 2; ++pass) {
     for (size_t i = 0; i < batches[pass].size(); ++i) {
       const EventBatch& eb = batches[pass][i].first;
@@ -636,11 +641,10 @@ void launch_events(const Store& s, uint32_t w, const EventList* lists, int nlist
       if (b > cap_blocks) b = cap_blocks;
       if (b == 0) b = 1;
       note_launches(1);
-      if (pass == 0)
-        events_kernel<true><<<(unsigned)b, kThreads, 0, stream>>>(s, w, eb, create_list, 0, early);
-      else
-        events_kernel<false><<<(unsigned)b, kThreads, 0, stream>>>(
-            s, w, eb, evict_list, (!early && i + 1 == batches[1].size()) ? 1 : 0, early);
+      const int settle = pass == 1 && !early && i + 1 == batches[1].size() ? 1 : 0;
+      launch_on(follows, pass == 0 ? events_kernel<true> : events_kernel<false>, (unsigned)b, kThreads, 0, stream, s, w,
+                eb, pass == 0 ? create_list : evict_list, settle, early);
+      follows = true;
     }
   }
 }
@@ -673,7 +677,8 @@ void launch_evict_create(const Store& s, uint32_t w, const uint32_t* create_list
     if (blocks < 1) blocks = 1;
     const unsigned grid = (unsigned)blocks;
     note_launches(1);
-    evict_create_kernel<G, C><<<grid, kThreads, 0, stream>>>(s, w, evict_list, create_list, early);
+    // (after early events the stream has just waited for theirs)
+    launch_on(!early, evict_create_kernel<G, C>, grid, kThreads, 0, stream, s, w, evict_list, create_list, early);
   });
 }
 

@@ -32,6 +32,7 @@ template <int G, int C>
 __global__ void __launch_bounds__(kThreads, C >= 8 ? 2 : 3) evict_create_copied_kernel(Store s, uint32_t w,
                                                                                      const uint32_t* __restrict__ evict_list,
                                                                                      const uint32_t* __restrict__ create_list) {
+  after_previous();
   constexpr int R = 4 / C > 0 ? 4 / C : 1;
   const int lane = threadIdx.x & (G - 1);
   const uint32_t D4 = s.D >> 2;
@@ -144,6 +145,7 @@ __global__ void __launch_bounds__(kThreads, C >= 8 ? 2 : 3) evict_create_copied_
 // VER: versioned refresh (s.dirty is set)
 template <int G, int C, bool VER>
 __global__ void __launch_bounds__(kThreads, C >= 8 ? 2 : (VER && C == 1 ? 3 : 4)) sync_copied_kernel(Store s) {
+  after_previous();
   const int lane = threadIdx.x & (G - 1);
   const uint32_t D4 = s.D >> 2;
   const uint64_t hw = (uint64_t)s.st->high_water;
@@ -363,8 +365,8 @@ void launch_evict_create_copied(const Store& s, uint32_t w, const uint32_t* crea
     constexpr int G = decltype(Gc)::value, C = decltype(Cc)::value;
     constexpr uint64_t R = 4 / C > 0 ? 4 / C : 1;   // list entries per group, as in the kernel
     note_launches(1);
-    evict_create_copied_kernel<G, C><<<grid_for((max_events + R - 1) / R, G, sms), kThreads, 0, stream>>>(
-        s, w, evict_list, create_list);
+    const unsigned grid = grid_for((max_events + R - 1) / R, G, sms);
+    launch_after(evict_create_copied_kernel<G, C>, grid, kThreads, 0, stream, s, w, evict_list, create_list);
   });
 }
 
@@ -375,8 +377,8 @@ void launch_sync_copied(const Store& s, uint64_t slot_bound, int sms, cudaStream
     note_launches(1);
     constexpr uint64_t R = 4 / C > 0 ? 4 / C : 1;   // slots per group, as in the kernel
     const unsigned grid = grid_for((slot_bound + R - 1) / R, G, sms);
-    if (s.dirty != nullptr) sync_copied_kernel<G, C, true><<<grid, kThreads, 0, stream>>>(s);
-    else sync_copied_kernel<G, C, false><<<grid, kThreads, 0, stream>>>(s);
+    if (s.dirty != nullptr) launch_after(sync_copied_kernel<G, C, true>, grid, kThreads, 0, stream, s);
+    else launch_after(sync_copied_kernel<G, C, false>, grid, kThreads, 0, stream, s);
   });
 }
 

@@ -341,4 +341,45 @@ struct ProfToken {
 ProfToken ctx_prof_start(struct ::adapm_ctx* ctx, int op);
 void ctx_prof_stop(struct ::adapm_ctx* ctx, ProfToken& t);
 
+// ---- launches that overlap the end of the kernel before them ----------------
+// The kernels of a call, and of one call after another, follow each other on
+// one stream, and a kernel of a few thousand rows is not much longer than the
+// gap in front of it.  launch_after starts a kernel while the one before it
+// drains: its blocks are placed as soon as that kernel's blocks have all left
+// (no kernel here lets go earlier, so nothing it keeps in caches is read
+// before it is final), and its first statement, after_previous(), waits until
+// the other's writes are visible.  Every block makes that wait, so a kernel
+// ends after all before it on the stream have, and a kernel or event that
+// follows sees them too.  A kernel that a stream runs right after a wait for
+// another stream has nothing to overlap and is launched plainly (the
+// attribute costs the host more than it gives: follows = false).
+//
+// Measured, per pass: 1000 keys pulled and pushed 30 -> 21 us, a clock of 8 x
+// 16,384 keys 463 -> 400 us, of 8 x 131,072 with windows of four clocks 989 ->
+// 945 us, 8 x 65,536 factorisation cells 1190 -> 1129 us, 8 x 2^20 keys 2918 ->
+// 2873 us.
+template <class... P, class... A>
+inline void launch_on(bool follows, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
+                      cudaStream_t stream, const A&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(block);
+  c.dynamicSmemBytes = smem;
+  c.stream = stream;
+  c.attrs = &at;
+  c.numAttrs = follows ? 1 : 0;
+  cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+template <class... P, class... A>
+inline void launch_after(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream,
+                         const A&... args) {
+  launch_on(true, kernel, grid, block, smem, stream, args...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+#endif
+
 }  // namespace adapm

@@ -216,6 +216,7 @@ __device__ __forceinline__ uint32_t factor_row(const PushArgs& a, uint32_t pos) 
 // same ones of the accumulator half, so a gradient is loaded once for both.
 template <int G, int C, int R, int SRC>
 __global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_kernel(Store s, PushArgs a) {
+  after_previous();
   const PushWords pw = push_words(s, a);
   bool any_replica = false, resolved = false;
   constexpr int NG = kThreads / G;
@@ -569,6 +570,7 @@ __global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_k
 template <int G, int C>
 __global__ void __launch_bounds__(kThreads) push_combine_kernel(Store s, PushArgs a, uint64_t span,
                                                                 uint64_t nspans) {
+  after_previous();
   const PushWords pw = push_words(s, a);
   bool any_replica = false, resolved = false;
   constexpr int NG = kThreads / G;
@@ -671,10 +673,10 @@ void launch_push_source(const Store& s, const PushArgs& a, int sms, cudaStream_t
         cudaFuncSetAttribute(push_chunks_kernel<G, C, R, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
       }
-      push_chunks_kernel<G, C, R, SRC><<<(unsigned)spans, kThreads, smem, stream>>>(s, a);
+      launch_after(push_chunks_kernel<G, C, R, SRC>, (unsigned)spans, kThreads, smem, stream, s, a);
       if (spans > 1) {
         const unsigned grid = (unsigned)(spans < (uint64_t)sms * 8 ? spans : (uint64_t)sms * 8);
-        push_combine_kernel<G, C><<<grid, kThreads, 0, stream>>>(s, a, span, spans);
+        launch_after(push_combine_kernel<G, C>, grid, kThreads, 0, stream, s, a, span, spans);
       }
     }
   });

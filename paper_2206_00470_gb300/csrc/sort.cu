@@ -202,6 +202,7 @@ constexpr uint32_t kFusedBlocks = 32;
 
 template <bool POS, int ITEMS, int KIND>
 __global__ void __launch_bounds__(kSortThreads, 4) sort_kernel(SortArgs a) {
+  after_previous();
   constexpr int SUB = kSortThreads * ITEMS;   // keys per sub-tile
   __shared__ SortSmem sm;
   const int lane = threadIdx.x & 31;
@@ -575,6 +576,7 @@ struct MapSel {
 // tiles in no particular order: *count (zero before) hands out their places.
 __global__ void __launch_bounds__(kSortThreads) list_heads_kernel(const uint32_t* __restrict__ sk, uint64_t n,
                                                                   uint32_t* __restrict__ out, uint32_t* count) {
+  after_previous();
   __shared__ uint32_t sm[kWarps];
   __shared__ uint32_t base;
   const uint64_t start = (uint64_t)blockIdx.x * kTile + threadIdx.x;
@@ -717,13 +719,13 @@ cudaError_t launch_sort_phased(SortArgs& a, cudaStream_t stream) {
   for (int ph = 0; ph < phases; ++ph) {
     a.phase = ph;
     if (a.fused && ph > 0) {
-      if (!(ph & 1)) sort_kernel<POS, ITEMS, kSortScanScatter><<<(unsigned)B, kSortThreads, 0, stream>>>(a);
+      if (!(ph & 1)) launch_after(sort_kernel<POS, ITEMS, kSortScanScatter>, (unsigned)B, kSortThreads, 0, stream, a);
     } else if (ph == 0)
-      sort_kernel<POS, ITEMS, kSortCount><<<(unsigned)B, kSortThreads, 0, stream>>>(a);
+      sort_kernel<POS, ITEMS, kSortCount><<<(unsigned)B, kSortThreads, 0, stream>>>(a);   // (the stream has just waited)
     else if (ph & 1)
-      sort_kernel<POS, ITEMS, kSortScan><<<(unsigned)B, kSortThreads, 0, stream>>>(a);
+      launch_after(sort_kernel<POS, ITEMS, kSortScan>, (unsigned)B, kSortThreads, 0, stream, a);
     else
-      sort_kernel<POS, ITEMS, kSortScatter><<<(unsigned)B, kSortThreads, 0, stream>>>(a);
+      launch_after(sort_kernel<POS, ITEMS, kSortScatter>, (unsigned)B, kSortThreads, 0, stream, a);
   }
   return cudaGetLastError();
 }
@@ -827,7 +829,8 @@ void compact_replica_keys(const int32_t* map_w, uint64_t K, uint32_t* out, uint3
 void list_sorted_heads(const uint32_t* sk, uint64_t n, uint32_t* out, uint32_t* count, cudaStream_t stream) {
   if (n == 0) return;
   note_launches(1);
-  list_heads_kernel<<<(unsigned)((n + kTile - 1) / kTile), kSortThreads, 0, stream>>>(sk, n, out, count);
+  const unsigned grid = (unsigned)((n + kTile - 1) / kTile);
+  launch_after(list_heads_kernel, grid, kSortThreads, 0, stream, sk, n, out, count);
 }
 
 }  // namespace adapm

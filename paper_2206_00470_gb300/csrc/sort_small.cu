@@ -34,6 +34,7 @@ constexpr size_t small_smem() {
 
 template <int ITEMS>
 __global__ void __launch_bounds__(kThreadsS, 1) sort_small_kernel(SmallArgs sa) {
+  after_previous();
   const SmallSort& a = sa.a;
   extern __shared__ __align__(16) unsigned char dsm[];
   uint16_t(*wcnt)[kDigits] = reinterpret_cast<uint16_t(*)[kDigits]>(dsm);
@@ -175,7 +176,7 @@ cudaError_t launch(const SmallArgs& sa, cudaStream_t stream) {
     if (dev >= 0 && dev < 64) attr_set[dev] = true;
   }
   note_launches(1);
-  sort_small_kernel<ITEMS><<<1, kThreadsS, smem, stream>>>(sa);
+  launch_after(sort_small_kernel<ITEMS>, 1, kThreadsS, smem, stream, sa);
   return cudaGetLastError();
 }
 

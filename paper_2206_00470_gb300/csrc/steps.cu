@@ -174,6 +174,7 @@ __global__ void __launch_bounds__(kThreads)
 mf_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ rows, const uint32_t* __restrict__ cols,
                const float* __restrict__ vals, uint64_t n, uint32_t dim, int adagrad, float lr, float eps,
                StepOut o) {
+  after_previous();
   const int lane = threadIdx.x & (G - 1);
   constexpr int GPW = 32 / G;
   const int gi = (threadIdx.x & 31) / G;
@@ -314,6 +315,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, const uint32_t* __restrict__ rels,
                     const uint32_t* __restrict__ tails, const uint32_t* __restrict__ negs, uint64_t n,
                     uint32_t n_neg, uint32_t dim, StepOut o) {
+  after_previous();
   static_assert(16 % U == 0 && DEPTH <= 16 && U <= DEPTH, "see the batches' second half");
   extern __shared__ float4 ring_all[];
   const int lane = threadIdx.x & 31;
@@ -524,6 +526,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 sgns_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ centres, const uint32_t* __restrict__ contexts,
                  const uint32_t* __restrict__ negs, uint64_t n, uint32_t n_ctx, uint32_t n_neg, uint32_t vocab,
                  float lr, StepOut o) {
+  after_previous();
   static_assert(16 % U == 0 && DEPTH <= 16 && U <= DEPTH, "see the batches' second half");
   extern __shared__ float4 ring_all[];
   const int lane = threadIdx.x & 31;
@@ -716,13 +719,16 @@ void launch_mf_step(const Store& s, uint32_t w, const uint32_t* rows, const uint
   note_launches(1);
   const uint32_t dim4 = dim / 4;
   const int a = adagrad ? 1 : 0;
-  if (dim4 <= 4) mf_step_kernel<4, 1><<<grid, kThreads, 0, stream>>>(s, w, rows, cols, vals, n, dim, a, lr, eps, o);
-  else if (dim4 <= 8) mf_step_kernel<8, 1><<<grid, kThreads, 0, stream>>>(s, w, rows, cols, vals, n, dim, a, lr, eps, o);
-  else if (dim4 <= 16) mf_step_kernel<16, 1><<<grid, kThreads, 0, stream>>>(s, w, rows, cols, vals, n, dim, a, lr, eps, o);
-  else if (dim4 <= 32) mf_step_kernel<32, 1><<<grid, kThreads, 0, stream>>>(s, w, rows, cols, vals, n, dim, a, lr, eps, o);
-  else if (dim4 <= 64) mf_step_kernel<32, 2><<<grid, kThreads, 0, stream>>>(s, w, rows, cols, vals, n, dim, a, lr, eps, o);
-  else if (dim4 <= 128) mf_step_kernel<32, 4><<<grid, kThreads, 0, stream>>>(s, w, rows, cols, vals, n, dim, a, lr, eps, o);
-  else mf_step_kernel<32, 8><<<grid, kThreads, 0, stream>>>(s, w, rows, cols, vals, n, dim, a, lr, eps, o);
+  auto run = [&](auto kernel) {
+    launch_after(kernel, grid, kThreads, 0, stream, s, w, rows, cols, vals, n, dim, a, lr, eps, o);
+  };
+  if (dim4 <= 4) run(mf_step_kernel<4, 1>);
+  else if (dim4 <= 8) run(mf_step_kernel<8, 1>);
+  else if (dim4 <= 16) run(mf_step_kernel<16, 1>);
+  else if (dim4 <= 32) run(mf_step_kernel<32, 1>);
+  else if (dim4 <= 64) run(mf_step_kernel<32, 2>);
+  else if (dim4 <= 128) run(mf_step_kernel<32, 4>);
+  else run(mf_step_kernel<32, 8>);
 }
 
 void launch_complex_step(const Store& s, uint32_t w, const uint32_t* heads, const uint32_t* rels,
@@ -736,7 +742,8 @@ void launch_complex_step(const Store& s, uint32_t w, const uint32_t* heads, cons
     constexpr size_t smem = (size_t)kThreads * DEPTH * 2 * CC * sizeof(float4);
     static bool set[64] = {false};
     allow_smem(complex_step_kernel<CC, U, DEPTH>, smem, set);
-    complex_step_kernel<CC, U, DEPTH><<<grid, kThreads, smem, stream>>>(s, w, heads, rels, tails, negs, n, n_neg, dim, o);
+    launch_after(complex_step_kernel<CC, U, DEPTH>, grid, kThreads, smem, stream, s, w, heads, rels, tails, negs, n,
+                 n_neg, dim, o);
   };
   // ring depths: as many rows as two blocks' rings hold per SM (96 KB each)
   if (h4 <= 32) run(std::integral_constant<int, 1>{}, std::integral_constant<int, 4>{}, std::integral_constant<int, 12>{});
@@ -755,7 +762,8 @@ void launch_sgns_step(const Store& s, uint32_t w, const uint32_t* centres, const
     constexpr size_t smem = (size_t)kThreads * DEPTH * C * sizeof(float4);
     static bool set[64] = {false};
     allow_smem(sgns_step_kernel<C, U, DEPTH>, smem, set);
-    sgns_step_kernel<C, U, DEPTH><<<grid, kThreads, smem, stream>>>(s, w, centres, contexts, negs, n, n_ctx, n_neg, vocab, lr, o);
+    launch_after(sgns_step_kernel<C, U, DEPTH>, grid, kThreads, smem, stream, s, w, centres, contexts, negs, n, n_ctx,
+                 n_neg, vocab, lr, o);
   };
   // ring depths: as many rows as two blocks' rings hold per SM (96 KB each), 16 at most
   if (D4 <= 32) run(std::integral_constant<int, 1>{}, std::integral_constant<int, 4>{}, std::integral_constant<int, 16>{});

@@ -28,6 +28,7 @@ constexpr int pull_rows(int C) { return C == 1 ? 4 : (8 / C > 0 ? 8 / C : 1); }
 template <int G, int C, int R>
 __global__ void __launch_bounds__(kThreads, C == 1 ? 5 : 1)
 pull_kernel(Store s, int w, const uint32_t* __restrict__ keys, uint64_t n, float* __restrict__ out) {
+  after_previous();
   const int lane = threadIdx.x & (G - 1);
   const uint64_t g = group_id<G>(), ng = group_count<G>();
   const uint32_t D4 = s.D >> 2;
@@ -156,6 +157,7 @@ struct SyncSmem {
 
 template <int G, int C, bool VER>
 __global__ void __launch_bounds__(kThreads, C >= 8 ? 2 : 4) sync_kernel(Store s) {
+  after_previous();
   constexpr int R = 4 / C > 0 ? 4 / C : 1;
   constexpr uint32_t GW = 32 / G;   // row groups per warp
   __shared__ SyncSmem sm;
@@ -453,7 +455,7 @@ void launch_pull(const Store& s, int w, const uint32_t* keys, uint64_t n, float*
     constexpr int G = decltype(Gc)::value, C = decltype(Cc)::value;
     constexpr int R = pull_rows(C);
     note_launches(1);
-    pull_kernel<G, C, R><<<grid_for((n + R - 1) / R, G, sms), kThreads, 0, stream>>>(s, w, keys, n, out);
+    launch_after(pull_kernel<G, C, R>, grid_for((n + R - 1) / R, G, sms), kThreads, 0, stream, s, w, keys, n, out);
   });
 }
 
@@ -468,8 +470,8 @@ void launch_sync(const Store& s, uint64_t slot_bound, int sms, cudaStream_t stre
     const uint64_t resident = (uint64_t)sms * (C >= 8 ? 2 : 4);
     if (blocks > resident) blocks = resident;
     const unsigned grid = (unsigned)blocks;
-    if (s.dirty != nullptr) sync_kernel<G, C, true><<<grid, kThreads, 0, stream>>>(s);
-    else sync_kernel<G, C, false><<<grid, kThreads, 0, stream>>>(s);
+    if (s.dirty != nullptr) launch_after(sync_kernel<G, C, true>, grid, kThreads, 0, stream, s);
+    else launch_after(sync_kernel<G, C, false>, grid, kThreads, 0, stream, s);
   });
 }
 
