@@ -331,9 +331,9 @@ __global__ void events_kernel(Store s, uint32_t w, EventBatch eb, uint32_t* out_
 // worker joins or leaves a key, not both).
 //
 // Creating moves no row: the new replica is an alias of its main row (with
-// relocation, where it is a copy, copied.cu).  Of an evicted replica only pending updates move, main[k] += acc by vector atomic
-// adds, after the other holders' aliases of the old main row have got it as a
-// value of their own.
+// relocation, where it is a copy, copied.cu).  Of an evicted replica only
+// pending updates move, main[k] += acc by vector atomic adds, after the other
+// holders' aliases of the old main row have got it as a value of their own.
 //
 // What is done once per entry (list entries, owner records, holder masks,
 // map entries, the stack) is done by one lane per entry, a warp taking up to
@@ -345,7 +345,7 @@ __global__ void events_kernel(Store s, uint32_t w, EventBatch eb, uint32_t* out_
 // Bound by its random row and word accesses.  Measured per clock of 8
 // advances, copies made and moved by row groups before -> now: 198k replicas
 // of 64 floats destroyed and created each (100M keys) 833 -> 713 us, 366k of
-// 512 floats 5809 -> 4170 us, 27k of 200 floats 297 -> 270 us.
+// 512 floats 5809 -> 3980 us, 27k of 200 floats 297 -> 270 us.
 //
 // After early events (AdvCounts given) every block takes the list lengths
 // from the counters and the stack top from the store (the same values in

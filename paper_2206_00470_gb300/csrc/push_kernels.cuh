@@ -564,8 +564,9 @@ __global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_k
 
 // Segments that run past a span: the span where one begins owns it; its sum
 // is that span's tail piece plus the head pieces of the spans it continues
-// into (the spans whose first row holds the key, counted by the block).  The groups of the block take those head pieces in strides, in
-// increasing order, then group 0 adds the tail piece and the group sums in
+// into (the spans whose first row holds the key, counted by the block).  The
+// groups of the block take those head pieces in strides, in increasing order,
+// then group 0 adds the tail piece and the group sums in
 // group order: a fixed order, whatever the number of spans.
 template <int G, int C>
 __global__ void __launch_bounds__(kThreads) push_combine_kernel(Store s, PushArgs a, uint64_t span,

@@ -119,8 +119,8 @@ pull_kernel(Store s, int w, const uint32_t* __restrict__ keys, uint64_t n, float
 // sync
 // ---------------------------------------------------------------------------
 // Every replica is an alias of its main row afterwards (REP_ALIAS; with
-// relocation, where they are copies, copied.cu), so only pending rows move: main[k] += acc for every holder with updates, in
-// ascending worker order.  A warp scans the slots' owner words, up to 32 at a
+// relocation, where they are copies, copied.cu), so only pending rows move:
+// main[k] += acc for every holder with updates, in ascending worker order.  A warp scans the slots' owner words, up to 32 at a
 // time, and lists those with updates; replicas nobody touched since the last
 // sync cost their 8-byte word alone.  Once 32 are listed (or the scan ends)
 // one lane per listed slot looks up the key's holders, which of them merges
