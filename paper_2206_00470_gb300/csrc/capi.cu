@@ -680,7 +680,7 @@ adapm_status push_device(adapm_ctx* ctx, uint32_t w, const uint32_t* dkeys, uint
   CK(pool_alloc(ctx, &kb, n));
   CK(pool_alloc(ctx, &va, n));
   CK(pool_alloc(ctx, &vb, n));
-  CK(pool_alloc(ctx, &hist, sort_scratch_words(n)));
+  CK(pool_alloc(ctx, &hist, sort_scratch_words(n, ctx->bits, ctx->sms)));
   const uint64_t chunk = push_chunk_rows(ctx->s.D, n, ctx->sms);
   const uint64_t nchunks = (n + chunk - 1) / chunk;
   float* sparts = nullptr;
@@ -801,7 +801,7 @@ cudaError_t make_plan(adapm_ctx* ctx, IntentList& L, cudaEvent_t after) {
                                  reinterpret_cast<void**>(p));
   };
   if ((e = palloc(&tk, n)) != cudaSuccess || (e = palloc(&tv, n)) != cudaSuccess ||
-      (e = palloc(&hist, plan_scratch_words(n, ctx->bits))) != cudaSuccess)
+      (e = palloc(&hist, sort_scratch_words(n, ctx->bits, ctx->sms))) != cudaSuccess)
     return e;
   const bool odd = sort_passes(ctx->bits) % 2 == 1;   // the sort ends in ka / va after odd passes
   unsigned long long no_barriers = 0;

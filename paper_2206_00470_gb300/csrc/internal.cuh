@@ -233,7 +233,7 @@ __device__ __forceinline__ bool sort_failed(const DevState* st) {
 // ping-pong space of n keys; with va/vb non-null the positions 0..n-1
 // travel with the keys.  The sorted keys (and positions) end in the buffers
 // returned through *keys_out / *pos_out.  `scratch` holds
-// sort_scratch_words(n) uint32 words.  *bar_base is the host's copy of
+// sort_scratch_words(n, bits, sms) uint32 words.  *bar_base is the host's copy of
 // st->bar_arrivals, advanced by the launch.  clear0 / clear1 (may be null)
 // are device words the launch sets to zero before any later kernel on the
 // stream runs (counters of the consumer).  If a grid-barrier wait gives
@@ -252,10 +252,8 @@ __device__ __forceinline__ bool sort_failed(const DevState* st) {
 // of grid barriers, *bar_base untouched): for a stream that runs beside other
 // work, where a cooperative launch would wait for the whole GPU.  One for the
 // count and two per pass, or one per pass when the blocks are few enough that
-// each scans the digit table itself.  `scratch` then holds
-// plan_scratch_words(n, bits) words.
-size_t sort_scratch_words(uint64_t n);
-size_t plan_scratch_words(uint64_t n, int bits);
+// each scans the digit table itself.
+size_t sort_scratch_words(uint64_t n, int bits, int sms);
 int sort_passes(int bits);
 cudaError_t sort_keys(const uint32_t* raw, uint64_t n, uint64_t K, bool allow_nokey, int bits,
                       uint32_t* ka, uint32_t* kb, uint32_t* va, uint32_t* vb, uint32_t* scratch, int sms,

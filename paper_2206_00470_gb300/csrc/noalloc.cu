@@ -63,7 +63,7 @@ struct Layout {
   uint64_t chunk, nchunks;
 };
 
-Layout layout(uint32_t D, uint64_t n, int sms) {
+Layout layout(uint32_t D, uint64_t n, int bits, int sms) {
   Layout L{};
   L.chunk = adapm::push_chunk_rows(D, n, sms);
   L.nchunks = (n + L.chunk - 1) / L.chunk;
@@ -77,7 +77,7 @@ Layout layout(uint32_t D, uint64_t n, int sms) {
   L.kb = take(n * 4);
   L.va = take(n * 4);
   L.vb = take(n * 4);
-  L.hist = take(adapm::sort_scratch_words(n) * 4);
+  L.hist = take(adapm::sort_scratch_words(n, bits, sms) * 4);
   L.sparts = take(adapm::push_span_part_rows(L.nchunks) * D * 4);
   L.total = off;
   return L;
@@ -119,7 +119,7 @@ extern "C" adapm_status adapm_push_noalloc(adapm_ctx* ctx, uint32_t worker, cons
     ctx_set_error(ctx, "adapm_push_noalloc needs 16-byte aligned delta rows");
     return ADAPM_EINVAL;
   }
-  const Layout L = layout(v.s.D, n, v.sms);
+  const Layout L = layout(v.s.D, n, v.bits, v.sms);
   if (L.total > kScratchBytes) {
     char msg[160];
     snprintf(msg, sizeof msg,

@@ -680,17 +680,26 @@ int sort_blocks_per_sm() {
   return occ;
 }
 
+// Batches that would give fewer blocks than SMs take sub-tiles of half the
+// size: twice the blocks, half the ranking work per block.
+bool small_tiles(uint64_t n, int sms) { return (n + kSub - 1) / kSub < (uint64_t)sms; }
+// Blocks of a sort of n keys, one per sub-tile (a cooperative launch takes
+// fewer when they would not all be resident): the columns of its digit tables.
+uint64_t sort_blocks(uint64_t n, int sms) {
+  const uint64_t sub = small_tiles(n, sms) ? kSubMin : kSub;
+  const uint64_t B = (n + sub - 1) / sub;
+  return B < 1 ? 1 : (B > kMaxSortBlocks ? kMaxSortBlocks : B);
+}
+
 template <bool POS, int ITEMS>
 cudaError_t launch_sort(SortArgs& a, unsigned long long* bar_base, int sms, cudaStream_t stream) {
-  constexpr uint64_t SUB = (uint64_t)kSortThreads * ITEMS;
   const int occ = sort_blocks_per_sm<POS, ITEMS>();
-  uint64_t B = (a.n + SUB - 1) / SUB;
+  uint64_t B = sort_blocks(a.n, sms);
   // A launch that checks a plan expects it to match and only to check: one
   // block per SM needs room for one block on each SM, not four, before it can
   // start beside other streams' kernels (a miss then sorts with that grid).
   const uint64_t resident = (uint64_t)sms * (a.plan_keys ? 1 : (occ < 4 ? occ : 4));
   if (B > resident) B = resident;
-  if (B > kMaxSortBlocks) B = kMaxSortBlocks;
   if (B < 1) B = 1;
   a.bar_base = *bar_base;
   a.phase = -1;
@@ -707,11 +716,8 @@ cudaError_t launch_sort(SortArgs& a, unsigned long long* bar_base, int sms, cuda
 // the blocks need not be resident together (for a stream that runs beside
 // other work).  B = one block per sub-tile of keys.
 template <bool POS, int ITEMS>
-cudaError_t launch_sort_phased(SortArgs& a, cudaStream_t stream) {
-  constexpr uint64_t SUB = (uint64_t)kSortThreads * ITEMS;
-  uint64_t B = (a.n + SUB - 1) / SUB;
-  if (B > kMaxSortBlocks) B = kMaxSortBlocks;
-  if (B < 1) B = 1;
+cudaError_t launch_sort_phased(SortArgs& a, int sms, cudaStream_t stream) {
+  const uint64_t B = sort_blocks(a.n, sms);
   a.bar_base = 0;
   a.fused = B <= kFusedBlocks ? 1 : 0;
   const int phases = 1 + 2 * a.passes;
@@ -738,21 +744,12 @@ int bits_for(uint64_t num_keys) {
   return b;
 }
 
-size_t plan_scratch_words(uint64_t n, int bits) {
-  uint64_t rows = (n + kSubMin - 1) / kSubMin;
-  if (rows > kMaxSortBlocks) rows = kMaxSortBlocks;
-  if (rows < 1) rows = 1;
-  // totals, and two tables or (few blocks) one per pass
+size_t sort_scratch_words(uint64_t n, int bits, int sms) {
+  const uint64_t rows = sort_blocks(n, sms);
+  // totals, and two tables or (phased, few blocks) one per pass
   uint64_t columns = (uint64_t)plan_for(bits).passes * (rows < kFusedBlocks ? rows : kFusedBlocks);
   if (columns < 2 * rows) columns = 2 * rows;
   return (size_t)(kScratchHead + kDigits + columns * kDigits);
-}
-
-size_t sort_scratch_words(uint64_t n) {
-  uint64_t rows = (n + kSubMin - 1) / kSubMin;
-  if (rows > kMaxSortBlocks) rows = kMaxSortBlocks;
-  if (rows < 1) rows = 1;
-  return (size_t)(kScratchHead + kDigits + 2 * rows * kDigits);   // totals, two tables
 }
 
 int sort_passes(int bits) { return plan_for(bits).passes; }
@@ -807,12 +804,10 @@ cudaError_t sort_keys(const uint32_t* raw, uint64_t n, uint64_t K, bool allow_no
   a.passes = pl.passes;
   a.per = pl.per;
   a.bits = bits;
-  // batches that would give fewer blocks than SMs take sub-tiles of half the
-  // size: twice the blocks, half the ranking work per block
-  const bool small = (n + kSub - 1) / kSub < (uint64_t)sms;
+  const bool small = small_tiles(n, sms);
   if (phased) {
-    if (small) return va ? launch_sort_phased<true, 4>(a, stream) : launch_sort_phased<false, 4>(a, stream);
-    return va ? launch_sort_phased<true, kItems>(a, stream) : launch_sort_phased<false, kItems>(a, stream);
+    if (small) return va ? launch_sort_phased<true, 4>(a, sms, stream) : launch_sort_phased<false, 4>(a, sms, stream);
+    return va ? launch_sort_phased<true, kItems>(a, sms, stream) : launch_sort_phased<false, kItems>(a, sms, stream);
   }
   if (small)
     return va ? launch_sort<true, 4>(a, bar_base, sms, stream) : launch_sort<false, 4>(a, bar_base, sms, stream);

@@ -99,7 +99,7 @@ def test_push_noalloc_rejects_what_it_cannot_serve(gpu_lib):
     with pytest.raises(A.AdaPMError) as e:
         pm.push_noalloc(0, np.array([1, 2]), np.zeros((2, D), np.float32))
     assert e.value.status == A.EINVAL
-    # more rows than the 16 MiB scratch holds (about 790k at value_len 64)
+    # more rows than the 16 MiB scratch holds (about 880k at value_len 64)
     n = 900000
     with pytest.raises(A.AdaPMError) as e:
         pm.push_noalloc(0, torch.zeros(n, dtype=torch.int32, device="cuda"),
