@@ -252,7 +252,8 @@ adapm_status adapm_wait(adapm_ctx* ctx);
  * valid after adapm_wait(). */
 
 /* Matrix factorisation, loss 1/2 (v - u.w)^2 per cell (App. C "Matrix
- * factorization"): row_keys[i], col_keys[i], vals[i] for i < n. */
+ * factorization"): row_keys[i], col_keys[i], vals[i] for i < n.  With AdaGrad
+ * dim is a multiple of 4 (ADAPM_EINVAL otherwise). */
 adapm_status adapm_mf_step(adapm_ctx* ctx, uint32_t worker, const uint32_t* row_keys,
                            const uint32_t* col_keys, const float* vals, uint64_t n,
                            uint32_t dim, int adagrad, float lr, float eps, double* loss_out);
@@ -260,7 +261,8 @@ adapm_status adapm_mf_step(adapm_ctx* ctx, uint32_t worker, const uint32_t* row_
 /* ComplEx knowledge-graph embeddings with logistic loss (App. C "Knowledge
  * graph embeddings"): rows [re(dim/2) | im(dim/2)] (+ AdaGrad), score
  * Re(sum h r conj(t)); per triple i: heads[i], rels[i], tails[i] positive and
- * neg_tails[i*n_neg + j] negative (label -1).  AdaGrad always (D = 2*dim). */
+ * neg_tails[i*n_neg + j] negative (label -1).  AdaGrad always (D = 2*dim);
+ * dim is a multiple of 8 (ADAPM_EINVAL otherwise). */
 adapm_status adapm_complex_step(adapm_ctx* ctx, uint32_t worker, const uint32_t* heads,
                                 const uint32_t* rels, const uint32_t* tails,
                                 const uint32_t* neg_tails, uint64_t n, uint32_t n_neg,

@@ -1316,6 +1316,8 @@ adapm_status adapm_mf_step(adapm_ctx* ctx, uint32_t worker, const uint32_t* row_
     return fail(ctx, ADAPM_EINVAL, "bad pointers/n");
   if (dim == 0 || (adagrad ? 2 * dim : dim) != ctx->s.D)
     return fail(ctx, ADAPM_EINVAL, "dim %u does not match value_len %u", dim, ctx->s.D);
+  // (theta and accumulators are read and written as float4 halves of a row)
+  if (adagrad && dim % 4 != 0) return fail(ctx, ADAPM_EINVAL, "dim %u: need a multiple of 4 with AdaGrad", dim);
   Output<double> lo;
   if (loss_out) CK(stage_out(ctx, loss_out, 1, &lo));
   if (n == 0) {
@@ -1372,8 +1374,9 @@ adapm_status adapm_complex_step(adapm_ctx* ctx, uint32_t worker, const uint32_t*
   if (n > kMaxN / (3 + (uint64_t)n_neg) ||
       (n > 0 && (!heads || !rels || !tails || (n_neg > 0 && !neg_tails))))
     return fail(ctx, ADAPM_EINVAL, "bad pointers/n");
-  if (dim == 0 || dim % 2 != 0 || 2 * dim != ctx->s.D)
-    return fail(ctx, ADAPM_EINVAL, "dim %u: need even dim with value_len = 2*dim", dim);
+  // (re and im parts are read and written as float4 quarters of a row)
+  if (dim == 0 || dim % 8 != 0 || 2 * dim != ctx->s.D)
+    return fail(ctx, ADAPM_EINVAL, "dim %u: need a multiple of 8 with value_len = 2*dim", dim);
   Output<double> lo;
   if (loss_out) CK(stage_out(ctx, loss_out, 1, &lo));
   if (n == 0) {
