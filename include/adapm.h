@@ -43,6 +43,16 @@
  *     barriers, and a barrier wait is limited.  Work enqueued after such a failure does not
  *     touch the store, and the context is unusable afterwards (destroy it).
  *   - ADAPM_ECUDA reports a CUDA runtime error; the context is then unusable.
+ *   - Stream capture.  While the library stream records a CUDA graph, calls
+ *     with device (or pinned host) arrays that pull, push (adapm_push_noalloc
+ *     too), take a training step or sync are recorded, and every launch of the
+ *     graph repeats them on the arrays and state it finds; such pushes use no
+ *     push plan.
+ *     adapm_intent, adapm_advance_clock and (with ADAPM_ACT_ADAPTIVE)
+ *     adapm_sync move the host's clocks and intents, which a launch cannot
+ *     repeat: they return ADAPM_EINVAL and change nothing.  Make the first
+ *     call on a device before a capture.  Counts kept on the host (push_rows
+ *     of adapm_stats) count a recorded call once.
  *   - No C++ exception crosses the ABI.  A context is driven by one host
  *     thread at a time.
  */

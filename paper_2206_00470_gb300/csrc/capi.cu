@@ -45,7 +45,9 @@ class BlockCache {
  public:
   // capturing: the stream records a graph.  Its blocks come from the pool and
   // go back to it inside the graph (a kept block would outlive its allocation
-  // node, or be handed to other work while the graph runs).
+  // node, or be handed to other work while the graph runs).  What a recorded
+  // call gives back it took itself: blocks that outlive a call are an intent's,
+  // and intents and advances are refused then (refuse_capture).
   cudaError_t take(cudaMemPool_t pool, cudaStream_t stream, size_t bytes, bool capturing, void** p) {
     const bool keep = bytes <= kLargest && !capturing;
     const size_t size = keep ? round_up(bytes) : bytes;
@@ -378,7 +380,7 @@ cudaError_t stage_in(adapm_ctx* ctx, const T* p, size_t count, Input<T>* in) {
     return cudaSuccess;
   }
   const uint64_t bytes = count * sizeof(T);
-  if (kind == MemKind::PinnedHost) {
+  if (kind == MemKind::PinnedHost && !ctx->capturing) {   // (a graph records its copies on `stream`)
     cudaError_t e = ensure_copy_in(ctx);
     if (e == cudaSuccess) e = stage_mark(ctx, bytes);
     if (e != cudaSuccess) return e;
@@ -475,6 +477,18 @@ adapm_status check_ctx(adapm_ctx* ctx) {
   return ADAPM_OK;
 }
 
+// While the stream records a graph, calls whose work every launch of the
+// graph can repeat are recorded: pulls, pushes, steps and syncs, all of whose
+// state is on the device.  They take no push plan, start no early events and
+// sort without grid barriers (early_make, find_plan, ctx_sort_phased): the
+// host numbers plan checks and barrier arrivals per call, and side streams
+// would join the capture.  Calls that move the host's clocks and intent lists
+// cannot be repeated and are refused.
+adapm_status refuse_capture(adapm_ctx* ctx, const char* what) {
+  if (!ctx->capturing) return ADAPM_OK;
+  return fail(ctx, ADAPM_EINVAL, "%s cannot be recorded in a graph: it moves the manager's clocks or intents", what);
+}
+
 constexpr uint64_t kMaxN = 1ull << 31;
 // Keys of an intent that one block sorts (8 x 8000 keys per clock: 474 us so,
 // 441 us with the phased sort; 8 x 4000: 397 us, 519 us).
@@ -541,7 +555,7 @@ std::vector<EventList> event_lists(adapm_ctx* ctx, const std::vector<int64_t>& o
 
 adapm_status early_make(adapm_ctx* ctx, uint32_t w) {
   WorkerState& ws = ctx->workers[w];
-  if (!early_enabled(ctx) || ws.early.active) return ADAPM_OK;
+  if (!early_enabled(ctx) || ws.early.active || ctx->capturing) return ADAPM_OK;
   WorkerState::Early E;
   E.clock = ws.clock + 1;
   advance_lists(ws, E.clock, E.open, E.close);
@@ -633,6 +647,7 @@ adapm_status apply_events(adapm_ctx* ctx, uint32_t w, const std::vector<EventLis
 // The plan a push of n keys by worker w may use: the newest recorded intent
 // of w with n keys whose window (as signalled) holds the worker's clock.
 IntentList* find_plan(adapm_ctx* ctx, uint32_t w, uint64_t n) {
+  if (ctx->capturing) return nullptr;
   WorkerState& ws = ctx->workers[w];
   for (auto it = ws.order.rbegin(); it != ws.order.rend(); ++it) {
     IntentList& L = ctx->lists[*it];
@@ -689,7 +704,8 @@ adapm_status push_device(adapm_ctx* ctx, uint32_t w, const uint32_t* dkeys, uint
   uint32_t *sk = nullptr, *sp = nullptr;
   CK(sort_keys(dkeys, n, ctx->s.K, allow_nokey, ctx->bits, ka, kb, va, vb, hist, ctx->sms, ctx->dstate,
                &ctx->bar_base, &ctx->dstate->last_unique, nullptr, ctx->stream, &sk, &sp,
-               plan ? plan->px : nullptr, plan ? &ctx->dstate->plan_miss : nullptr, seq));
+               plan ? plan->px : nullptr, plan ? &ctx->dstate->plan_miss : nullptr, seq,
+               ctx_sort_phased(ctx, n)));
   ctx->push_rows_host += n;
   PushArgs a = source;
   a.skeys = sk;
@@ -863,6 +879,8 @@ void adapm::ctx_set_error(adapm_ctx* ctx, const char* msg) {
 void adapm::ctx_add_push_rows(adapm_ctx* ctx, uint64_t n) {
   if (ctx) ctx->push_rows_host += n;
 }
+
+bool adapm::ctx_sort_phased(adapm_ctx* ctx, uint64_t n) { return ctx->capturing && n > kSmallSort; }
 
 int adapm::ctx_begin(adapm_ctx* ctx) { return check_ctx(ctx); }
 
@@ -1042,6 +1060,8 @@ adapm_status adapm_intent(adapm_ctx* ctx, uint32_t worker, const uint32_t* keys,
   if (st != ADAPM_OK) return st;
   if (worker >= ctx->s.W) return fail(ctx, ADAPM_EINVAL, "worker %u >= %u", worker, ctx->s.W);
   if (n > kMaxN || (n > 0 && !keys)) return fail(ctx, ADAPM_EINVAL, "bad keys/n");
+  st = refuse_capture(ctx, "an intent");
+  if (st != ADAPM_OK) return st;
   WorkerState& ws = ctx->workers[worker];
   if (clock_end <= clock_start || clock_end <= ws.clock) return ADAPM_OK;   // never active
   const int64_t signalled_start = clock_start;
@@ -1146,6 +1166,8 @@ adapm_status adapm_advance_clock(adapm_ctx* ctx, uint32_t worker) {
   adapm_status st = check_ctx(ctx);
   if (st != ADAPM_OK) return st;
   if (worker >= ctx->s.W) return fail(ctx, ADAPM_EINVAL, "worker %u >= %u", worker, ctx->s.W);
+  st = refuse_capture(ctx, "an advance");
+  if (st != ADAPM_OK) return st;
   WorkerState& ws = ctx->workers[worker];
   ws.clock += 1;
   const int64_t c = ws.clock;
@@ -1254,6 +1276,8 @@ adapm_status adapm_push(adapm_ctx* ctx, uint32_t worker, const uint32_t* keys, u
 
 adapm_status adapm_sync(adapm_ctx* ctx) {
   adapm_status st = check_ctx(ctx);
+  if (st != ADAPM_OK) return st;
+  if (ctx->cfg.action_timing == ADAPM_ACT_ADAPTIVE) st = refuse_capture(ctx, "a sync with adaptive action timing");
   if (st != ADAPM_OK) return st;
   {
     ProfScope ps(ctx, 4);

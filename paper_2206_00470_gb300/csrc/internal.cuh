@@ -324,6 +324,10 @@ void ctx_add_push_rows(struct ::adapm_ctx* ctx, uint64_t n);
 // null, ADAPM_ECUDA once it is unusable), its last error cleared, its device
 // current.  Returns an adapm_status value (0 = ADAPM_OK).
 int ctx_begin(struct ::adapm_ctx* ctx);
+// Whether a push of n keys sorts in ordinary launches: its stream records a
+// graph (the grid barriers' arrival count is the host's, per launch) and the
+// keys are too many for one block.
+bool ctx_sort_phased(struct ::adapm_ctx* ctx, uint64_t n);
 // A CUDA runtime error: records "where: message", marks the context unusable
 // (as every entry point does) and returns ADAPM_ECUDA.
 int ctx_fail_cuda(struct ::adapm_ctx* ctx, cudaError_t e, const char* where);
