@@ -360,8 +360,8 @@ constexpr int evict_blocks_per_sm(int C) { return C >= 8 ? 2 : 4; }
 
 template <int G, int C>
 __global__ void __launch_bounds__(kThreads, evict_blocks_per_sm(C)) evict_create_kernel(Store s, uint32_t w,
-                                                                              const uint32_t* __restrict__ evict_list,
-                                                                              const uint32_t* __restrict__ create_list,
+                                                                              const uint32_t* evict_list,
+                                                                              const uint32_t* create_list,
                                                                               AdvCounts* early) {
   after_previous();
   constexpr int R = C == 3 || C == 4 ? 2 : (4 / C > 0 ? 4 / C : 1);
@@ -568,14 +568,14 @@ __global__ void events_undo_kernel(Store s, uint32_t w, EventBatch eb, int sign)
 // kernel: a device-to-device copy and a clearing of the count are two
 // operations of the copy path, whose hand-over the next kernel waits for.
 __global__ void __launch_bounds__(kThreads)
-copy_keys_kernel(const uint32_t* __restrict__ keys, uint64_t n, uint32_t* __restrict__ out, uint32_t* zero) {
+copy_keys_kernel(const uint32_t* keys, uint64_t n, uint32_t* __restrict__ out, uint32_t* zero) {
   after_previous();
   if (zero && blockIdx.x == 0 && threadIdx.x == 0) *zero = 0;
   const uint64_t i = 4 * ((uint64_t)blockIdx.x * kThreads + threadIdx.x);
   if (i + 4 <= n && (reinterpret_cast<uintptr_t>(keys) & 15) == 0) {   // out is the library's own: aligned
-    reinterpret_cast<uint4*>(out)[i / 4] = __ldg(reinterpret_cast<const uint4*>(keys) + i / 4);
+    reinterpret_cast<uint4*>(out)[i / 4] = reinterpret_cast<const uint4*>(keys)[i / 4];
   } else {
-    for (uint64_t j = i; j < i + 4 && j < n; ++j) out[j] = __ldg(keys + j);
+    for (uint64_t j = i; j < i + 4 && j < n; ++j) out[j] = keys[j];
   }
 }
 

@@ -30,8 +30,8 @@ namespace {
 // go out together with the next round's list entries.
 template <int G, int C>
 __global__ void __launch_bounds__(kThreads, C >= 8 ? 2 : 3) evict_create_copied_kernel(Store s, uint32_t w,
-                                                                                     const uint32_t* __restrict__ evict_list,
-                                                                                     const uint32_t* __restrict__ create_list) {
+                                                                                     const uint32_t* evict_list,
+                                                                                     const uint32_t* create_list) {
   after_previous();
   constexpr int R = 4 / C > 0 ? 4 / C : 1;
   const int lane = threadIdx.x & (G - 1);

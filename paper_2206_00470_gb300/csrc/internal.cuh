@@ -352,7 +352,12 @@ void ctx_prof_stop(struct ::adapm_ctx* ctx, ProfToken& t);
 // before it is final), and its first statement, after_previous(), waits until
 // the other's writes are visible.  Every block makes that wait, so a kernel
 // ends after all before it on the stream have, and a kernel or event that
-// follows sees them too.  A kernel that a stream runs right after a wait for
+// follows sees them too.  Such a kernel runs from before the other's last
+// writes, so it reads with plain loads alone: __ldg and const __restrict__
+// parameters promise data that does not change while the kernel runs, and need
+// not stay behind the wait.  (Plain loads in their place: between 0.998 and
+// 1.02 times as fast over the timed cases.)
+// A kernel that a stream runs right after a wait for
 // another stream has nothing to overlap and is launched plainly (the
 // attribute costs the host more than it gives: follows = false).
 //

@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_k
           if (seg_begin) ++heads;
           // (AdaGrad sources: also where the accumulators of a piece's first row are)
           if ((f[u] & 7) == 7 || (SRC == kSrcAda && (f[u] & 8))) e[u] = s.map[(uint64_t)a.worker * s.K + k];
-          if (SRC != kSrcRows) coef[u] = __ldg(a.coef + sp[i]);
+          if (SRC != kSrcRows) coef[u] = a.coef[sp[i]];
         } else if (k != kNoKey || sp[i] >= a.n) {
           set_error(s.st, ERR_INTERNAL);
         }
@@ -392,14 +392,14 @@ __global__ void __launch_bounds__(kThreads, push_blocks_per_sm(C)) push_chunks_k
 #pragma unroll
           for (int c = 0; c < C; ++c) {
             const uint32_t col = lane + c * G;
-            d[r][c] = ((f[r] & 16) && col < D4) ? __ldg(d4 + (uint64_t)src * D4 + col) : f4zero();
+            d[r][c] = ((f[r] & 16) && col < D4) ? d4[(uint64_t)src * D4 + col] : f4zero();
           }
         } else {
           // gradient factor, and (where a piece begins) the key's accumulators
 #pragma unroll
           for (int c = 0; c < C / 2; ++c) {
             const uint32_t q = lane + c * G;
-            d[r][c] = ((f[r] & 16) && q < T4) ? __ldg(d4 + (uint64_t)src * T4 + q) : f4zero();
+            d[r][c] = ((f[r] & 16) && q < T4) ? d4[(uint64_t)src * T4 + q] : f4zero();
           }
           if (f[r] & 8) {
             const uint32_t state = f[r] >> 5;

@@ -143,7 +143,7 @@ __device__ __forceinline__ void load_rank(const SortArgs& a, const uint32_t* kin
     uint32_t k = 0;
     if (valid) {
       if (first) {
-        k = __ldg(kin + i);
+        k = kin[i];
         if (k >= a.K) {
           if (!(a.allow_nokey && k == kNoKey)) bad = true;
           k = kNoKey;
@@ -232,8 +232,8 @@ __global__ void __launch_bounds__(kSortThreads, 4) sort_kernel(SortArgs a) {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const uint64_t i = i0 + u * stride;
-        kv[u] = i < a.n ? __ldg(a.raw + i) : 0u;
-        xv[u] = i < a.n ? __ldg(a.plan_keys + i) : 0u;
+        kv[u] = i < a.n ? a.raw[i] : 0u;
+        xv[u] = i < a.n ? a.plan_keys[i] : 0u;
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) sort_kernel(SortArgs a) {
 #pragma unroll
         for (int it = 0; it < ITEMS; ++it) {
           const uint64_t i = i0 + (uint64_t)it * kSortThreads;
-          kk[it] = i < c1 ? __ldg(kin + i) : 0u;
+          kk[it] = i < c1 ? kin[i] : 0u;
         }
 #pragma unroll
         for (int it = 0; it < ITEMS; ++it) {
@@ -574,7 +574,7 @@ struct MapSel {
 
 // The first copy of every valid key of a sorted array, a tile per block, the
 // tiles in no particular order: *count (zero before) hands out their places.
-__global__ void __launch_bounds__(kSortThreads) list_heads_kernel(const uint32_t* __restrict__ sk, uint64_t n,
+__global__ void __launch_bounds__(kSortThreads) list_heads_kernel(const uint32_t* sk, uint64_t n,
                                                                   uint32_t* __restrict__ out, uint32_t* count) {
   after_previous();
   __shared__ uint32_t sm[kWarps];

@@ -54,14 +54,14 @@ __global__ void __launch_bounds__(kThreadsS, 1) sort_small_kernel(SmallArgs sa) 
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
     const uint32_t i = (uint32_t)((warp * ITEMS + it) * 32 + lane);
-    key[it] = i < a.n ? __ldg(a.raw + i) : kNoKey;
+    key[it] = i < a.n ? a.raw[i] : kNoKey;
     pos[it] = i;
   }
   if (a.plan_keys) {
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
       if (pos[it] >= a.n) continue;
-      const uint32_t x = __ldg(a.plan_keys + pos[it]);
+      const uint32_t x = a.plan_keys[pos[it]];
       miss |= (key[it] < a.K ? key[it] : kNoKey) != (x < a.K ? x : kNoKey);
     }
   }

@@ -171,8 +171,8 @@ __device__ void block_loss(double v, const StepOut& o) {
 // the resident warps (step 395 -> 587 us).
 template <int G, int C>
 __global__ void __launch_bounds__(kThreads)
-mf_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ rows, const uint32_t* __restrict__ cols,
-               const float* __restrict__ vals, uint64_t n, uint32_t dim, int adagrad, float lr, float eps,
+mf_step_kernel(Store s, uint32_t w, const uint32_t* rows, const uint32_t* cols,
+               const float* vals, uint64_t n, uint32_t dim, int adagrad, float lr, float eps,
                StepOut o) {
   after_previous();
   const int lane = threadIdx.x & (G - 1);
@@ -312,8 +312,8 @@ __device__ __forceinline__ void copy_wait() {   // all but the last N groups hav
 // ---------------------------------------------------------------------------
 template <int CC, int U, int DEPTH>
 __global__ void __launch_bounds__(kThreads, 2)
-complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, const uint32_t* __restrict__ rels,
-                    const uint32_t* __restrict__ tails, const uint32_t* __restrict__ negs, uint64_t n,
+complex_step_kernel(Store s, uint32_t w, const uint32_t* heads, const uint32_t* rels,
+                    const uint32_t* tails, const uint32_t* negs, uint64_t n,
                     uint32_t n_neg, uint32_t dim, StepOut o) {
   after_previous();
   static_assert(16 % U == 0 && DEPTH <= 16 && U <= DEPTH, "see the batches' second half");
@@ -523,8 +523,8 @@ complex_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ heads, con
 // ---------------------------------------------------------------------------
 template <int C, int U, int DEPTH>
 __global__ void __launch_bounds__(kThreads, 2)
-sgns_step_kernel(Store s, uint32_t w, const uint32_t* __restrict__ centres, const uint32_t* __restrict__ contexts,
-                 const uint32_t* __restrict__ negs, uint64_t n, uint32_t n_ctx, uint32_t n_neg, uint32_t vocab,
+sgns_step_kernel(Store s, uint32_t w, const uint32_t* centres, const uint32_t* contexts,
+                 const uint32_t* negs, uint64_t n, uint32_t n_ctx, uint32_t n_neg, uint32_t vocab,
                  float lr, StepOut o) {
   after_previous();
   static_assert(16 % U == 0 && DEPTH <= 16 && U <= DEPTH, "see the batches' second half");

@@ -27,7 +27,7 @@ constexpr int pull_rows(int C) { return C == 1 ? 4 : (8 / C > 0 ? 8 / C : 1); }
 
 template <int G, int C, int R>
 __global__ void __launch_bounds__(kThreads, C == 1 ? 5 : 1)
-pull_kernel(Store s, int w, const uint32_t* __restrict__ keys, uint64_t n, float* __restrict__ out) {
+pull_kernel(Store s, int w, const uint32_t* keys, uint64_t n, float* __restrict__ out) {
   after_previous();
   const int lane = threadIdx.x & (G - 1);
   const uint64_t g = group_id<G>(), ng = group_count<G>();
@@ -41,11 +41,11 @@ pull_kernel(Store s, int w, const uint32_t* __restrict__ keys, uint64_t n, float
   bool bad = false;
   auto load_keys = [&](uint64_t b, uint32_t (&k)[R]) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) k[r] = b + r < n ? __ldg(keys + b + r) : kNoKey;
+    for (int r = 0; r < R; ++r) k[r] = b + r < n ? keys[b + r] : kNoKey;
   };
   auto load_slots = [&](const uint32_t (&k)[R], int32_t (&sl)[R]) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) sl[r] = (mapw != nullptr && k[r] < s.K) ? __ldg(mapw + k[r]) : -1;
+    for (int r = 0; r < R; ++r) sl[r] = (mapw != nullptr && k[r] < s.K) ? mapw[k[r]] : -1;
   };
   uint64_t base = g * R;
   uint32_t k0[R], k1[R];
@@ -79,7 +79,7 @@ pull_kernel(Store s, int w, const uint32_t* __restrict__ keys, uint64_t n, float
     for (int c = 0; c < C; ++c) {
       const uint32_t col = lane + c * G;
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[r][c] = (src[r] != nullptr && col < D4) ? __ldg(src[r] + col) : f4zero();
+      for (int r = 0; r < R; ++r) v[r][c] = (src[r] != nullptr && col < D4) ? src[r][col] : f4zero();
     }
     if (sums) {
       const float4* acc4 = reinterpret_cast<const float4*>(s.acc);
@@ -89,7 +89,7 @@ pull_kernel(Store s, int w, const uint32_t* __restrict__ keys, uint64_t n, float
 #pragma unroll
           for (int c = 0; c < C; ++c) {
             const uint32_t col = lane + c * G;
-            if (col < D4) v[r][c] = f4add(v[r][c], __ldg(acc4 + (uint64_t)map_slot(sl0[r]) * D4 + col));
+            if (col < D4) v[r][c] = f4add(v[r][c], acc4[(uint64_t)map_slot(sl0[r]) * D4 + col]);
           }
     }
     // next round's slots and the keys of the round after
