@@ -16,10 +16,10 @@
 #include <new>
 #include <string>
 #include <tuple>
-#include <unordered_map>
 #include <vector>
 
 #include "adapm.h"
+#include "blocks.h"
 #include "internal.cuh"
 #include "store_launch.cuh"
 
@@ -33,72 +33,16 @@ void adapm::note_launches(uint64_t n) { g_launches.fetch_add(n, std::memory_orde
 
 namespace {
 
-// Scratch blocks kept for reuse on one stream: a block given back is handed
-// out again to later work of the same stream, whose order makes that safe
-// (what other streams do with a block is waited for before it is given back).
-// Taking and giving back are host bookkeeping, where a pool allocation and
-// its free are two calls into the driver (0.7 to 1 us each, six pairs a push).
-// Sizes are rounded up to one of four steps per power of two.  Blocks above
-// kLargest are not kept, and not more than kKeep bytes in all; the rest goes
-// back to the pool, which the context owns and destroys.
-class BlockCache {
- public:
-  // capturing: the stream records a graph.  Its blocks come from the pool and
-  // go back to it inside the graph (a kept block would outlive its allocation
-  // node, or be handed to other work while the graph runs).  What a recorded
-  // call gives back it took itself: blocks that outlive a call are an intent's,
-  // and intents and advances are refused then (refuse_capture).
-  cudaError_t take(cudaMemPool_t pool, cudaStream_t stream, size_t bytes, bool capturing, void** p) {
-    const bool keep = bytes <= kLargest && !capturing;
-    const size_t size = keep ? round_up(bytes) : bytes;
-    auto it = keep ? free_.find(size) : free_.end();
-    if (it != free_.end() && !it->second.empty()) {
-      *p = it->second.back();
-      it->second.pop_back();
-      kept_ -= size;
-      return cudaSuccess;
-    }
-    const cudaError_t e = cudaMallocFromPoolAsync(p, size, pool, stream);
-    if (e == cudaSuccess && keep) {
-      try {
-        size_[*p] = size;
-      } catch (...) {   // no host memory to remember it by: given back like any other
-      }
-    }
-    return e;
+// The pool behind a cache of scratch blocks, on the cache's stream.
+struct PoolMem {
+  cudaMemPool_t pool;
+  cudaStream_t stream;
+  int alloc(void** p, size_t bytes) {
+    const cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, stream);
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();   // tried again, or returned to the caller
+    return (int)e;
   }
-  void give(void* p, cudaStream_t stream) {
-    auto it = size_.find(p);
-    if (it != size_.end() && kept_ + it->second <= kKeep) {
-      try {
-        free_[it->second].push_back(p);
-        kept_ += it->second;
-        return;
-      } catch (...) {
-      }
-    }
-    if (it != size_.end()) size_.erase(it);
-    cudaFreeAsync(p, stream);
-  }
-  void release() {   // the stream is idle
-    for (auto& f : free_)
-      for (void* p : f.second) cudaFree(p);
-    free_.clear();
-    size_.clear();
-    kept_ = 0;
-  }
-
- private:
-  static constexpr size_t kLargest = 64u << 20, kKeep = 512u << 20;
-  static size_t round_up(size_t bytes) {
-    if (bytes <= 1024) return 1024;
-    size_t step = 256;
-    while (step * 8 < bytes) step <<= 1;   // four steps between 4 * step and 8 * step
-    return (bytes + step - 1) / step * step;
-  }
-  std::unordered_map<size_t, std::vector<void*>> free_;
-  std::unordered_map<void*, size_t> size_;
-  size_t kept_ = 0;
+  void free(void* p) { cudaFreeAsync(p, stream); }
 };
 
 struct IntentList {
@@ -354,11 +298,12 @@ cudaError_t stage_mark(adapm_ctx* ctx, uint64_t next_bytes) {
 template <class T>
 cudaError_t pool_alloc(adapm_ctx* ctx, T** p, size_t count) {
   if (count == 0) count = 1;
-  return ctx->blocks.take(ctx->pool, ctx->stream, count * sizeof(T), ctx->capturing, reinterpret_cast<void**>(p));
+  return (cudaError_t)ctx->blocks.take(PoolMem{ctx->pool, ctx->stream}, count * sizeof(T), ctx->capturing,
+                                       reinterpret_cast<void**>(p));
 }
 
 void pool_free(adapm_ctx* ctx, void* p) {
-  if (p) ctx->blocks.give(p, ctx->stream);
+  if (p) ctx->blocks.give(PoolMem{ctx->pool, ctx->stream}, p);
 }
 
 // Device view of an input array; copies host arrays in.
@@ -812,9 +757,10 @@ cudaError_t make_plan(adapm_ctx* ctx, IntentList& L, cudaEvent_t after) {
     return cudaEventRecord(L.ready, ps);
   }
   uint32_t *tk = nullptr, *tv = nullptr, *hist = nullptr;
+  const PoolMem plan_mem{ctx->plan_pool, ps};
   auto palloc = [&](uint32_t** p, size_t words) {
-    return ctx->plan_blocks.take(ctx->plan_pool, ps, (words ? words : 1) * sizeof(uint32_t), ctx->capturing,
-                                 reinterpret_cast<void**>(p));
+    return (cudaError_t)ctx->plan_blocks.take(plan_mem, (words ? words : 1) * sizeof(uint32_t), false,
+                                              reinterpret_cast<void**>(p));
   };
   if ((e = palloc(&tk, n)) != cudaSuccess || (e = palloc(&tv, n)) != cudaSuccess ||
       (e = palloc(&hist, sort_scratch_words(n, ctx->bits, ctx->sms))) != cudaSuccess)
@@ -827,7 +773,7 @@ cudaError_t make_plan(adapm_ctx* ctx, IntentList& L, cudaEvent_t after) {
                 ps, &sk, &sp, nullptr, nullptr, 0, /*phased=*/true);
   if (e != cudaSuccess) return e;
   if (L.from_plan) list_sorted_heads(L.psk, n, L.keys, L.count, ps);   // (the sort zeroed the count)
-  for (uint32_t* p : {tk, tv, hist}) ctx->plan_blocks.give(p, ps);
+  for (uint32_t* p : {tk, tv, hist}) ctx->plan_blocks.give(plan_mem, p);
   if ((e = take_ready_event(ctx, &L.ready)) != cudaSuccess) return e;
   if ((e = cudaEventRecord(L.ready, ps)) != cudaSuccess) return e;
   return cudaGetLastError();
@@ -1025,8 +971,8 @@ adapm_status adapm_destroy(adapm_ctx* ctx) {
     if (kv.second.listed) cudaEventDestroy(kv.second.listed);
   }
   for (auto e : ctx->spare_ready) cudaEventDestroy(e);
-  ctx->blocks.release();
-  ctx->plan_blocks.release();
+  ctx->blocks.release(cudaFree);
+  ctx->plan_blocks.release(cudaFree);
   Store& s = ctx->s;
   void* ptrs[] = {s.main, s.val, s.acc, s.map, s.rc, s.holders, s.slot_owner, s.free_stack,
                   s.stamp, s.own, s.dirty, ctx->dstate, ctx->early_counts};
