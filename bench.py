@@ -19,7 +19,7 @@ CPU oracle's rate on a bounded sample (one thread), SM clocks sampled during
 the timed region, and the number of library kernels launched in it.  With the
 MF workload (the default) the same line carries a `micro` record: the
 parameter-access microbenchmark (100M keys x 64 floats, 2^20 Zipf(1.1) keys
-per worker and clock, span 1) measured the same way, with pull, push and sync
+per worker and clock, span 1) measured the same way, with pull, push and advance
 against the HBM roofline (--micro-zipf adds other exponents as `micro_sweep`).
 
 With --gpus N > 1 (torchrun) every rank runs an independent replica of the
@@ -604,11 +604,12 @@ def moved_bytes_per_step(wk, d, steps, relocate=False):
     """The least bytes the kernels move per step, which the roofline fractions are taken of.
 
     Replicas are aliases of their main rows until somebody writes (see the replica states in internal.cuh), so
-    always replicating a push stores one row per distinct key, a destroyed replica moves three (its pending row
-    read, main read and written), a created one none and a sync reads 8 bytes per replica (the pending rows it
-    merges are not counted by the library).  The ComplEx and SGNS steps write a key and a scalar per row
-    occurrence and a few rows per sample, which their push reads instead of delta rows.  With relocation replicas
-    are copies and alg_bytes_per_step holds."""
+    always replicating a push stores one row per distinct key, a created replica moves none, and a destroyed one three
+    (its pending row read, main read and written) if its last push was not merged by a sync before: always with
+    windows of one clock.  How many pending rows a sync merges, or an advance after longer windows, the library does
+    not count: no bytes are given for those, and so no fraction.  The ComplEx and SGNS steps write a key and a scalar
+    per row occurrence and a few rows per sample, which their push reads instead of delta rows.  With relocation
+    replicas are copies and alg_bytes_per_step holds."""
     out = alg_bytes_per_step(wk, d, steps, relocate)
     row = wk.row
     per = {k: v / steps for k, v in d.items()}
@@ -620,8 +621,9 @@ def moved_bytes_per_step(wk, d, steps, relocate=False):
     if not relocate:
         out["push"] = R * 4 + rows_in + U * (4 + rows_out)
         out["push_kernel"] = R * 8 + rows_in + U * (4 + rows_out)
-        out["sync"] = per["sync_replicas"] * 8
-        out["advance"] = per["destroyed"] * 3 * row
+        del out["sync"], out["advance"]
+        if wk.span == 1:
+            out["advance"] = per["destroyed"] * 3 * row
     elif hasattr(wk, "step_moved_bytes"):
         out["push"] = R * 4 + rows_in + U * (4 + 2 * row)
         out["push_kernel"] = R * 8 + rows_in + U * (4 + 2 * row)

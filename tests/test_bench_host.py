@@ -92,3 +92,18 @@ def test_manager_options_name_every_switch():
     assert m.workload == "micro" and m.zipf == 1.4 and m.batch is None and m.keys is None and m.span is None
     assert m.no_early_events and m.steps == 3
     assert "early_events_per_step" in bench.MICRO_KEYS and "early_advances" in bench.COUNTERS
+
+
+@pytest.mark.parametrize("span", [1, 4])
+def test_moved_bytes_are_given_only_where_they_are_a_lower_bound(span):
+    """Always replicating, the merged rows are not counted: none for a sync, and for an advance only with windows of
+    one clock, whose replicas are destroyed with their push still pending."""
+    wk = bench.Micro(argparse.Namespace(batch=1024, zipf=None, span=span, keys=10_000), None)
+    row, W, B, U = 256, 8, 1024, 700
+    d = counters(push_rows=W * B, push_unique=U, sync_keys=300, sync_replicas=500, sync_refreshed=500, created=40,
+                 destroyed=30)
+    m = bench.moved_bytes_per_step(wk, d, steps=1)
+    assert "sync" not in m and m.get("advance") == (30 * 3 * row if span == 1 else None)
+    assert m["push"] == W * B * (4 + row) + U * (4 + row) and m["pull"] == W * B * (4 + row) + U * (4 + row)
+    r = bench.moved_bytes_per_step(wk, d, steps=1, relocate=True)
+    assert r == bench.alg_bytes_per_step(wk, d, 1, relocate=True)
