@@ -148,6 +148,7 @@ struct adapm_ctx {
   uint64_t early_advances = 0;   // advances that used their early events
   uint64_t early_undone = 0;     // early events taken back
   bool fake_launch_error = false;   // adapm_debug_fail_next_launch
+  bool fail_barrier = false;        // adapm_debug_fail_next_barrier
 };
 
 namespace {
@@ -425,7 +426,7 @@ adapm_status check_ctx(adapm_ctx* ctx) {
 // While the stream records a graph, calls whose work every launch of the
 // graph can repeat are recorded: pulls, pushes, steps and syncs, all of whose
 // state is on the device.  They take no push plan, start no early events and
-// sort without grid barriers (early_make, find_plan, ctx_sort_phased): the
+// sort without grid barriers (early_make, find_plan, ctx_sort_by): the
 // host numbers plan checks and barrier arrivals per call, and side streams
 // would join the capture.  Calls that move the host's clocks and intent lists
 // cannot be repeated and are refused.
@@ -650,7 +651,7 @@ adapm_status push_device(adapm_ctx* ctx, uint32_t w, const uint32_t* dkeys, uint
   CK(sort_keys(dkeys, n, ctx->s.K, allow_nokey, ctx->bits, ka, kb, va, vb, hist, ctx->sms, ctx->dstate,
                &ctx->bar_base, &ctx->dstate->last_unique, nullptr, ctx->stream, &sk, &sp,
                plan ? plan->px : nullptr, plan ? &ctx->dstate->plan_miss : nullptr, seq,
-               ctx_sort_phased(ctx, n)));
+               ctx_sort_by(ctx, n)));
   ctx->push_rows_host += n;
   PushArgs a = source;
   a.skeys = sk;
@@ -770,7 +771,7 @@ cudaError_t make_plan(adapm_ctx* ctx, IntentList& L, cudaEvent_t after) {
   uint32_t *sk = nullptr, *sp = nullptr;
   e = sort_keys(L.px, n, ctx->s.K, false, ctx->bits, odd ? L.psk : tk, odd ? tk : L.psk, odd ? L.psp : tv,
                 odd ? tv : L.psp, hist, ctx->sms, ctx->dstate, &no_barriers, L.from_plan ? L.count : nullptr, nullptr,
-                ps, &sk, &sp, nullptr, nullptr, 0, /*phased=*/true);
+                ps, &sk, &sp, nullptr, nullptr, 0, SORT_BY_LAUNCHES);
   if (e != cudaSuccess) return e;
   if (L.from_plan) list_sorted_heads(L.psk, n, L.keys, L.count, ps);   // (the sort zeroed the count)
   for (uint32_t* p : {tk, tv, hist}) ctx->plan_blocks.give(plan_mem, p);
@@ -826,7 +827,13 @@ void adapm::ctx_add_push_rows(adapm_ctx* ctx, uint64_t n) {
   if (ctx) ctx->push_rows_host += n;
 }
 
-bool adapm::ctx_sort_phased(adapm_ctx* ctx, uint64_t n) { return ctx->capturing && n > kSmallSort; }
+SortBy adapm::ctx_sort_by(adapm_ctx* ctx, uint64_t n) {
+  if (ctx->capturing) return n > kSmallSort ? SORT_BY_LAUNCHES : SORT_BY_SIZE;
+  if (!ctx->fail_barrier) return SORT_BY_SIZE;
+  ctx->fail_barrier = false;
+  ctx->bar_base += 1ull << 40;   // the sort expects arrivals far beyond those that can happen
+  return SORT_BY_BARRIERS;
+}
 
 int adapm::ctx_begin(adapm_ctx* ctx) { return check_ctx(ctx); }
 
@@ -1249,8 +1256,7 @@ adapm_status adapm_debug_fail_next_launch(adapm_ctx* ctx) {
 
 adapm_status adapm_debug_fail_next_barrier(adapm_ctx* ctx) {
   if (!ctx) return ADAPM_EINVAL;
-  // the next sort expects arrivals far beyond those that can happen
-  ctx->bar_base += 1ull << 40;
+  ctx->fail_barrier = true;
   return ADAPM_OK;
 }
 

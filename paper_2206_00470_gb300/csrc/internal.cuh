@@ -248,11 +248,14 @@ __device__ __forceinline__ bool sort_failed(const DevState* st) {
 // otherwise its blocks account their remaining barriers and return, leaving
 // ka/kb/va/vb as they are (the plan holds the result).  Out-of-range keys
 // are reported by the check as the sort would.
-// phased = true runs the sort as ordinary launches (kernel boundaries instead
-// of grid barriers, *bar_base untouched): for a stream that runs beside other
-// work, where a cooperative launch would wait for the whole GPU.  One for the
+// `by`: SORT_BY_SIZE sorts few keys in one block (below) and others in the
+// cooperative launch, SORT_BY_BARRIERS all in the latter; SORT_BY_LAUNCHES
+// runs the sort as ordinary launches (kernel boundaries instead of grid
+// barriers, *bar_base untouched): for a stream that runs beside other work,
+// where a cooperative launch would wait for the whole GPU, and for a graph.  One for the
 // count and two per pass, or one per pass when the blocks are few enough that
 // each scans the digit table itself.
+enum SortBy { SORT_BY_SIZE, SORT_BY_BARRIERS, SORT_BY_LAUNCHES };
 size_t sort_scratch_words(uint64_t n, int bits, int sms);
 int sort_passes(int bits);
 cudaError_t sort_keys(const uint32_t* raw, uint64_t n, uint64_t K, bool allow_nokey, int bits,
@@ -260,7 +263,7 @@ cudaError_t sort_keys(const uint32_t* raw, uint64_t n, uint64_t K, bool allow_no
                       DevState* st, unsigned long long* bar_base, uint32_t* clear0, uint32_t* clear1,
                       cudaStream_t stream, uint32_t** keys_out, uint32_t** pos_out,
                       const uint32_t* plan_keys = nullptr, uint32_t* plan_word = nullptr, uint32_t plan_seq = 0,
-                      bool phased = false);
+                      SortBy by = SORT_BY_SIZE);
 
 // Up to kSmallSort keys are sorted by one block in one ordinary launch
 // (sort_small.cu; sort_keys calls it for a push).  keys_out / pos_out: the
@@ -324,10 +327,11 @@ void ctx_add_push_rows(struct ::adapm_ctx* ctx, uint64_t n);
 // null, ADAPM_ECUDA once it is unusable), its last error cleared, its device
 // current.  Returns an adapm_status value (0 = ADAPM_OK).
 int ctx_begin(struct ::adapm_ctx* ctx);
-// Whether a push of n keys sorts in ordinary launches: its stream records a
+// How a push of n keys sorts: in ordinary launches while its stream records a
 // graph (the grid barriers' arrival count is the host's, per launch) and the
-// keys are too many for one block.
-bool ctx_sort_phased(struct ::adapm_ctx* ctx, uint64_t n);
+// keys are too many for one block; with the grid barriers, whose first one
+// will wait in vain, after adapm_debug_fail_next_barrier (taken once).
+SortBy ctx_sort_by(struct ::adapm_ctx* ctx, uint64_t n);
 // A CUDA runtime error: records "where: message", marks the context unusable
 // (as every entry point does) and returns ADAPM_ECUDA.
 int ctx_fail_cuda(struct ::adapm_ctx* ctx, cudaError_t e, const char* where);

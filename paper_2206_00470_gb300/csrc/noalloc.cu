@@ -139,7 +139,7 @@ extern "C" adapm_status adapm_push_noalloc(adapm_ctx* ctx, uint32_t worker, cons
   // sort clears
   e = sort_keys(keys, n, v.s.K, false, v.bits, at(L.ka), at(L.kb), at(L.va), at(L.vb), at(L.hist), v.sms,
                 v.dstate, v.bar_base, &v.dstate->last_unique, nullptr, v.stream, &sk, &sp, nullptr, nullptr, 0,
-                ctx_sort_phased(ctx, n));
+                ctx_sort_by(ctx, n));
   if (e != cudaSuccess) return static_cast<adapm_status>(ctx_fail_cuda(ctx, e, "push_noalloc sort"));
   ctx_add_push_rows(ctx, n);
   PushArgs a{sk,

@@ -758,10 +758,10 @@ cudaError_t sort_keys(const uint32_t* raw, uint64_t n, uint64_t K, bool allow_no
                       uint32_t* ka, uint32_t* kb, uint32_t* va, uint32_t* vb, uint32_t* scratch, int sms,
                       DevState* st, unsigned long long* bar_base, uint32_t* clear0, uint32_t* clear1,
                       cudaStream_t stream, uint32_t** keys_out, uint32_t** pos_out, const uint32_t* plan_keys,
-                      uint32_t* plan_word, uint32_t plan_seq, bool phased) {
+                      uint32_t* plan_word, uint32_t plan_seq, SortBy by) {
   const PassPlan pl = plan_for(bits);
-  // (a context whose next grid barrier was made to fail sorts with one)
-  if (n <= (plan_keys ? kSmallPlan : kSmallSort) && va && !phased && n > 0 && (*bar_base >> 40) == 0) {
+  const bool phased = by == SORT_BY_LAUNCHES;
+  if (n <= (plan_keys ? kSmallPlan : kSmallSort) && va && by == SORT_BY_SIZE && n > 0) {
     if (keys_out) *keys_out = ka;
     if (pos_out) *pos_out = va;
     SmallSort a{};
