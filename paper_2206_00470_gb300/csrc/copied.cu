@@ -38,6 +38,7 @@ __global__ void __launch_bounds__(kThreads, C >= 8 ? 2 : 3) evict_create_copied_
   const uint32_t D4 = s.D >> 2;
   const uint32_t ne = s.st->adv_ne, nc = s.st->adv_nc;
   const int32_t top = s.st->adv_top;
+  if (s.st->errors & ERR_TIMEOUT) return;   // a sort gave up: the events that fill the lists have returned, too
   const uint64_t n = ne > nc ? ne : nc;
   float4* main4 = reinterpret_cast<float4*>(s.main);
   float4* val4 = reinterpret_cast<float4*>(s.val);
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(kThreads, C >= 8 ? 2 : (VER && C == 1 ? 3 : 4)
   const int lane = threadIdx.x & (G - 1);
   const uint32_t D4 = s.D >> 2;
   const uint64_t hw = (uint64_t)s.st->high_water;
+  if (s.st->errors & ERR_TIMEOUT) return;   // a sort gave up
   float4* main4 = reinterpret_cast<float4*>(s.main);
   float4* val4 = reinterpret_cast<float4*>(s.val);
   float4* acc4 = reinterpret_cast<float4*>(s.acc);

@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(kThreads, C >= 8 ? 2 : 4) sync_kernel(Store s)
   const uint32_t D4 = s.D >> 2;
   const uint64_t hw = (uint64_t)s.st->high_water;
   s.par = s.st->par;
+  if (s.st->errors & ERR_TIMEOUT) return;   // a sort gave up (read with the words above, in one latency)
   float4* main4 = reinterpret_cast<float4*>(s.main);
   const float4* acc4 = reinterpret_cast<const float4*>(s.acc);
   const uint64_t warps = (uint64_t)gridDim.x * (kThreads / 32);
