@@ -435,8 +435,9 @@ __global__ void __launch_bounds__(kThreads, evict_blocks_per_sm(C)) evict_create
     int32_t es = ev && e < s.S ? (int32_t)e : -1;
     bool bad = (ev && es < 0) || (cr && ck >= s.K);
     if (ck >= s.K) ck = kNoKey;
-    // slot of the creation: the paired evicted slot, else popped (top first)
-    int32_t cs = ck == kNoKey ? -1 : (es >= 0 ? es : s.free_stack[top - 1 - (int32_t)(i - ne)]);
+    // slot of the creation: the paired evicted slot, else popped (top first;
+    // a pair whose evicted slot is out of range has none)
+    int32_t cs = ck == kNoKey || (es < 0 && ev) ? -1 : (es >= 0 ? es : s.free_stack[top - 1 - (int32_t)(i - ne)]);
     const unsigned long long ow = es >= 0 ? s.slot_owner[es] : 0ull;
     const uint32_t k = (uint32_t)ow, a = owner_worker(ow);
     if (ck != kNoKey && (cs < 0 || (uint64_t)cs >= s.S)) {   // a free-stack entry out of range

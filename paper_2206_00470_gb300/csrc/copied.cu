@@ -70,8 +70,11 @@ __global__ void __launch_bounds__(kThreads, C >= 8 ? 2 : 3) evict_create_copied_
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const uint64_t i = i0 + r;
-      // slot of the creation: the paired evicted slot, else popped (top first)
-      cs[r] = ck[r] == kNoKey ? -1 : (es[r] >= 0 ? es[r] : s.free_stack[top - 1 - (int32_t)(i - ne)]);
+      // slot of the creation: the paired evicted slot, else popped (top first;
+      // a pair whose evicted slot is out of range has none)
+      cs[r] = ck[r] == kNoKey || (es[r] < 0 && i < ne)
+                  ? -1
+                  : (es[r] >= 0 ? es[r] : s.free_stack[top - 1 - (int32_t)(i - ne)]);
       ow[r] = es[r] >= 0 ? s.slot_owner[es[r]] : 0ull;
       const bool bad_slot = ck[r] != kNoKey && (cs[r] < 0 || (uint64_t)cs[r] >= s.S);
       const bool bad_owner = es[r] >= 0 && ((uint32_t)ow[r] >= s.K || (ow[r] >> 32) >= s.W);
