@@ -1,8 +1,10 @@
 // extern "C" entry points of libadapm (include/adapm.h) and the host-side
 // state of a context: worker clocks and the per-clock buckets of stored
 // intent lists (Sec. 3: an intent is inactive before C_start, active in
-// [C_start, C_end), expired after).  All device work is enqueued on one
-// stream; scratch comes from a context-owned stream-ordered memory pool.
+// [C_start, C_end), expired after).  Device work is ordered by one stream;
+// copies of host inputs, push plans and early events run beside it on streams
+// of the context's own, which it waits for where it needs them.  Scratch comes
+// from context-owned stream-ordered memory pools.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -442,7 +444,6 @@ constexpr uint64_t kSmallIntent = kSmallPlan;
 constexpr int kPlanPatience = 4;       // unused plans in a row after which a worker gets none ...
 constexpr uint64_t kPlanProbe = 16;    // ... but for one intent in this many
 
-// Refcount events of one worker -> destroy, then create replicas.
 // ---------------------------------------------------------------------------
 // Early advance events.  The refcount events of a worker's next advance
 // read and write only that worker's refcounts and read its slot map, which
@@ -565,6 +566,7 @@ adapm_status early_apply(adapm_ctx* ctx, uint32_t w) {
   return check_launch(ctx, "advance");
 }
 
+// Refcount events of one worker -> destroy, then create replicas.
 adapm_status apply_events(adapm_ctx* ctx, uint32_t w, const std::vector<EventList>& ev,
                           const std::vector<cudaEvent_t>& waits = {}) {
   {
@@ -588,8 +590,6 @@ adapm_status apply_events(adapm_ctx* ctx, uint32_t w, const std::vector<EventLis
   return check_launch(ctx, "apply_events");
 }
 
-// Group, sum and apply n delta rows (device keys/rows); keys may hold kNoKey
-// when allow_nokey (rows the caller wants skipped).
 // The plan a push of n keys by worker w may use: the newest recorded intent
 // of w with n keys whose window (as signalled) holds the worker's clock.
 IntentList* find_plan(adapm_ctx* ctx, uint32_t w, uint64_t n) {
@@ -613,9 +613,10 @@ PushArgs step_factors(const StepOut& o, uint32_t kind, uint64_t n, uint32_t per)
   return f;
 }
 
-// `source`: the rows (deltas), or a step's factors.  plans = false: the caller
-// knows its keys never follow an intent's order
-// (the SGNS step), so no plan is looked up.
+// Group, sum and apply n delta rows.  `source`: the rows (deltas), or a step's
+// factors.  Keys may hold kNoKey when allow_nokey (rows the caller wants
+// skipped).  plans = false: the caller knows its keys never follow an intent's
+// order (the SGNS step), so no plan is looked up.
 adapm_status push_device(adapm_ctx* ctx, uint32_t w, const uint32_t* dkeys, uint64_t n,
                          const PushArgs& source, bool allow_nokey, bool plans = true) {
   if (n == 0) return ADAPM_OK;
@@ -743,7 +744,8 @@ SmallSort small_plan(adapm_ctx* ctx, const IntentList& L, const uint32_t* keys) 
 // Sort an intent's keys (L.px) with their positions on the plan stream (a phased
 // sort: no block waits for another, so it runs in whatever the library
 // stream leaves of the GPU), into L.psk / L.psp; with from_plan the distinct
-// keys follow from the sorted ones (ascending) into L.keys / L.count.
+// keys follow from the sorted ones, in no particular order, into L.keys /
+// L.count.
 // L.ready is recorded on the plan stream after all of it.  The library
 // stream must have enqueued the keys (and L's arrays) before `after`.
 cudaError_t make_plan(adapm_ctx* ctx, IntentList& L, cudaEvent_t after) {
@@ -1210,7 +1212,7 @@ adapm_status adapm_push(adapm_ctx* ctx, uint32_t worker, const uint32_t* keys, u
   CK(stage_in(ctx, deltas, n * ctx->s.D, &id));
   CK(stage_join(ctx));
   if (reinterpret_cast<uintptr_t>(id.dev) % 16 != 0) {
-    // the push copies whole rows with the bulk-copy engine: 16-byte aligned rows
+    // the push reads rows as float4: 16-byte aligned rows
     float* aligned = nullptr;
     CK(pool_alloc(ctx, &aligned, n * ctx->s.D));
     CK(cudaMemcpyAsync(aligned, id.dev, n * ctx->s.D * sizeof(float), cudaMemcpyDeviceToDevice,
@@ -1265,7 +1267,7 @@ adapm_status adapm_wait(adapm_ctx* ctx) {
   if (ctx->broken) return fail(ctx, ADAPM_ECUDA, "context unusable after an earlier CUDA error");
   cudaSetDevice(ctx->device);
   CK(cudaStreamSynchronize(ctx->stream));
-  if (ctx->plan_stream) CK(cudaStreamSynchronize(ctx->plan_stream));   // plans read the callers' keys
+  if (ctx->plan_stream) CK(cudaStreamSynchronize(ctx->plan_stream));   // plans are part of their intents
   if (ctx->early_stream) CK(cudaStreamSynchronize(ctx->early_stream));
   uint32_t errors = 0;
   CK(cudaMemcpy(&errors, &ctx->dstate->errors, sizeof errors, cudaMemcpyDeviceToHost));

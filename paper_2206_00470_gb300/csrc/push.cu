@@ -7,8 +7,12 @@ uint64_t push_chunk_rows(uint32_t D, uint64_t n, int sms) {
   // one span per resident block where the span fits in shared memory, else
   // as few full waves of resident blocks as do: rows per group = n / (groups
   // per block x resident blocks x waves), in [8, kPushSpan / groups].  (Spans
-  // of kPushSpan rows whatever the last wave holds: 696 blocks on 456 places
-  // at 2.1M rows of 300 floats, 475 us against 410 us for 912.)
+  // of kPushSpan rows whatever the last wave holds: 2.1M rows of 300 floats of
+  // the SGNS step make 696 blocks, 2.3 waves of the 304 that run at a time, and
+  // take 475 us against 410 us for 912, three full waves.)  The blocks counted
+  // are those of rows from an array: AdaGrad sources of 65 to 96 vectors, four
+  // per lane, and sources with scalars (push_blocks_per_sm) run fewer at a
+  // time, so that their last wave can be partly empty.
   uint64_t ch = 0;
   dispatch_push_gc(D / 4, false, [&](auto Gc, auto Cc) {
     constexpr int G = decltype(Gc)::value, C = decltype(Cc)::value;

@@ -15,9 +15,10 @@
 // and a scalar per row occurrence, and the delta rows are formed here, where
 // they are summed: they never travel through memory, and the few rows they
 // are formed from stay in L2.  Written and read back, they were two thirds of
-// the steps' traffic.  Per clock of 8 workers, step + scatter: SGNS, 8192
-// centres of 261 rows x 300 floats 9.88 + 8.43 -> 6.58 + 3.81 ms; ComplEx,
-// 4096 triples of 103 rows x 512 floats 3.77 + 2.29 -> 1.22 + 2.46 ms.
+// the steps' traffic.  Per clock of 8 workers, step + scatter, delta rows and
+// as both are now: SGNS, 8192 centres of 261 rows x 300 floats 9.88 + 8.43 and
+// 3.64 + 3.11 ms; ComplEx, 4096 triples of 103 rows x 512 floats 3.77 + 2.29
+// and 1.10 + 2.42 ms.
 #pragma once
 
 #include "internal.cuh"
@@ -170,9 +171,12 @@ __device__ __forceinline__ void take_and_apply(const Store& s, uint32_t w, uint3
 // chunk (a tail piece in the chunk it starts in, head pieces in the chunks
 // it continues into).
 constexpr int kPushSpan = 3072;
-constexpr uint32_t kPushCopies = 512;   // (with a step's scalars three blocks still fit an SM)
-// resident push_chunks blocks per SM (its launch bounds), and rows a group
-// keeps in flight
+constexpr uint32_t kPushCopies = 512;
+// push_chunks blocks per SM by its launch bounds, and rows a group keeps in
+// flight.  Shared memory fits as many, but for a step's scalars: rows of three
+// vectors per lane then take 82 KB a block, of which two fit an SM, rows of
+// eight 123 KB, of which one does.  (There the registers are cut for a block
+// more than runs, and push_chunk_rows counts its place.)
 constexpr int push_blocks_per_sm(int C) { return C >= 4 ? 2 : 3; }
 constexpr int push_rows_in_flight(int C) { return C == 3 ? 2 : (4 / C > 0 ? 4 / C : 1); }
 

@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) sort_kernel(SortArgs a) {
   constexpr bool has_count = KIND == kSortAll || KIND == kSortCount;
   constexpr bool has_scan = KIND == kSortAll || KIND == kSortScan;
   constexpr bool has_scatter = KIND == kSortAll || KIND == kSortScatter || KIND == kSortScanScatter;
-    const uint64_t chunk = (a.n + B - 1) / B;
+  const uint64_t chunk = (a.n + B - 1) / B;
   const uint64_t c0 = a.n < b * chunk ? a.n : b * chunk;
   const uint64_t c1 = a.n < c0 + chunk ? a.n : c0 + chunk;
   const bool single = c1 - c0 <= (uint64_t)SUB;
