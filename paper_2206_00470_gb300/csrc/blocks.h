@@ -14,7 +14,7 @@ namespace adapm {
 // where a pool allocation and its free are two calls into the driver (0.7 to 1
 // us each, six pairs a push).  Sizes are rounded up to one of four steps per
 // power of two.  Blocks above kLargest are not kept, and not more than kKeep
-// bytes in all: beyond that, blocks of the size that has gone unused longest
+// bytes in all: beyond that, blocks of the class that has gone unused longest
 // go back to the pool, which the context owns and destroys.  An allocation
 // that fails gives every kept block back to the pool, where their memory
 // serves any size, and is tried once more.
@@ -38,25 +38,23 @@ class BlockCache {
       drop_all(mem);
       return mem.alloc(p, bytes);
     }
-    const size_t size = round_up(bytes);
-    const auto it = kept_of_.find(size);
-    if (it != kept_of_.end()) {
-      it->second.used = ++clock_;
-      if (!it->second.blocks.empty()) {
-        *p = it->second.blocks.back();
-        it->second.blocks.pop_back();
-        kept_ -= size;
-        return 0;
-      }
+    const int c = size_class(bytes);
+    Kept& k = kept_of_[c];
+    k.used = ++clock_;
+    if (!k.blocks.empty()) {
+      *p = k.blocks.back();
+      k.blocks.pop_back();
+      kept_ -= class_bytes(c);
+      return 0;
     }
-    int e = mem.alloc(p, size);
+    int e = mem.alloc(p, class_bytes(c));
     if (e != 0 && kept_ != 0) {
       drop_all(mem);
-      e = mem.alloc(p, size);
+      e = mem.alloc(p, class_bytes(c));
     }
     if (e == 0) {
       try {
-        size_[*p] = size;
+        class_of_[*p] = c;
       } catch (...) {   // no host memory to remember it by: given back like any other
       }
     }
@@ -65,21 +63,21 @@ class BlockCache {
 
   template <class Mem>
   void give(Mem mem, void* p) {
-    const auto it = size_.find(p);
-    if (it == size_.end()) {   // one that is not kept
+    const auto it = class_of_.find(p);
+    if (it == class_of_.end()) {   // one that is not kept
       mem.free(p);
       return;
     }
-    const size_t size = it->second;
+    Kept& k = kept_of_[it->second];
+    const size_t size = class_bytes(it->second);
+    k.used = ++clock_;
+    while (kept_ + size > kKeep && drop_oldest(mem)) {
+    }
     try {
-      Kept& k = kept_of_[size];
-      k.used = ++clock_;
-      while (kept_ + size > kKeep && drop_oldest(mem)) {
-      }
       k.blocks.push_back(p);
       kept_ += size;
     } catch (...) {
-      size_.erase(p);
+      class_of_.erase(p);
       mem.free(p);
     }
   }
@@ -87,10 +85,11 @@ class BlockCache {
   // Every kept block, when the stream is idle and nothing more is taken.
   template <class Free>
   void release(Free free) {
-    for (auto& k : kept_of_)
-      for (void* p : k.second.blocks) free(p);
-    kept_of_.clear();
-    size_.clear();
+    for (Kept& k : kept_of_) {
+      for (void* p : k.blocks) free(p);
+      k.blocks.clear();
+    }
+    class_of_.clear();
     kept_ = 0;
   }
 
@@ -99,29 +98,30 @@ class BlockCache {
  private:
   struct Kept {
     std::vector<void*> blocks;
-    uint64_t used = 0;   // clock_ when a block of this size was last taken or given back
+    uint64_t used = 0;   // clock_ when a block of this class was last taken or given back
   };
-  static size_t round_up(size_t bytes) {
-    if (bytes <= 1024) return 1024;
-    size_t step = 256;
-    while (step * 8 < bytes) step <<= 1;   // four steps between 4 * step and 8 * step
-    return (bytes + step - 1) / step * step;
+  // Class 4 e + q holds blocks of up to (5 + q) * 256 * 2^e bytes, q = 0 .. 3;
+  // class 0 those of up to 1280.
+  static constexpr int kClasses = 64;
+  static size_t class_bytes(int c) { return (size_t)(5 + c % 4) << (8 + c / 4); }
+  static int size_class(size_t bytes) {
+    int e = 0;
+    while (((size_t)8 << (8 + e)) < bytes) ++e;
+    const size_t step = (size_t)1 << (8 + e);
+    const int q = (int)((bytes + step - 1) >> (8 + e)) - 5;
+    return 4 * e + (q < 0 ? 0 : q);
   }
-  // A block of the size unused longest goes back to the pool; false: none is kept.
+  // A block of the class unused longest goes back to the pool; false: none is kept.
   template <class Mem>
   bool drop_oldest(Mem mem) {
-    Kept* oldest = nullptr;
-    size_t size = 0;
-    for (auto& k : kept_of_) {
-      if (k.second.blocks.empty() || (oldest && oldest->used <= k.second.used)) continue;
-      oldest = &k.second;
-      size = k.first;
-    }
-    if (!oldest) return false;
-    void* p = oldest->blocks.back();
-    oldest->blocks.pop_back();
-    kept_ -= size;
-    size_.erase(p);
+    int oldest = -1;
+    for (int c = 0; c < kClasses; ++c)
+      if (!kept_of_[c].blocks.empty() && (oldest < 0 || kept_of_[c].used < kept_of_[oldest].used)) oldest = c;
+    if (oldest < 0) return false;
+    void* p = kept_of_[oldest].blocks.back();
+    kept_of_[oldest].blocks.pop_back();
+    kept_ -= class_bytes(oldest);
+    class_of_.erase(p);
     mem.free(p);
     return true;
   }
@@ -131,8 +131,8 @@ class BlockCache {
     }
   }
 
-  std::unordered_map<size_t, Kept> kept_of_;   // by size (about a hundred sizes at most)
-  std::unordered_map<void*, size_t> size_;     // of every block that will be kept when given back
+  Kept kept_of_[kClasses];
+  std::unordered_map<void*, int> class_of_;   // of every block that will be kept when given back
   size_t kept_ = 0;
   uint64_t clock_ = 0;
 };
